@@ -26,6 +26,7 @@ namespace gb300ntt {
 // BN254 base field q (254 bits).
 struct FieldBn254Fq {
   static constexpr int kId = 2;
+  static constexpr bool kSubtract = false;
   static constexpr uint32_t P0 = 0xd87cfd47u, P1 = 0x3c208c16u, P2 = 0x6871ca8du, P3 = 0x97816a91u,
                             P4 = 0x8181585du, P5 = 0xb85045b6u, P6 = 0xe131a029u, P7 = 0x30644e72u;
   static constexpr uint32_t NP = neg_inv_u32(P0);

@@ -1,13 +1,12 @@
 // fp384.cuh -- 381-bit prime-field arithmetic for sm_103a, 12 x 32-bit limbs:
 // the base field of BLS12-381 G1 (for the multi-scalar multiplication).
 //
-// The same Montgomery product as fp256.cuh (CIOS, radix 2^32, Koc, Acar and
-// Kaliski 1996) over twelve limbs: per row the a*b_i products run as two
-// carry chains (even limbs, odd limbs; the low and high halves of a product
-// adjacent in one chain), then m = t0 * (-q^-1 mod 2^32) and the m*q rows the
-// same way.  With a, b < q < 2^381 the running value stays below 2^415, so it
-// fits in thirteen limbs and the last carry of every odd chain is zero; the
-// result is below 2q and one conditional subtraction makes it canonical.
+// The same Montgomery product as fp256.cuh over twelve limbs: operand scanning
+// in radix 2^32 with the products of even and odd limbs in two accumulators of
+// aligned word pairs (T = sum E_k 2^(32 k) + sum O_k 2^(32 (k + 1))).  With
+// a, b < q < 2^381 the running value stays below 2^415, so it fits in thirteen
+// words; the result is below 2q and one conditional subtraction makes it
+// canonical.
 //
 // Conventions: element = uint32_t[12], limb 0 least significant; in memory
 // 48 bytes, moved as three 128-bit accesses (an element is 16-byte aligned).
@@ -30,81 +29,116 @@ namespace fp384 {
 
 using F = FieldBls12381Fq;
 
-// t[0..12] += (a0, a2, ..., a10) * b at limbs (0,1), (2,3), ..., (10,11), carry into t12.
-__device__ __forceinline__ void row_even(uint32_t t[13], const uint32_t a[12], uint32_t b) {
-  asm("mad.lo.cc.u32  %0,  %13, %19, %0;\n\t"
-      "madc.hi.cc.u32 %1,  %13, %19, %1;\n\t"
-      "madc.lo.cc.u32 %2,  %14, %19, %2;\n\t"
-      "madc.hi.cc.u32 %3,  %14, %19, %3;\n\t"
-      "madc.lo.cc.u32 %4,  %15, %19, %4;\n\t"
-      "madc.hi.cc.u32 %5,  %15, %19, %5;\n\t"
-      "madc.lo.cc.u32 %6,  %16, %19, %6;\n\t"
-      "madc.hi.cc.u32 %7,  %16, %19, %7;\n\t"
-      "madc.lo.cc.u32 %8,  %17, %19, %8;\n\t"
-      "madc.hi.cc.u32 %9,  %17, %19, %9;\n\t"
+// d = (x0, ..., x5) * y over aligned word pairs
+__device__ __forceinline__ void pairs_mul6(uint32_t d[12], uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t x4,
+                                           uint32_t x5, uint32_t y) {
+  asm("mul.lo.u32 %0, %12, %18;\n\t"
+      "mul.hi.u32 %1, %12, %18;\n\t"
+      "mul.lo.u32 %2, %13, %18;\n\t"
+      "mul.hi.u32 %3, %13, %18;\n\t"
+      "mul.lo.u32 %4, %14, %18;\n\t"
+      "mul.hi.u32 %5, %14, %18;\n\t"
+      "mul.lo.u32 %6, %15, %18;\n\t"
+      "mul.hi.u32 %7, %15, %18;\n\t"
+      "mul.lo.u32 %8, %16, %18;\n\t"
+      "mul.hi.u32 %9, %16, %18;\n\t"
+      "mul.lo.u32 %10, %17, %18;\n\t"
+      "mul.hi.u32 %11, %17, %18;"
+      : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7]), "=r"(d[8]),
+        "=r"(d[9]), "=r"(d[10]), "=r"(d[11])
+      : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(x4), "r"(x5), "r"(y));
+}
+
+// d += (x0, ..., x5) * y, no carry out
+__device__ __forceinline__ void pairs_mad6(uint32_t d[12], uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t x4,
+                                           uint32_t x5, uint32_t y) {
+  asm("mad.lo.cc.u32 %0, %12, %18, %0;\n\t"
+      "madc.hi.cc.u32 %1, %12, %18, %1;\n\t"
+      "madc.lo.cc.u32 %2, %13, %18, %2;\n\t"
+      "madc.hi.cc.u32 %3, %13, %18, %3;\n\t"
+      "madc.lo.cc.u32 %4, %14, %18, %4;\n\t"
+      "madc.hi.cc.u32 %5, %14, %18, %5;\n\t"
+      "madc.lo.cc.u32 %6, %15, %18, %6;\n\t"
+      "madc.hi.cc.u32 %7, %15, %18, %7;\n\t"
+      "madc.lo.cc.u32 %8, %16, %18, %8;\n\t"
+      "madc.hi.cc.u32 %9, %16, %18, %9;\n\t"
+      "madc.lo.cc.u32 %10, %17, %18, %10;\n\t"
+      "madc.hi.u32 %11, %17, %18, %11;"
+      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7]), "+r"(d[8]),
+        "+r"(d[9]), "+r"(d[10]), "+r"(d[11])
+      : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(x4), "r"(x5), "r"(y));
+}
+
+// d += (x0, ..., x5) * y, carry into top
+__device__ __forceinline__ void pairs_mad6_top(uint32_t d[12], uint32_t &top, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t x4,
+                                           uint32_t x5, uint32_t y) {
+  asm("mad.lo.cc.u32 %0, %13, %19, %0;\n\t"
+      "madc.hi.cc.u32 %1, %13, %19, %1;\n\t"
+      "madc.lo.cc.u32 %2, %14, %19, %2;\n\t"
+      "madc.hi.cc.u32 %3, %14, %19, %3;\n\t"
+      "madc.lo.cc.u32 %4, %15, %19, %4;\n\t"
+      "madc.hi.cc.u32 %5, %15, %19, %5;\n\t"
+      "madc.lo.cc.u32 %6, %16, %19, %6;\n\t"
+      "madc.hi.cc.u32 %7, %16, %19, %7;\n\t"
+      "madc.lo.cc.u32 %8, %17, %19, %8;\n\t"
+      "madc.hi.cc.u32 %9, %17, %19, %9;\n\t"
       "madc.lo.cc.u32 %10, %18, %19, %10;\n\t"
       "madc.hi.cc.u32 %11, %18, %19, %11;\n\t"
-      "addc.u32       %12, %12, 0;"
-      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]),
-        "+r"(t[8]), "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12])
-      : "r"(a[0]), "r"(a[2]), "r"(a[4]), "r"(a[6]), "r"(a[8]), "r"(a[10]), "r"(b));
+      "addc.u32 %12, %12, 0;"
+      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7]), "+r"(d[8]),
+        "+r"(d[9]), "+r"(d[10]), "+r"(d[11]), "+r"(top)
+      : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(x4), "r"(x5), "r"(y));
 }
 
-// t[1..12] += (a1, a3, ..., a11) * b at limbs (1,2), ..., (11,12); no carry out.
-__device__ __forceinline__ void row_odd(uint32_t t[13], const uint32_t a[12], uint32_t b) {
-  asm("mad.lo.cc.u32  %0,  %12, %18, %0;\n\t"
-      "madc.hi.cc.u32 %1,  %12, %18, %1;\n\t"
-      "madc.lo.cc.u32 %2,  %13, %18, %2;\n\t"
-      "madc.hi.cc.u32 %3,  %13, %18, %3;\n\t"
-      "madc.lo.cc.u32 %4,  %14, %18, %4;\n\t"
-      "madc.hi.cc.u32 %5,  %14, %18, %5;\n\t"
-      "madc.lo.cc.u32 %6,  %15, %18, %6;\n\t"
-      "madc.hi.cc.u32 %7,  %15, %18, %7;\n\t"
-      "madc.lo.cc.u32 %8,  %16, %18, %8;\n\t"
-      "madc.hi.cc.u32 %9,  %16, %18, %9;\n\t"
-      "madc.lo.cc.u32 %10, %17, %18, %10;\n\t"
-      "madc.hi.u32    %11, %17, %18, %11;"
-      : "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(t[8]),
-        "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12])
-      : "r"(a[1]), "r"(a[3]), "r"(a[5]), "r"(a[7]), "r"(a[9]), "r"(a[11]), "r"(b));
+// The division by 2^32 with the next odd chain: e0 += s[1], d = s[2..11] + (x0, ..., x5) * y.
+__device__ __forceinline__ void pairs_shift_mad6(uint32_t &e0, uint32_t d[12], const uint32_t s[12], uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t x4,
+                                           uint32_t x5, uint32_t y) {
+  asm("add.cc.u32 %0, %0, %13;\n\t"
+      "madc.lo.cc.u32 %1, %24, %30, %14;\n\t"
+      "madc.hi.cc.u32 %2, %24, %30, %15;\n\t"
+      "madc.lo.cc.u32 %3, %25, %30, %16;\n\t"
+      "madc.hi.cc.u32 %4, %25, %30, %17;\n\t"
+      "madc.lo.cc.u32 %5, %26, %30, %18;\n\t"
+      "madc.hi.cc.u32 %6, %26, %30, %19;\n\t"
+      "madc.lo.cc.u32 %7, %27, %30, %20;\n\t"
+      "madc.hi.cc.u32 %8, %27, %30, %21;\n\t"
+      "madc.lo.cc.u32 %9, %28, %30, %22;\n\t"
+      "madc.hi.cc.u32 %10, %28, %30, %23;\n\t"
+      "madc.lo.cc.u32 %11, %29, %30, 0;\n\t"
+      "madc.hi.u32 %12, %29, %30, 0;"
+      : "+&r"(e0), "=&r"(d[0]), "=&r"(d[1]), "=&r"(d[2]), "=&r"(d[3]), "=&r"(d[4]), "=&r"(d[5]), "=&r"(d[6]),
+        "=&r"(d[7]), "=&r"(d[8]), "=&r"(d[9]), "=&r"(d[10]), "=&r"(d[11])
+      : "r"(s[1]), "r"(s[2]), "r"(s[3]), "r"(s[4]), "r"(s[5]), "r"(s[6]), "r"(s[7]), "r"(s[8]), "r"(s[9]),
+        "r"(s[10]), "r"(s[11]),
+        "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(x4), "r"(x5), "r"(y));
 }
 
-// The same two chains with q (immediates) as the multi-limb operand.
-__device__ __forceinline__ void row_even_q(uint32_t t[13], uint32_t m) {
-  asm("mad.lo.cc.u32  %0,  %13, %14, %0;\n\t"
-      "madc.hi.cc.u32 %1,  %13, %14, %1;\n\t"
-      "madc.lo.cc.u32 %2,  %13, %15, %2;\n\t"
-      "madc.hi.cc.u32 %3,  %13, %15, %3;\n\t"
-      "madc.lo.cc.u32 %4,  %13, %16, %4;\n\t"
-      "madc.hi.cc.u32 %5,  %13, %16, %5;\n\t"
-      "madc.lo.cc.u32 %6,  %13, %17, %6;\n\t"
-      "madc.hi.cc.u32 %7,  %13, %17, %7;\n\t"
-      "madc.lo.cc.u32 %8,  %13, %18, %8;\n\t"
-      "madc.hi.cc.u32 %9,  %13, %18, %9;\n\t"
-      "madc.lo.cc.u32 %10, %13, %19, %10;\n\t"
-      "madc.hi.cc.u32 %11, %13, %19, %11;\n\t"
-      "addc.u32       %12, %12, 0;"
-      : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]),
-        "+r"(t[8]), "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12])
-      : "r"(m), "n"(F::P0), "n"(F::P2), "n"(F::P4), "n"(F::P6), "n"(F::P8), "n"(F::P10));
+// t = e + the words s[1..11] of the other accumulator
+__device__ __forceinline__ void pairs_merge6(uint32_t t[12], const uint32_t e[12], const uint32_t s[12]) {
+  asm("add.cc.u32 %0, %12, %24;\n\t"
+      "addc.cc.u32 %1, %13, %25;\n\t"
+      "addc.cc.u32 %2, %14, %26;\n\t"
+      "addc.cc.u32 %3, %15, %27;\n\t"
+      "addc.cc.u32 %4, %16, %28;\n\t"
+      "addc.cc.u32 %5, %17, %29;\n\t"
+      "addc.cc.u32 %6, %18, %30;\n\t"
+      "addc.cc.u32 %7, %19, %31;\n\t"
+      "addc.cc.u32 %8, %20, %32;\n\t"
+      "addc.cc.u32 %9, %21, %33;\n\t"
+      "addc.cc.u32 %10, %22, %34;\n\t"
+      "addc.u32 %11, %23, 0;"
+      : "=&r"(t[0]), "=&r"(t[1]), "=&r"(t[2]), "=&r"(t[3]), "=&r"(t[4]), "=&r"(t[5]), "=&r"(t[6]), "=&r"(t[7]), "=&r"(t[8]), "=&r"(t[9]), "=&r"(t[10]), "=&r"(t[11])
+      : "r"(e[0]), "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(e[8]), "r"(e[9]),
+        "r"(e[10]), "r"(e[11]),
+        "r"(s[1]), "r"(s[2]), "r"(s[3]), "r"(s[4]), "r"(s[5]), "r"(s[6]), "r"(s[7]), "r"(s[8]), "r"(s[9]),
+        "r"(s[10]), "r"(s[11]));
 }
 
-__device__ __forceinline__ void row_odd_q(uint32_t t[13], uint32_t m) {
-  asm("mad.lo.cc.u32  %0,  %12, %13, %0;\n\t"
-      "madc.hi.cc.u32 %1,  %12, %13, %1;\n\t"
-      "madc.lo.cc.u32 %2,  %12, %14, %2;\n\t"
-      "madc.hi.cc.u32 %3,  %12, %14, %3;\n\t"
-      "madc.lo.cc.u32 %4,  %12, %15, %4;\n\t"
-      "madc.hi.cc.u32 %5,  %12, %15, %5;\n\t"
-      "madc.lo.cc.u32 %6,  %12, %16, %6;\n\t"
-      "madc.hi.cc.u32 %7,  %12, %16, %7;\n\t"
-      "madc.lo.cc.u32 %8,  %12, %17, %8;\n\t"
-      "madc.hi.cc.u32 %9,  %12, %17, %9;\n\t"
-      "madc.lo.cc.u32 %10, %12, %18, %10;\n\t"
-      "madc.hi.u32    %11, %12, %18, %11;"
-      : "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(t[8]),
-        "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12])
-      : "r"(m), "n"(F::P1), "n"(F::P3), "n"(F::P5), "n"(F::P7), "n"(F::P9), "n"(F::P11));
+// One row's reduction: T += m q, T becomes a multiple of 2^32.
+__device__ __forceinline__ void redc_row(uint32_t E[12], uint32_t O[12]) {
+  const uint32_t m = E[0] * F::NP;
+  pairs_mad6(O, F::P1, F::P3, F::P5, F::P7, F::P9, F::P11, m);
+  pairs_mad6_top(E, O[11], F::P0, F::P2, F::P4, F::P6, F::P8, F::P10, m);
 }
 
 // d = a - q with borrow mask (all ones when a < q).
@@ -142,37 +176,31 @@ __device__ __forceinline__ void reduce_once(uint32_t r[12], const uint32_t t[12]
 
 // r = a * b * 2^-384 mod q.  a, b canonical; r canonical; r may alias a or b.
 __device__ __forceinline__ void mont_mul(uint32_t r[12], const uint32_t a[12], const uint32_t b[12]) {
-  uint32_t t[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  uint32_t E[12], O[12];
+  pairs_mul6(E, a[0], a[2], a[4], a[6], a[8], a[10], b[0]);
+  pairs_mul6(O, a[1], a[3], a[5], a[7], a[9], a[11], b[0]);
+  redc_row(E, O);
 #pragma unroll
-  for (int i = 0; i < 12; ++i) {
-    row_even(t, a, b[i]);
-    row_odd(t, a, b[i]);
-    const uint32_t m = t[0] * F::NP;
-    row_even_q(t, m);
-    row_odd_q(t, m);
+  for (int i = 1; i < 12; ++i) {
+    uint32_t X[12];
+    pairs_shift_mad6(O[0], X, E, a[1], a[3], a[5], a[7], a[9], a[11], b[i]);
+    pairs_mad6_top(O, X[11], a[0], a[2], a[4], a[6], a[8], a[10], b[i]);
+    redc_row(O, X);
 #pragma unroll
-    for (int j = 0; j < 12; ++j) t[j] = t[j + 1];
-    t[12] = 0;
+    for (int j = 0; j < 12; ++j) {
+      E[j] = O[j];
+      O[j] = X[j];
+    }
   }
+  uint32_t t[12];
+  pairs_merge6(t, O, E);
   reduce_once(r, t);
 }
 
-// y = x * 2^-384 mod q (Montgomery reduction alone).
+// y = x * 2^-384 mod q.
 __device__ __forceinline__ void mont_redc(uint32_t y[12], const uint32_t x[12]) {
-  uint32_t t[13];
-#pragma unroll
-  for (int j = 0; j < 12; ++j) t[j] = x[j];
-  t[12] = 0;
-#pragma unroll
-  for (int i = 0; i < 12; ++i) {
-    const uint32_t m = t[0] * F::NP;
-    row_even_q(t, m);
-    row_odd_q(t, m);
-#pragma unroll
-    for (int j = 0; j < 12; ++j) t[j] = t[j + 1];
-    t[12] = 0;
-  }
-  reduce_once(y, t);
+  const uint32_t one[12] = {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  mont_mul(y, x, one);
 }
 
 // r = a + b mod q (a + b < 2q < 2^384: no carry out of the top limb).

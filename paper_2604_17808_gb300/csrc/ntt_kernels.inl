@@ -389,23 +389,24 @@ __global__ void mul_vec_kernel(uint4 *out, const uint4 *a, const uint4 *b, uint6
 
 // Pointwise quotient of a prover on coset evaluations:
 //   out[i] = (a[i] b[i] - c[i]) z[i mod len]
-// in one pass over the vectors (3 reads, 1 write, two products and one
-// reduction per element): u = a b 2^-256, v = c 2^-256, and the multiplier
-// z 2^512 turns (u - v) back into standard form.
+// in one pass over the vectors (3 reads, 1 write, two products per element):
+// a b + (p - c) goes through one Montgomery reduction, which leaves
+// (a b - c) 2^-256, and the multiplier z 2^512 turns that back into standard
+// form.
 __global__ void quotient_kernel(uint4 *out, const uint4 *a, const uint4 *b, const uint4 *c, const QuotientZ z,
                                 uint64_t count) {
   const uint64_t zmask = z.len - 1;
+  const uint32_t zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (uint64_t idx = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; idx < count;
        idx += (uint64_t)gridDim.x * blockDim.x) {
     uint32_t x[8], y[8], w[8];
+    fe_load_global(w, c, idx);
+    sub_mod<F>(w, zero, w);             // -c
     fe_load_global(x, a, idx);
     fe_load_global(y, b, idx);
-    mont_mul<F>(x, x, y);          // a b 2^-256
-    fe_load_global(y, c, idx);
-    mont_redc<F>(y, y);            // c 2^-256
-    sub_mod<F>(x, x, y);
+    mont_mul_add<F>(x, x, y, w);        // (a b - c) 2^-256
     fe_from_param(w, z.z[idx & zmask]);
-    mont_mul<F>(x, x, w);          // (a b - c) z
+    mont_mul<F>(x, x, w);               // (a b - c) z
     fe_store_global(out, idx, x);
   }
 }

@@ -325,30 +325,15 @@ __device__ __forceinline__ void byte_merge(uint32_t z[9], const uint32_t u[32], 
 }
 
 // r = z * t * 2^-288 mod p for z < 2^280 (nine limbs) and canonical t: the
-// CIOS rows of mont_mul (fp256.cuh) over the nine limbs of z.  The running
-// value stays below 2^288 (as in mont_mul: t < p, one limb of z per row) and
-// the result is below 2p; one conditional subtraction makes it canonical
-// (lazy: left in [0, 2p) for a pass that is not the last).
+// rows of mont_mul (fp256.cuh) over the nine limbs of z, result below 2p;
+// one conditional subtraction makes it canonical where the rows leave it in
+// [0, 2p) (lazy: kept so for a pass that is not the last).
 template <class F>
 __device__ __forceinline__ void mont_mul_z9(uint32_t r[8], const uint32_t z[9], const uint32_t t[8], bool lazy) {
-  uint32_t acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    row_even(acc, t, z[i]);
-    row_odd(acc, t, z[i]);
-    const uint32_t m = mont_m<F>(acc[0]);
-    row_even_p<F>(acc, m);
-    row_odd_p<F>(acc, m);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = acc[j + 1];
-    acc[8] = 0;
-  }
-  if (lazy) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) r[j] = acc[j];   // in [0, 2p): the next pass takes any 256-bit input
-  } else {
-    reduce_once<F>(r, acc);
-  }
+  uint32_t y[8];
+  mont_rows<F, 9>(y, t, z, nullptr);
+  if (F::kSubtract || lazy) fe_copy(r, y);   // the next pass takes any 256-bit input
+  else reduce_once<F>(r, y);
 }
 
 // r = z mod p for z < 2^280 (nine limbs): q = floor(floor(z / 2^224) mu /
@@ -360,10 +345,10 @@ template <class F>
 __device__ __forceinline__ void barrett_z9(uint32_t r[8], const uint32_t z[9], uint64_t mu, bool lazy) {
   const uint64_t zt = ((uint64_t)z[8] << 32) | z[7];
   const uint32_t q = (uint32_t)__umul64hi(zt, mu);
-  uint32_t qp[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  row_even_p<F>(qp, q);
-  row_odd_p<F>(qp, q);
-  uint32_t d[8];
+  // z - q p mod 2^256: q times the even limbs of p, then the odd ones
+  uint32_t e[8], o[8], d[8];
+  pairs_mul4(e, F::P0, F::P2, F::P4, F::P6, q);
+  pairs_mul4(o, F::P1, F::P3, F::P5, F::P7, q);
   asm("sub.cc.u32  %0, %8,  %16;\n\t"
       "subc.cc.u32 %1, %9,  %17;\n\t"
       "subc.cc.u32 %2, %10, %18;\n\t"
@@ -372,9 +357,18 @@ __device__ __forceinline__ void barrett_z9(uint32_t r[8], const uint32_t z[9], u
       "subc.cc.u32 %5, %13, %21;\n\t"
       "subc.cc.u32 %6, %14, %22;\n\t"
       "subc.u32    %7, %15, %23;"
-      : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7])
-      : "r"(z[0]), "r"(z[1]), "r"(z[2]), "r"(z[3]), "r"(z[4]), "r"(z[5]), "r"(z[6]), "r"(z[7]), "r"(qp[0]),
-        "r"(qp[1]), "r"(qp[2]), "r"(qp[3]), "r"(qp[4]), "r"(qp[5]), "r"(qp[6]), "r"(qp[7]));
+      : "=&r"(d[0]), "=&r"(d[1]), "=&r"(d[2]), "=&r"(d[3]), "=&r"(d[4]), "=&r"(d[5]), "=&r"(d[6]), "=&r"(d[7])
+      : "r"(z[0]), "r"(z[1]), "r"(z[2]), "r"(z[3]), "r"(z[4]), "r"(z[5]), "r"(z[6]), "r"(z[7]), "r"(e[0]),
+        "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]));
+  asm("sub.cc.u32  %0, %0, %7;\n\t"
+      "subc.cc.u32 %1, %1, %8;\n\t"
+      "subc.cc.u32 %2, %2, %9;\n\t"
+      "subc.cc.u32 %3, %3, %10;\n\t"
+      "subc.cc.u32 %4, %4, %11;\n\t"
+      "subc.cc.u32 %5, %5, %12;\n\t"
+      "subc.u32    %6, %6, %13;"
+      : "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7])
+      : "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]));
   if (lazy) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) r[j] = d[j];
