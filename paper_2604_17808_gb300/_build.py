@@ -24,8 +24,7 @@ LIB_PATH = os.path.join(OUT_DIR, LIB_NAME)
 # hooks) are compiled again; the rest are the release objects.
 DEBUG_LIB_PATH = os.path.join(OUT_DIR, "libntt_gb300_debug.so")
 DEBUG_OBJ_DIR = os.path.join(HERE, "_build_debug")
-DEBUG_UNITS = ("ntt_plan.cu", "kernels_bls12_381_pass10.cu", "kernels_bls12_381_pass11.cu",
-               "kernels_bls12_381_batch.cu", "kernels_bn254_pass10.cu", "kernels_bn254_pass11.cu",
+DEBUG_UNITS = ("ntt_plan.cu", "kernels_bls12_381_pass.cu", "kernels_bls12_381_batch.cu", "kernels_bn254_pass.cu",
                "kernels_bn254_batch.cu")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

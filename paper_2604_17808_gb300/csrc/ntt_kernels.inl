@@ -4,7 +4,7 @@
 // NTT_NS (a namespace for the field's launchers) and one NTT_PART_* macro,
 // so that the kernel families of a field compile in parallel, one nvcc
 // process each:
-//   NTT_PART_PASS = 10 or 11  the pass kernels of one tile shape;
+//   NTT_PART_PASS             the pass kernels;
 //   NTT_PART_BATCH            the persistent batched kernel;
 //   NTT_PART_MATRIX           the matrix-form (tensor-core) pass;
 //   NTT_PART_MISC             table generators, element-wise kernels and
@@ -16,10 +16,8 @@ namespace gb300ntt {
 namespace NTT_NS {
 
 // launchers defined by the other parts of this field
-cudaError_t prepare_pass10();
-cudaError_t prepare_pass11();
-cudaError_t pass10(int logs, int mode, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st);
-cudaError_t pass11(int logs, int mode, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st);
+cudaError_t prepare_pass();
+cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st);
 cudaError_t prepare_batch();
 cudaError_t batch(const BatchLaunch &b, cudaStream_t st);
 cudaError_t prepare_matrix();
@@ -41,7 +39,7 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
-// Launch with programmatic stream serialisation (see pdl_trigger_and_wait):
+// Launch with programmatic stream serialisation (see pdl_wait_and_trigger):
 // consecutive passes overlap their launch latency and CTA scheduling.
 template <class K, class... A>
 cudaError_t launch_pdl(K kernel, dim3 grid, dim3 block, int smem, cudaStream_t st, const A &...a) {
@@ -70,142 +68,58 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t *p) {
 
 namespace {
 
-// The fused tile is instantiated for the 1024-element tile only: that is
-// the shape of the one-wave passes it is chosen for (sizes up to 2^20).
-template <int LOGS, int TL>
-constexpr bool has_fused() {
-  return TL == 10 && LOGS >= 4;
-}
-
-template <int LOGS, int MODE, int TL>
+template <int MODE>
 cudaError_t set_pass_attr() {
-  cudaError_t e = cudaFuncSetAttribute(ntt_pass_kernel<F, LOGS, MODE, TL, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, TileCfg<TL>::kBytes);
-  if constexpr (has_fused<LOGS, TL>()) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ntt_pass_kernel<F, LOGS, MODE, TL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               TileCfg<TL>::kBytes);
-  }
+  cudaError_t e = cudaFuncSetAttribute(ntt_pass_kernel<F, MODE, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       128 * 8 * 32);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(ntt_pass_kernel<F, MODE, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 8 * 32);
   return e;
 }
 
-template <int LOGS, int TL>
-cudaError_t set_pass_attrs() {
-  cudaError_t e = set_pass_attr<LOGS, kModeInner, TL>();
-  if (e == cudaSuccess) e = set_pass_attr<LOGS, kModeFirst, TL>();
-  if (e == cudaSuccess) e = set_pass_attr<LOGS, kModeFirstPre, TL>();
-  return e;
-}
-
-template <int TL>
-cudaError_t set_all_pass_attrs() {
-  cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = set_pass_attrs<1, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<2, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<3, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<4, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<5, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<6, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<7, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<8, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<9, TL>();
-  if (e == cudaSuccess) e = set_pass_attrs<10, TL>();
-  if constexpr (TL >= 11) {
-    if (e == cudaSuccess) e = set_pass_attrs<11, TL>();
-  }
-  return e;
-}
-
-template <int LOGS, int TL, bool FUSED>
-cudaError_t pass_launch(int mode, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  const dim3 grid((unsigned)tiles), block(TileCfg<TL>::kThreads);
-  const int smem = TileCfg<TL>::kBytes;
-  switch (mode) {
-    case kModeInner: return launch_pdl(ntt_pass_kernel<F, LOGS, kModeInner, TL, FUSED>, grid, block, smem, st, a);
-    case kModeFirst: return launch_pdl(ntt_pass_kernel<F, LOGS, kModeFirst, TL, FUSED>, grid, block, smem, st, a);
-    case kModeFirstPre:
-      return launch_pdl(ntt_pass_kernel<F, LOGS, kModeFirstPre, TL, FUSED>, grid, block, smem, st, a);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <int LOGS, int TL>
-cudaError_t pass_logs(int mode, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  if constexpr (has_fused<LOGS, TL>()) {
-    if (fused) return pass_launch<LOGS, TL, true>(mode, a, tiles, st);
-  }
-  return pass_launch<LOGS, TL, false>(mode, a, tiles, st);
-}
-
-template <int TL>
-cudaError_t pass_tl(int logs, int mode, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  switch (logs) {
-    case 1: return pass_logs<1, TL>(mode, fused, a, tiles, st);
-    case 2: return pass_logs<2, TL>(mode, fused, a, tiles, st);
-    case 3: return pass_logs<3, TL>(mode, fused, a, tiles, st);
-    case 4: return pass_logs<4, TL>(mode, fused, a, tiles, st);
-    case 5: return pass_logs<5, TL>(mode, fused, a, tiles, st);
-    case 6: return pass_logs<6, TL>(mode, fused, a, tiles, st);
-    case 7: return pass_logs<7, TL>(mode, fused, a, tiles, st);
-    case 8: return pass_logs<8, TL>(mode, fused, a, tiles, st);
-    case 9: return pass_logs<9, TL>(mode, fused, a, tiles, st);
-    case 10: return pass_logs<10, TL>(mode, fused, a, tiles, st);
-    case 11:
-      if constexpr (TL >= 11) return pass_logs<11, TL>(mode, fused, a, tiles, st);
-      return cudaErrorInvalidValue;
-    default: return cudaErrorInvalidValue;
-  }
+template <int MODE>
+cudaError_t pass_mode(const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
+  const dim3 grid((unsigned)tiles), block(1u << (s.tl - s.pl));
+  const int smem = 32 << s.tl;
+  if (block.x <= 128) return launch_pdl(ntt_pass_kernel<F, MODE, 128>, grid, block, smem, st, a, s);
+  return launch_pdl(ntt_pass_kernel<F, MODE, 256>, grid, block, smem, st, a, s);
 }
 
 }  // namespace
 
-#if NTT_PART_PASS == 10
-cudaError_t prepare_pass10() { return set_all_pass_attrs<10>(); }
-cudaError_t pass10(int logs, int mode, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  return pass_tl<10>(logs, mode, fused, a, tiles, st);
+cudaError_t prepare_pass() {
+  cudaError_t e = set_pass_attr<kModeInner>();
+  if (e == cudaSuccess) e = set_pass_attr<kModeFirst>();
+  if (e == cudaSuccess) e = set_pass_attr<kModeFirstPre>();
+  return e;
 }
-#else
-cudaError_t prepare_pass11() { return set_all_pass_attrs<11>(); }
-cudaError_t pass11(int logs, int mode, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  return pass_tl<11>(logs, mode, fused, a, tiles, st);
+
+cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
+  if (s.pl < 1 || s.pl > 3 || s.tl > 11 || s.logs < 1 || s.logs > s.tl || s.tl - s.pl > 8)
+    return cudaErrorInvalidValue;
+  switch (mode) {
+    case kModeInner: return pass_mode<kModeInner>(s, a, tiles, st);
+    case kModeFirst: return pass_mode<kModeFirst>(s, a, tiles, st);
+    case kModeFirstPre: return pass_mode<kModeFirstPre>(s, a, tiles, st);
+    default: return cudaErrorInvalidValue;
+  }
 }
-#endif
 
 #elif defined(NTT_PART_BATCH)
 
 namespace {
 
-// One tile of one segment.  Each (size, mode) variant is a separate,
-// non-inlined function: the call costs nothing next to a 2048-element tile,
-// and ptxas then compiles 33 small functions instead of one kernel holding
-// every variant inline (which took minutes).
-template <int LOGS, int MODE>
+// One tile of one segment (a non-inlined function per mode).
+template <int MODE>
 __device__ __noinline__ void batch_tile_fn(const BatchSeg &sg, uint64_t tile, uint4 *smem) {
-  pass_tile<F, LOGS, MODE, true, 11, true>(sg.a, tile, smem);
-}
-
-template <int LOGS>
-__device__ __forceinline__ void batch_tile_logs(const BatchSeg &sg, uint64_t tile, uint4 *smem) {
-  switch (sg.mode) {
-    case kModeInner: batch_tile_fn<LOGS, kModeInner>(sg, tile, smem); break;
-    case kModeFirst: batch_tile_fn<LOGS, kModeFirst>(sg, tile, smem); break;
-    default: batch_tile_fn<LOGS, kModeFirstPre>(sg, tile, smem); break;
-  }
+  pass_tile<F, MODE>(sg.a, TileShape{sg.logs, (uint32_t)kTileLog, 3u}, tile, smem);
 }
 
 __device__ __forceinline__ void batch_tile(const BatchSeg &sg, uint64_t tile, uint4 *smem) {
-  switch (sg.logs) {
-    case 1: batch_tile_logs<1>(sg, tile, smem); break;
-    case 2: batch_tile_logs<2>(sg, tile, smem); break;
-    case 3: batch_tile_logs<3>(sg, tile, smem); break;
-    case 4: batch_tile_logs<4>(sg, tile, smem); break;
-    case 5: batch_tile_logs<5>(sg, tile, smem); break;
-    case 6: batch_tile_logs<6>(sg, tile, smem); break;
-    case 7: batch_tile_logs<7>(sg, tile, smem); break;
-    case 8: batch_tile_logs<8>(sg, tile, smem); break;
-    case 9: batch_tile_logs<9>(sg, tile, smem); break;
-    case 10: batch_tile_logs<10>(sg, tile, smem); break;
-    default: batch_tile_logs<11>(sg, tile, smem); break;
+  switch (sg.mode) {
+    case kModeInner: batch_tile_fn<kModeInner>(sg, tile, smem); break;
+    case kModeFirst: batch_tile_fn<kModeFirst>(sg, tile, smem); break;
+    default: batch_tile_fn<kModeFirstPre>(sg, tile, smem); break;
   }
 }
 
@@ -376,6 +290,21 @@ __global__ void gen_1d_kernel(uint4 *out, uint64_t count, const Pow2Table pw, co
   }
 }
 
+// Table of the DFT twiddles: entry i holds base^i as the residues of mul_split,
+// A = base^i 2^128 and B = base^i 2^256 mod p.
+__global__ void gen_split_kernel(uint4 *out, uint64_t count, const Pow2Table pw, const Fe32 one) {
+  const uint32_t r128[8] = {0, 0, 0, 0, 1, 0, 0, 0};
+  for (uint64_t idx = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; idx < count;
+       idx += (uint64_t)gridDim.x * blockDim.x) {
+    uint32_t acc[8], low[8];
+    fe_from_param(acc, one);
+    ladder_mul(acc, idx, pw);
+    mont_mul<F>(low, acc, r128);
+    fe_store_global(out, 2 * idx, low);
+    fe_store_global(out, 2 * idx + 1, acc);
+  }
+}
+
 __global__ void mul_vec_kernel(uint4 *out, const uint4 *a, const uint4 *b, uint64_t count) {
   for (uint64_t idx = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; idx < count;
        idx += (uint64_t)gridDim.x * blockDim.x) {
@@ -440,17 +369,10 @@ __global__ void mul_rep_coop_kernel(uint32_t *out, const uint32_t *a, const uint
 }
 
 cudaError_t prepare() {
-  cudaError_t e = prepare_pass11();
+  cudaError_t e = prepare_pass();
   if (e == cudaSuccess) e = prepare_matrix();
-  if (e == cudaSuccess) e = prepare_pass10();
   if (e == cudaSuccess) e = prepare_batch();
   return e;
-}
-
-cudaError_t pass(int logs, int mode, int tl, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  if (tl == 11) return pass11(logs, mode, fused, a, tiles, st);
-  if (tl == 10) return pass10(logs, mode, fused, a, tiles, st);
-  return cudaErrorInvalidValue;
 }
 
 unsigned grid_for(uint64_t count) {
@@ -467,6 +389,11 @@ cudaError_t gen_2d(uint4 *out, uint32_t log_s, uint32_t log_mp, const Pow2Table 
 
 cudaError_t gen_1d(uint4 *out, uint64_t count, const Pow2Table &pw, Fe32 init, cudaStream_t st) {
   gen_1d_kernel<<<grid_for(count), 256, 0, st>>>(out, count, pw, init);
+  return cudaGetLastError();
+}
+
+cudaError_t gen_split(uint4 *out, uint64_t count, const Pow2Table &pw, Fe32 one, cudaStream_t st) {
+  gen_split_kernel<<<grid_for(count), 256, 0, st>>>(out, count, pw, one);
   return cudaGetLastError();
 }
 
@@ -493,7 +420,8 @@ cudaError_t quotient(uint4 *out, const uint4 *a, const uint4 *b, const uint4 *c,
   return cudaGetLastError();
 }
 
-const FieldLaunchers kLaunchers = {prepare, pass, gen_2d, gen_1d, mul_vec, batch, mul_rep, matrix_pass, quotient};
+const FieldLaunchers kLaunchers = {prepare, pass,    gen_2d,      gen_1d,  gen_split,
+                                   mul_vec, batch,   mul_rep,     matrix_pass, quotient};
 
 }  // namespace
 

@@ -59,14 +59,15 @@ struct BatchLaunch {
 
 struct FieldLaunchers {
   cudaError_t (*prepare)();
-  // one pass; tl = log2 of the tile (10 or 11), logs <= tl; fused selects the
-  // fused tile where one exists (tl = 10, logs >= 4), else the staged one
-  cudaError_t (*pass)(int logs, int mode, int tl, bool fused, const PassArgs &a, uint64_t tiles, cudaStream_t st);
+  // one pass over `tiles` tiles of the given shape
+  cudaError_t (*pass)(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st);
   // out[n * Mp + q] = init * fac[n] * base^(n*q)    (fac may be null)
   cudaError_t (*gen_2d)(uint4 *out, uint32_t log_s, uint32_t log_mp, const Pow2Table &pw, const uint4 *fac,
                         Fe32 init, cudaStream_t st);
   // out[i] = init * base^i, i < count
   cudaError_t (*gen_1d)(uint4 *out, uint64_t count, const Pow2Table &pw, Fe32 init, cudaStream_t st);
+  // the same as pairs of residues for mul_split (fp256.cuh), 64 bytes per entry
+  cudaError_t (*gen_split)(uint4 *out, uint64_t count, const Pow2Table &pw, Fe32 one, cudaStream_t st);
   // out[i] = a[i] * b[i] * 2^-256 (element-wise Montgomery product; tests)
   cudaError_t (*mul_vec)(uint4 *out, const uint4 *a, const uint4 *b, uint64_t count, cudaStream_t st);
   // persistent batched kernel over the items of `b`

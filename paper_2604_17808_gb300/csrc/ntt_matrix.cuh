@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(kMatThreads, 1)
     load_e(tile_q(u_begin));
     e_issued = 1;
   }
-  pdl_trigger_and_wait();
+  pdl_wait_and_trigger();
 
   if (warp == 0) {
     // ------------------------------------------------------ MMA issuer

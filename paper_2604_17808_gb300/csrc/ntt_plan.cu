@@ -3,7 +3,8 @@
 // A plan fixes (field, log_n), splits N into passes of at most 2^8 points
 // (the four-step / six-step decomposition of ntt_pass.cuh), and builds on
 // the device every constant the passes multiply by, in Montgomery form:
-//   * per distinct pass size S: omega_S^i and omega_S^-i, i < S/2;
+//   * per distinct pass size S: omega_S^i and omega_S^-i, i < S/2 (two
+//     residues each, see mul_split in fp256.cuh);
 //   * per pass j >= 1 and kind: the inter-pass table omega_M^(n q) [S_j][Mp]
 //     (inverse: omega^-1 and, in the last pass, N^-1; coset: times
 //     s^(n * N/M) for the digit the pass transforms);
@@ -205,8 +206,8 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
       if (p->dft_tw[dir][logs]) continue;
       const U256 w = square_times(F, dir ? p->omega_inv : p->omega, log_n - logs);
       const uint64_t count = std::max<uint64_t>(1, (1ull << logs) / 2);
-      NTT_TRY(alloc_tab(p, &p->dft_tw[dir][logs], count));
-      NTT_CUDA(L.gen_1d(p->dft_tw[dir][logs], count, make_ladder(F, w), one, st));
+      NTT_TRY(alloc_tab(p, &p->dft_tw[dir][logs], 2 * count));
+      NTT_CUDA(L.gen_split(p->dft_tw[dir][logs], count, make_ladder(F, w), one, st));
     }
   }
   // inter-pass tables (forward, inverse)
@@ -278,12 +279,21 @@ void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j
   a->dbg_err = p->d_err;
 }
 
-// Tile structure of a pass: the fused tile when the pass is one wave of
-// 1024-element tiles (every CTA resident at once, 7 per SM), the staged
-// tile otherwise (see pass_tile in ntt_pass.cuh for the measurements).
-bool use_fused_tile(ntt_plan p, uint32_t logs, uint32_t tl) {
-  return tl == 10 && logs >= 4 &&
-         pass_tiles(p->log_n, logs, tl) <= (uint64_t)p->sm_count * (uint64_t)TileCfg<10>::kMinBlocks;
+// Tile of a pass launch.  Elements per thread (2^pl) trade parallelism for
+// barriers: as few as still fit the GPU at once (7 CTAs of 128 threads per SM)
+// while a sub-transform fits 128 threads, so that a small transform is spread
+// over as many warps as there are and its serial chain is short: 2 up to 2^18
+// points, 4 at 2^19, 8 from 2^20 on (and for sub-transforms of 2^9 and 2^10
+// points 4 and 8).  Tiles of the small shapes hold one sub-transform (at least
+// one warp).
+TileShape pass_shape(ntt_plan p, uint32_t logs, uint32_t tl) {
+  if (tl != 10) return TileShape{logs, tl, 3};
+  const uint64_t slots = (uint64_t)p->sm_count * 128u * (uint64_t)TileBounds<128>::kMinBlocks;
+  for (uint32_t pl = 1; pl < 3; ++pl) {
+    const uint32_t t = std::max(logs, pl + 5);
+    if (t - pl <= 7 && (1ull << p->log_n) >> pl <= slots) return TileShape{logs, t, pl};
+  }
+  return TileShape{logs, tl, 3};
 }
 
 // Enqueue one transform: one kernel launch per pass.
@@ -298,9 +308,8 @@ ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cu
     if (shrink) a.n_vec >>= 1;
     const uint32_t logs = p->pass_log[j];
     cudaError_t e = timing_begin(p, (int)j, st);
-    const uint32_t tl = p->pass_tl[j];
-    if (e == cudaSuccess)
-      e = L.pass((int)logs, mode, (int)tl, use_fused_tile(p, logs, tl), a, pass_tiles(p->log_n, logs, tl), st);
+    const TileShape shape = pass_shape(p, logs, p->pass_tl[j]);
+    if (e == cudaSuccess) e = L.pass(mode, shape, a, pass_tiles(p->log_n, logs, shape.tl), st);
     if (e == cudaSuccess) e = timing_end(p, st);
     if (e != cudaSuccess) return cuda_status(e);
   }
@@ -503,8 +512,11 @@ ntt_status ntt_plan_read_table(ntt_plan plan, ntt_kind kind, uint32_t pass, uint
   const uint32_t logs = plan->pass_log[pass];
   const uint4 *src = nullptr;
   uint64_t size = 0;
+  uint32_t stride = 2;   // uint4 per entry
   if (table == 0) {
     src = plan->dft_tw[tk == kInverse ? 1 : 0][logs];
+    if (src) src += 2;   // the second residue is the Montgomery form
+    stride = 4;
     size = std::max<uint64_t>(1, (1ull << logs) / 2);
   } else if (table == 1) {
     if (pass == 0) {
@@ -524,7 +536,8 @@ ntt_status ntt_plan_read_table(ntt_plan plan, ntt_kind kind, uint32_t pass, uint
   }
   if (!src || first > size || count > size - first) return NTT_ERR_INVALID_ARG;
   std::vector<uint64_t> buf(count * 4);
-  NTT_CUDA(cudaMemcpy(buf.data(), src + 2 * first, count * 32, cudaMemcpyDeviceToHost));
+  if (count)
+    NTT_CUDA(cudaMemcpy2D(buf.data(), 32, src + stride * first, 16 * stride, 32, count, cudaMemcpyDeviceToHost));
   const HostField F = host_field(plan->field);
   const U256 rinv = F.r_inv();
   uint64_t *o = (uint64_t *)h_out;
