@@ -157,42 +157,63 @@ __device__ __forceinline__ uint32_t swz(uint32_t e) {
   return ((kSwzLut0 >> (3 * x0)) ^ (kSwzLut1 >> (3 * x1)) ^ (kSwzLut2 >> (3 * x2))) & 7u;
 }
 
-// Chunk of the low half of element e; the high half is chunk ^ 1.
-__device__ __forceinline__ uint32_t tile_chunk(uint32_t e) { return (e << 1) ^ swz(e); }
+// Byte offset in the tile of the low half of element e; the high half is at
+// the offset ^ 16.
+__device__ __forceinline__ uint32_t tile_offset(uint32_t e) { return ((e << 1) ^ swz(e)) << 4; }
 
-__device__ __forceinline__ void tile_store(uint4 *tile, uint32_t c, const uint32_t a[8]) {
-  tile[c] = make_uint4(a[0], a[1], a[2], a[3]);
-  tile[c ^ 1u] = make_uint4(a[4], a[5], a[6], a[7]);
+// `tile`: shared-memory address of the tile.  (The accesses keep their program
+// order: no address is formed twice, and a thread reads back what it wrote.)
+__device__ __forceinline__ void tile_store(uint32_t tile, uint32_t off, const uint32_t a[8]) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + off), "r"(a[0]), "r"(a[1]), "r"(a[2]),
+               "r"(a[3])
+               : "memory");
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + (off ^ 16u)), "r"(a[4]), "r"(a[5]), "r"(a[6]),
+               "r"(a[7])
+               : "memory");
 }
 
-__device__ __forceinline__ void tile_load(uint32_t r[8], const uint4 *tile, uint32_t c) {
-  const uint4 lo = tile[c];
-  const uint4 hi = tile[c ^ 1u];
-  r[0] = lo.x; r[1] = lo.y; r[2] = lo.z; r[3] = lo.w;
-  r[4] = hi.x; r[5] = hi.y; r[6] = hi.z; r[7] = hi.w;
+__device__ __forceinline__ void tile_load(uint32_t r[8], uint32_t tile, uint32_t off) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(tile + off)
+               : "memory");
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(tile + (off ^ 16u))
+               : "memory");
 }
 
 // Global -> shared copy of one element without registers, through L2 (data
 // that another CTA wrote earlier in the same launch is read coherently).
-__device__ __forceinline__ void tile_copy_async(uint4 *tile, uint32_t c, const uint4 *base, uint64_t elem) {
-  const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(tile + c);
-  const uint32_t s1 = (uint32_t)__cvta_generic_to_shared(tile + (c ^ 1u));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s0), "l"(base + 2 * elem) : "memory");
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s1), "l"(base + 2 * elem + 1) : "memory");
+__device__ __forceinline__ void tile_copy_async(uint32_t tile, uint32_t off, const uint4 *base, uint64_t elem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tile + off), "l"(base + 2 * elem) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tile + (off ^ 16u)), "l"(base + 2 * elem + 1)
+               : "memory");
 }
 
 __device__ __forceinline__ void tile_copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Twiddle entry w of the DFT table (mul_split's residues).
+__device__ __forceinline__ void load_twiddle(uint32_t A[8], uint32_t B[8], const uint4 *dft_tw, uint32_t w) {
+  const char *p = reinterpret_cast<const char *>(dft_tw) + (w << 6);
+  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(A[0]), "=r"(A[1]), "=r"(A[2]), "=r"(A[3]), "=r"(A[4]), "=r"(A[5]), "=r"(A[6]), "=r"(A[7])
+      : "l"(p));
+  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8+32];"
+      : "=r"(B[0]), "=r"(B[1]), "=r"(B[2]), "=r"(B[3]), "=r"(B[4]), "=r"(B[5]), "=r"(B[6]), "=r"(B[7])
+      : "l"(p));
+}
+
 // ----------------------------------------------------------- butterflies
 
-// A thread's 2^pl elements of one round: chunk of the first, and the chunk
-// differences of the private index bits (element j: base ^ sum of the set
-// bits' differences).
+// A thread's 2^pl elements of one round: tile offset of the first, and the
+// offset differences of the private index bits (element j: base ^ the set bits'
+// differences).
 struct Private {
   uint32_t base, d0, d1, d2;
 };
 
-__device__ __forceinline__ uint32_t private_chunk(const Private &v, uint32_t j) {
+__device__ __forceinline__ uint32_t private_offset(const Private &v, uint32_t j) {
   return v.base ^ ((j & 1u) ? v.d0 : 0u) ^ ((j & 2u) ? v.d1 : 0u) ^ ((j & 4u) ? v.d2 : 0u);
 }
 
@@ -201,10 +222,10 @@ __device__ __forceinline__ uint32_t private_chunk(const Private &v, uint32_t j) 
 __device__ __forceinline__ Private private_set(const TileShape &s, uint32_t e, uint32_t T, uint32_t r) {
   const uint32_t top = s.tl - s.pl;   // private bit k >= r is index bit top + k
   Private v;
-  v.base = tile_chunk(e);
-  v.d0 = tile_chunk(1u << (r > 0 ? T : top));
-  v.d1 = tile_chunk(1u << (r > 1 ? T + 1 : top + 1));
-  v.d2 = tile_chunk(1u << (r > 2 ? T + 2 : top + 2));
+  v.base = tile_offset(e);
+  v.d0 = tile_offset(1u << (r > 0 ? T : top));
+  v.d1 = tile_offset(1u << (r > 1 ? T + 1 : top + 1));
+  v.d2 = tile_offset(1u << (r > 2 ? T + 2 : top + 2));
   return v;
 }
 
@@ -212,7 +233,7 @@ __device__ __forceinline__ Private private_set(const TileShape &s, uint32_t e, u
 // b, twiddle omega_S^((p mod h) S / 2h) with h = 2^(T + b), p the position in
 // the sub-transform; low = its bits below T.
 template <class F>
-__device__ __forceinline__ void private_stages(uint4 *tile, const uint4 *dft_tw, const TileShape &s, const Private &v,
+__device__ __forceinline__ void private_stages(uint32_t tile, const uint4 *dft_tw, const TileShape &s, const Private &v,
                                                uint32_t T, int hi, int lo, uint32_t low) {
 #pragma unroll 1
   for (int b = hi - 1; b >= lo; --b) {
@@ -221,8 +242,8 @@ __device__ __forceinline__ void private_stages(uint4 *tile, const uint4 *dft_tw,
 #pragma unroll 1
     for (uint32_t i = 0; i < (1u << (s.pl - 1)); ++i) {
       const uint32_t j = (i & mask) | ((i & ~mask) << 1);
-      const uint32_t c = private_chunk(v, j);
-      const uint64_t w = (uint64_t)((low | ((j & mask) << T)) << sh);
+      const uint32_t c = private_offset(v, j);
+      const uint32_t w = (low | ((j & mask) << T)) << sh;
       uint32_t x[8], y[8], d[8];
       if (T == 0 && (j & mask) == 0) {   // twiddle 1, for every thread
         tile_load(x, tile, c);
@@ -234,8 +255,7 @@ __device__ __forceinline__ void private_stages(uint4 *tile, const uint4 *dft_tw,
         continue;
       }
       uint32_t A[8], B[8];
-      fe_load_global(A, dft_tw, 2 * w);
-      fe_load_global(B, dft_tw, 2 * w + 1);
+      load_twiddle(A, B, dft_tw, w);
       tile_load(x, tile, c);
       tile_load(y, tile, c ^ db);
       sub_lazy<F>(d, x, y);
@@ -277,7 +297,8 @@ __device__ __forceinline__ uint64_t elem_pos(const PassArgs &a, uint32_t logs, u
 // Process tile `tile` of one pass.  All threads of the CTA call this; the
 // caller separates two tiles on the same shared memory with a barrier.
 template <class F, int MODE>
-__device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, uint64_t tile, uint4 *smem) {
+__device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, uint64_t tile, uint4 *smem_tile) {
+  const uint32_t smem = (uint32_t)__cvta_generic_to_shared(smem_tile);
   const uint32_t t = threadIdx.x, logs = s.logs, pl = s.pl;
   const uint32_t logg = s.tl - logs;                 // log2 of the tile's sub-transforms
   const uint64_t d0 = tile << logg;
@@ -293,12 +314,18 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     const uint32_t dl = t & ((1u << gbits) - 1u), low = t >> gbits;
     const Private v = private_set(s, (dl << logs) | low, T, r);
     const uint32_t count = 1u << pl, rmask = (1u << r) - 1u;
+    // element j is input low + ((j mod 2^r) << T) of sub-transform d; with r =
+    // pl (all but sub-transforms of 2 and 4 points) its position is linear in j
+    const uint64_t dfirst = d0 + dl, step = 1ull << (a.log_mp + T);
+    const bool linear = r == pl;
+    auto sub_of = [&](uint32_t j) { return dfirst + ((uint64_t)(j >> r) << gbits); };
+    uint64_t pos = elem_pos<MODE>(a, logs, dfirst, low);
 #pragma unroll 1
-    for (uint32_t j = 0; j < count; ++j) {
-      const uint64_t d = d0 + dl + ((uint64_t)(j >> r) << gbits);
+    for (uint32_t j = 0; j < count; ++j, pos += step) {
+      const uint64_t d = linear ? dfirst : sub_of(j);
+      if (!linear) pos = elem_pos<MODE>(a, logs, d, low | ((j & rmask) << T));
       if (d >= a.num_sub) continue;
-      const uint64_t pos = elem_pos<MODE>(a, logs, d, low | ((j & rmask) << T));
-      const uint32_t c = private_chunk(v, j);
+      const uint32_t c = private_offset(v, j);
       if (dbg_in(a, pos, a.n_vec)) {
         tile_copy_async(smem, c, a.src, pos);
       } else {
@@ -309,25 +336,31 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     }
     if constexpr (MODE != kModeFirst) {
       // the multiplier of the next element is on its way during a product
-      auto load_mul = [&](uint32_t w[8], uint32_t j) {
-        const uint64_t d = d0 + dl + ((uint64_t)(j >> r) << gbits);
-        const uint32_t n = low | ((j & rmask) << T);
-        const uint64_t wi = MODE == kModeInner ? ((uint64_t)n << a.log_mp) + (d & ((1ull << a.log_mp) - 1)) : n;
-        if (d < a.num_sub && dbg_in(a, wi, a.n_mul)) fe_load_global(w, a.mul, wi);
-        else fe_zero(w);
+      const uint64_t q_mask = (1ull << a.log_mp) - 1;
+      auto mul_of = [&](uint64_t d, uint32_t n) {
+        return MODE == kModeInner ? ((uint64_t)n << a.log_mp) + (d & q_mask) : (uint64_t)n;
       };
+      const uint64_t wstep = MODE == kModeInner ? step : 1ull << T;
+      uint64_t wi = mul_of(dfirst, low);
       uint32_t w[8], next[8];
-      load_mul(w, 0);
+      auto load_mul = [&](uint32_t x[8], uint32_t j) {
+        const uint64_t d = linear ? dfirst : sub_of(j);
+        if (!linear) wi = mul_of(d, low | ((j & rmask) << T));
+        if (d < a.num_sub && dbg_in(a, wi, a.n_mul)) fe_load_global(x, a.mul, wi);
+        else fe_zero(x);
+        wi += wstep;
+      };
+      load_mul(next, 0);
       tile_copy_wait();
 #pragma unroll 1
       for (uint32_t j = 0; j < count; ++j) {
-        const uint32_t c = private_chunk(v, j);
-        load_mul(next, j + 1 < count ? j + 1 : j);
+        const uint32_t c = private_offset(v, j);
+        fe_copy(w, next);
+        if (j + 1 < count) load_mul(next, j + 1);
         uint32_t x[8];
         tile_load(x, smem, c);
         mont_mul_lazy<F>(x, w, x);
         tile_store(smem, c, x);
-        fe_copy(w, next);
       }
     } else {
       tile_copy_wait();
@@ -361,7 +394,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
 #pragma unroll 1
   for (uint32_t j = 0; j < (1u << pl); j += group) {
     const uint64_t d = d0 + dl + ((uint64_t)(j >> last) << gbits);
-    const uint32_t c = private_chunk(v, j);
+    const uint32_t c = private_offset(v, j);
     const uint32_t k = __brev(p0 | (j & lmask)) >> (32 - logs);   // output of the group's first position
     uint64_t out = 0;
     uint32_t sh = 0;
@@ -376,8 +409,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
       uint32_t x2[8], x3[8];
       {
         uint32_t A[8], B[8];   // omega_4 = omega_S^(S/4)
-        fe_load_global(A, a.dft_tw, 2 * (uint64_t)(half >> 1));
-        fe_load_global(B, a.dft_tw, 2 * (uint64_t)(half >> 1) + 1);
+        load_twiddle(A, B, a.dft_tw, half >> 1);
         tile_load(x1, smem, c ^ v.d0);
         tile_load(x3, smem, c ^ v.d0 ^ v.d1);
         sub_lazy<F>(y, x1, x3);
