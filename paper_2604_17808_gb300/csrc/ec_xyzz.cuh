@@ -37,7 +37,6 @@ static_assert(FieldBn254Fq::P0 * (0u - FieldBn254Fq::NP) == 1u, "NP");
 
 struct FqBn254 {
   static constexpr int L = 8;
-  static constexpr int kTopBit = 253;  // q < 2^254
   using F = FieldBn254Fq;
   __device__ static void mul(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) { mont_mul<F>(r, a, b); }
   __device__ static void add(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) { add_mod<F>(r, a, b); }
@@ -50,10 +49,9 @@ struct FqBn254 {
       if (a[j] != p[j]) return a[j] < p[j];
     return false;
   }
-  // exponent q - 2 (inversion by Fermat), limb j
-  __device__ static uint32_t inv_exp(int j) {
-    const uint32_t e[8] = {F::P0 - 2u, F::P1, F::P2, F::P3, F::P4, F::P5, F::P6, F::P7};
-    return e[j];
+  __device__ static constexpr uint32_t modulus(int j) {
+    return j == 0 ? F::P0 : j == 1 ? F::P1 : j == 2 ? F::P2 : j == 3 ? F::P3 : j == 4 ? F::P4 : j == 5 ? F::P5
+         : j == 6 ? F::P6 : F::P7;
   }
   __device__ static void load(uint32_t r[8], const uint4 *base, uint64_t e) { fe_load_global(r, base, e); }
   __device__ static void store(uint4 *base, uint64_t e, const uint32_t a[8]) { fe_store_global(base, e, a); }
@@ -61,16 +59,15 @@ struct FqBn254 {
 
 struct FqBls381 {
   static constexpr int L = 12;
-  static constexpr int kTopBit = 380;  // q < 2^381
   using F = FieldBls12381Fq;
   __device__ static void mul(uint32_t r[12], const uint32_t a[12], const uint32_t b[12]) { fp384::mont_mul(r, a, b); }
   __device__ static void add(uint32_t r[12], const uint32_t a[12], const uint32_t b[12]) { fp384::add_mod(r, a, b); }
   __device__ static void sub(uint32_t r[12], const uint32_t a[12], const uint32_t b[12]) { fp384::sub_mod(r, a, b); }
   __device__ static void redc(uint32_t r[12], const uint32_t a[12]) { fp384::mont_redc(r, a); }
   __device__ static bool canonical(const uint32_t a[12]) { return fp384::is_canonical(a); }
-  __device__ static uint32_t inv_exp(int j) {
-    const uint32_t e[12] = {F::P0 - 2u, F::P1, F::P2, F::P3, F::P4, F::P5, F::P6, F::P7, F::P8, F::P9, F::P10, F::P11};
-    return e[j];
+  __device__ static constexpr uint32_t modulus(int j) {
+    return j == 0 ? F::P0 : j == 1 ? F::P1 : j == 2 ? F::P2 : j == 3 ? F::P3 : j == 4 ? F::P4 : j == 5 ? F::P5
+         : j == 6 ? F::P6 : j == 7 ? F::P7 : j == 8 ? F::P8 : j == 9 ? F::P9 : j == 10 ? F::P10 : F::P11;
   }
   __device__ static void load(uint32_t r[12], const uint4 *base, uint64_t e) { fp384::load(r, base, e); }
   __device__ static void store(uint4 *base, uint64_t e, const uint32_t a[12]) { fp384::store(base, e, a); }
@@ -285,22 +282,173 @@ __device__ __forceinline__ void xyzz_add(Xyzz<T> &acc, const Xyzz<T> &q) {
   fv_copy<L>(acc.X, P);
 }
 
-// r = a^(q-2) = a^-1 (Fermat), Montgomery in and out; a = 0 gives 0.
-template <class T>
-__device__ __forceinline__ void f_inverse(uint32_t r[T::L], const uint32_t a[T::L], const uint32_t one[T::L]) {
-  uint32_t acc[T::L];
-  fv_copy<T::L>(acc, one);
-  for (int i = T::kTopBit; i >= 0; --i) {
-    T::mul(acc, acc, acc);
-    if ((T::inv_exp(i >> 5) >> (i & 31)) & 1u) T::mul(acc, acc, a);
+// ------------------------------------------------------------- inversion
+// By division steps (Bernstein and Yang, "Fast constant-time gcd computation
+// and modular inversion", TCHES 2019), 30 at a time: the steps on the low bits
+// of (f, g) give a 2 x 2 matrix with entries up to 2^30, which is then applied
+// to the long f, g (divided by 2^30) and to d, e mod q (divided by 2^30 mod q).
+// From f = q, g = a, d = 0, e = c it ends in g = 0, f = +-1, d = +-c / a.  Long
+// numbers are signed, in 30-bit limbs.  About 25 (254-bit q) or 37 (381-bit)
+// batches of some 600 instructions, against 380 or 570 dependent products of
+// 300 to 600 by Fermat's little theorem: one inversion alone on an SM took 571
+// us over the 381-bit field that way.
+template <int L>
+struct Div30 {
+  static constexpr int N = (32 * L + 29) / 30;   // 9 or 13 limbs: 270, 390 bits
+  static constexpr uint32_t kMask = (1u << 30) - 1u;
+  int32_t v[N];
+};
+
+template <int L>
+__device__ __forceinline__ void div30_from_words(Div30<L> &r, const uint32_t x[L]) {
+#pragma unroll
+  for (int j = 0; j < Div30<L>::N; ++j) {
+    const int bit = 30 * j, w = bit >> 5, sh = bit & 31;
+    const uint32_t lo = w < L ? x[w] : 0u, hi = w + 1 < L ? x[w + 1] : 0u;
+    r.v[j] = (int32_t)(__funnelshift_r(lo, hi, sh) & Div30<L>::kMask);
   }
-  fv_copy<T::L>(r, acc);
+}
+
+// r = a^-1 in Montgomery form for a in Montgomery form (r2 = 2^(64 L) mod q);
+// a = 0 gives 0.
+template <class T>
+__device__ __noinline__ void f_inverse(uint32_t r[T::L], const uint32_t a[T::L], const uint32_t r2[T::L]) {
+  constexpr int L = T::L, N = Div30<L>::N;
+  constexpr uint32_t kMask = Div30<L>::kMask;
+  if (fv_is_zero<L>(a)) {
+    fv_zero<L>(r);
+    return;
+  }
+  Div30<L> q, f, g, d, e;
+  {
+    uint32_t qw[L];
+#pragma unroll
+    for (int j = 0; j < L; ++j) qw[j] = T::modulus(j);
+    div30_from_words<L>(q, qw);
+  }
+  f = q;
+  div30_from_words<L>(g, a);
+  div30_from_words<L>(e, r2);   // a = x R: d ends as R^2 / (x R) = R / x
+#pragma unroll
+  for (int j = 0; j < N; ++j) d.v[j] = 0;
+  int32_t delta = 1;
+  // (49 * 381 + 57) / 17 = 1101 steps always suffice for 381 bits
+#pragma unroll 1
+  for (int batch = 0; batch < 40; ++batch) {
+    int32_t u = 1, v = 0, s = 0, t = 1;   // f' = u f + v g, g' = s f + t g
+    {
+      // 32 low bits of f and g: the 30 steps look at 30 of them
+      uint32_t fl = (uint32_t)f.v[0] | (uint32_t)f.v[1] << 30, gl = (uint32_t)g.v[0] | (uint32_t)g.v[1] << 30;
+      int left = 30;
+#pragma unroll 1
+      for (;;) {
+        const int z = min(left, __clz(__brev(gl)));   // even g: halve it
+        gl >>= z;
+        u = (int32_t)((uint32_t)u << z);
+        v = (int32_t)((uint32_t)v << z);
+        delta += z;
+        left -= z;
+        if (left == 0) break;
+        if (delta > 0) {   // (f, g) -> (g, -f): the sum below is then g - f
+          delta = -delta;
+          const uint32_t x = fl;
+          fl = gl;
+          gl = 0u - x;
+          const int32_t y = u, w = v;
+          u = s;
+          v = t;
+          s = -y;
+          t = -w;
+        }
+        gl += fl;
+        s += u;
+        t += v;
+        // the halving of this step comes with the next run of zeros
+      }
+    }
+    // f, g
+    {
+      int64_t cf = (int64_t)u * f.v[0] + (int64_t)v * g.v[0], cg = (int64_t)s * f.v[0] + (int64_t)t * g.v[0];
+      cf >>= 30;   // the low 30 bits are zero
+      cg >>= 30;
+#pragma unroll
+      for (int j = 1; j < N; ++j) {
+        cf += (int64_t)u * f.v[j] + (int64_t)v * g.v[j];
+        cg += (int64_t)s * f.v[j] + (int64_t)t * g.v[j];
+        f.v[j - 1] = (int32_t)((uint32_t)cf & kMask);
+        g.v[j - 1] = (int32_t)((uint32_t)cg & kMask);
+        cf >>= 30;
+        cg >>= 30;
+      }
+      f.v[N - 1] = (int32_t)cf;
+      g.v[N - 1] = (int32_t)cg;
+    }
+    // d, e: plus the multiple of q, |m| <= 2^29, that makes the low 30 bits
+    // zero; |d|, |e| grow by at most q / 2 per batch, 21 q in all, which the
+    // spare bits of the top limb hold
+    {
+      int64_t cd = (int64_t)u * d.v[0] + (int64_t)v * e.v[0], ce = (int64_t)s * d.v[0] + (int64_t)t * e.v[0];
+      const int32_t md = (int32_t)(((uint32_t)cd * T::F::NP) << 2) >> 2;
+      const int32_t me = (int32_t)(((uint32_t)ce * T::F::NP) << 2) >> 2;
+      cd = (cd + (int64_t)md * q.v[0]) >> 30;
+      ce = (ce + (int64_t)me * q.v[0]) >> 30;
+#pragma unroll
+      for (int j = 1; j < N; ++j) {
+        cd += (int64_t)u * d.v[j] + (int64_t)v * e.v[j];
+        ce += (int64_t)s * d.v[j] + (int64_t)t * e.v[j];
+        cd += (int64_t)md * q.v[j];
+        ce += (int64_t)me * q.v[j];
+        d.v[j - 1] = (int32_t)((uint32_t)cd & kMask);
+        e.v[j - 1] = (int32_t)((uint32_t)ce & kMask);
+        cd >>= 30;
+        ce >>= 30;
+      }
+      d.v[N - 1] = (int32_t)cd;
+      e.v[N - 1] = (int32_t)ce;
+    }
+    int32_t nz = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) nz |= g.v[j];
+    if (nz == 0) break;
+  }
+  // f = 1 or -1 (all limbs' sum: the top limb carries the sign); d f mod q
+  const int32_t sign = f.v[N - 1] < 0 ? -1 : 0;
+  int32_t c = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const int32_t w = (d.v[j] ^ sign) - sign + c;   // +-d, limb by limb
+    c = j + 1 < N ? w >> 30 : 0;
+    d.v[j] = j + 1 < N ? (int32_t)((uint32_t)w & kMask) : w;
+  }
+  // into [0, q): |d| < 22 q
+#pragma unroll 1
+  for (int k = 0; k < 48; ++k) {
+    const bool neg = d.v[N - 1] < 0;
+    Div30<L> w;
+    c = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int32_t x = d.v[j] + (neg ? q.v[j] : -q.v[j]) + c;
+      c = j + 1 < N ? x >> 30 : 0;
+      w.v[j] = j + 1 < N ? (int32_t)((uint32_t)x & kMask) : x;
+    }
+    if (!neg && w.v[N - 1] < 0) break;   // 0 <= d < q
+    d = w;
+  }
+#pragma unroll
+  for (int w = 0; w < L; ++w) {
+    const int bit = 32 * w, j = bit / 30, sh = bit % 30;
+    uint32_t x = (uint32_t)d.v[j] >> sh;
+    if (j + 1 < N) x |= (uint32_t)d.v[j + 1] << (30 - sh);
+    if (60 - sh < 32 && j + 2 < N) x |= (uint32_t)d.v[j + 2] << (60 - sh);
+    r[w] = x;
+  }
 }
 
 // Affine point of p in STANDARD form (x, y); O gives (0, 0).
 template <class T>
 __device__ __forceinline__ void xyzz_to_affine_std(uint32_t x[T::L], uint32_t y[T::L], const Xyzz<T> &p,
-                                                   const uint32_t one[T::L]) {
+                                                   const uint32_t r2[T::L]) {
   constexpr int L = T::L;
   if (xyzz_is_inf(p)) {
     fv_zero<L>(x);
@@ -309,13 +457,130 @@ __device__ __forceinline__ void xyzz_to_affine_std(uint32_t x[T::L], uint32_t y[
   }
   uint32_t t[L], inv[L], zi[L];
   T::mul(t, p.ZZ, p.ZZZ);
-  f_inverse<T>(inv, t, one);  // (ZZ ZZZ)^-1
+  f_inverse<T>(inv, t, r2);  // (ZZ ZZZ)^-1
   T::mul(zi, inv, p.ZZZ);     // ZZ^-1
   T::mul(t, p.X, zi);
   T::redc(x, t);
   T::mul(zi, inv, p.ZZ);      // ZZZ^-1
   T::mul(t, p.Y, zi);
   T::redc(y, t);
+}
+
+// -------------------------------------------------- four lanes per point
+// For the serial tails of the MSM (window merge, upper tree levels, long
+// pieces), where too few points are left to fill the GPU and the time is the
+// depth of dependent products: lane 0 of an aligned group of four holds X, lane
+// 1 Y, lane 2 ZZ, lane 3 ZZZ, and each step is one product per lane, all four
+// at once.  A doubling is 3 products deep instead of 9, an addition 4 instead
+// of 14.  Whole warps call these together (width-4 shuffles of the full warp).
+
+template <int L>
+__device__ __forceinline__ void quad_get(uint32_t r[L], const uint32_t v[L], int src) {
+#pragma unroll
+  for (int j = 0; j < L; ++j) r[j] = __shfl_sync(0xffffffffu, v[j], src, 4);
+}
+
+template <int L>
+__device__ __forceinline__ void quad_pick(uint32_t r[L], bool first, const uint32_t a[L], const uint32_t b[L]) {
+#pragma unroll
+  for (int j = 0; j < L; ++j) r[j] = first ? a[j] : b[j];
+}
+
+// v = 2 v (dbl-2008-s-1, a = 0); O stays O.
+template <class T>
+__device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
+  constexpr int L = T::L;
+  const int lane = threadIdx.x & 3;
+  uint32_t a[L], b[L], p[L], V[L], M[L], q[L], g[L], h[L];
+  T::add(a, v, v);
+  quad_pick<L>(a, lane == 1, a, v);       // lane 1: U = 2 Y; lane 0: X
+  f_mul<T, true>(p, a, a);                // lane 0: X^2, lane 1: V = U^2
+  quad_get<L>(V, p, 1);
+  quad_get<L>(g, p, 0);
+  T::add(M, g, g);
+  T::add(M, M, g);                        // M = 3 X^2
+  quad_pick<L>(a, lane == 3, M, a);
+  quad_pick<L>(a, lane == 2, v, a);
+  quad_pick<L>(b, lane == 3, M, V);
+  f_mul<T, true>(q, a, b);                // S = X V, W = U V, ZZ3 = ZZ V, M^2
+  quad_get<L>(g, q, lane == 0 ? 3 : 1);   // lane 0: M^2, lane 3: W
+  uint32_t x3[L];
+  T::sub(x3, g, q);
+  T::sub(x3, x3, q);                      // lane 0: X3 = M^2 - 2 S
+  T::sub(b, q, x3);                       // lane 0: S - X3
+  quad_pick<L>(a, lane == 0, M, q);
+  quad_pick<L>(a, lane == 3, g, a);
+  quad_pick<L>(b, lane == 0, b, v);
+  f_mul<T, true>(h, a, b);                // lane 0: M (S - X3), lane 1: W Y, lane 3: W ZZZ
+  quad_get<L>(g, h, 0);
+  T::sub(g, g, h);                        // lane 1: Y3
+  quad_pick<L>(v, lane == 0, x3, q);
+  quad_pick<L>(v, lane == 1, g, v);
+  quad_pick<L>(v, lane == 3, h, v);
+}
+
+// v += w (add-2008-s, with the cases it excludes).
+template <class T>
+__device__ __forceinline__ void quad_add(uint32_t v[T::L], const uint32_t w[T::L]) {
+  constexpr int L = T::L;
+  const int lane = threadIdx.x & 3;
+  const bool v_inf = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(v), 2, 4);
+  const bool w_inf = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(w), 2, 4);
+  uint32_t g[L], p[L], d[L], a[L], b[L], q[L], r[L], h[L];
+  quad_get<L>(g, w, lane ^ 2);
+  f_mul<T, true>(p, v, g);                // U1 = X1 ZZ2, S1 = Y1 ZZZ2, U2 = ZZ1 X2, S2 = ZZZ1 Y2
+  quad_get<L>(g, p, lane ^ 2);
+  quad_pick<L>(a, lane < 2, g, p);
+  quad_pick<L>(b, lane < 2, p, g);
+  T::sub(d, a, b);                        // lanes 0, 2: P = U2 - U1; lanes 1, 3: R = S2 - S1
+  const bool same_x = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(d), 0, 4);
+  const bool same_y = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(d), 1, 4);
+  quad_pick<L>(a, lane < 2, d, v);
+  quad_pick<L>(b, lane < 2, d, w);
+  f_mul<T, true>(q, a, b);                // PP, R^2, ZZ1 ZZ2, ZZZ1 ZZZ2
+  quad_get<L>(b, q, 0);                   // PP
+  quad_get<L>(a, d, 0);                   // P
+  quad_pick<L>(a, lane == 0, p, a);
+  quad_pick<L>(a, lane == 2, q, a);
+  f_mul<T, true>(r, a, b);                // Q = U1 PP, PPP, ZZ3, PPP
+  quad_get<L>(g, r, 0);                   // Q
+  uint32_t x3[L];
+  T::sub(x3, q, r);
+  T::sub(x3, x3, g);
+  T::sub(x3, x3, g);                      // lane 1: X3 = R^2 - PPP - 2 Q
+  T::sub(b, g, x3);                       // lane 1: Q - X3
+  quad_get<L>(a, p, 1);                   // S1
+  quad_get<L>(g, r, 1);                   // PPP
+  quad_pick<L>(a, lane == 1, d, a);
+  quad_pick<L>(a, lane == 3, q, a);
+  quad_pick<L>(b, lane == 1, b, g);
+  f_mul<T, true>(h, a, b);                // S1 PPP, R (Q - X3), -, ZZZ3
+  quad_pick<L>(a, lane == 0, h, x3);
+  quad_get<L>(g, a, lane ^ 1);            // lane 0: X3, lane 1: S1 PPP
+  T::sub(b, h, g);                        // lane 1: Y3
+  quad_pick<L>(a, lane == 0, g, r);       // lane 2: ZZ3
+  quad_pick<L>(a, lane == 1, b, a);
+  quad_pick<L>(a, lane == 3, h, a);
+  const bool twice = same_x && same_y && !v_inf && !w_inf;
+  if (__any_sync(0xffffffffu, twice)) {
+    fv_copy<L>(b, v);
+    quad_dbl<T>(b);
+    quad_pick<L>(a, twice, b, a);
+  }
+  const bool opposite = same_x && !same_y && !v_inf && !w_inf;
+#pragma unroll
+  for (int j = 0; j < L; ++j) v[j] = w_inf ? v[j] : v_inf ? w[j] : opposite ? 0u : a[j];
+}
+
+// Coordinate `lane` of point i.
+template <class T>
+__device__ __forceinline__ void quad_load(uint32_t v[T::L], const uint4 *base, uint64_t i) {
+  T::load(v, base, 4 * i + (threadIdx.x & 3));
+}
+
+template <class T>
+__device__ __forceinline__ void quad_store(uint4 *base, uint64_t i, const uint32_t v[T::L]) {
+  T::store(base, 4 * i + (threadIdx.x & 3), v);
 }
 
 }  // namespace gb300ntt

@@ -24,11 +24,12 @@
 //                                      straight to the bucket array and the
 //                                      pieces of the (at most two) buckets
 //                                      that cross its ends to piece slots;
-//                msm_combine_kernel    a pairwise tree over the pieces of each
-//                                      crossing bucket.  Every thread does the
-//                                      same number of additions whatever the
-//                                      bucket sizes (a skewed or constant
-//                                      scalar set stays parallel and balanced)
+//                msm_combine_kernel    the pieces of each crossing bucket added
+//                                      up, one thread or four lanes per bucket
+//                msm_combine_long_kernel  buckets over many segments: a radix-4
+//                                      tree over their pieces (a skewed or
+//                                      constant scalar set stays parallel and
+//                                      balanced)
 //   BR           msm_reduce_level_kernel  the tree of Algorithm 2, one launch
 //                                      per level, all windows at once:
 //                                      W_b = W_2b + W_2b+1 + B_2b+1,
@@ -74,6 +75,15 @@ constexpr int kScanPer = 8;
 constexpr int kScanTile = kScanThreads * kScanPer;
 constexpr int kEcThreads = 128;
 constexpr uint32_t kSignBit = 0x80000000u;
+// A bucket that crosses at most this many segment ends is added up by one
+// thread (or four lanes); longer ones by a tree of radix 4 over their pieces
+// (three additions a level; radix 8 took 154 us instead of the tree's 100 for
+// 1300 pieces of BLS12-381, radix 2 needs twice the launches).
+constexpr uint32_t kShortSpan = 8;
+constexpr uint32_t kSegMask = (1u << 28) - 1u;   // a segment index (span - 1 above it in a crossing item)
+constexpr int kLongLevels = 14;    // 4^14 pieces
+// Tree levels of at most this many nodes per SM take eight lanes per node.
+constexpr uint32_t kQuadNodesPerSm = 128;
 
 // Curves: base-field traits, the scalar modulus r (for the input check),
 // the curve constant b, and the CTAs of 128 threads per SM that the register
@@ -119,10 +129,21 @@ struct EcConst {
 };
 
 struct MsmTotals {
-  uint32_t entries;   // points placed in buckets (digit != 0)
-  uint32_t max_span;  // most segment boundaries one bucket crosses
-  uint32_t pad;
-  uint32_t err;       // MSM_ERR_* bits
+  uint32_t entries;                // points placed in buckets (digit != 0)
+  uint32_t seg_len;                // S, entries per segment (from the entries there are)
+  uint32_t crossing;               // buckets over 2 .. kShortSpan + 1 segments
+  uint32_t items[kLongLevels];     // work items of the levels of the long buckets' trees
+  uint32_t err;                    // MSM_ERR_* bits
+};
+
+// Work lists of the combine kernels, filled by the accumulation: `crossing` the
+// segment in which each short crossing bucket starts; `items` + item_base[l]
+// the segments whose piece is a node of level l of a long bucket's tree (bit
+// 31: the head piece, in the segment where the bucket starts).
+struct CombineLists {
+  uint32_t *crossing;
+  uint32_t *items;
+  uint32_t item_base[kLongLevels];
 };
 
 // ----------------------------------------------------------- small helpers
@@ -271,9 +292,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const uint32_
 }
 
 // Scan pass 2 (one CTA): exclusive scan of the tile sums in place; the total
-// goes to tot->entries and offsets[nb].
+// goes to tot->entries and offsets[nb], and fixes the segment length.
 __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(uint32_t *tile_sums, uint32_t num_tiles,
-                                                                  uint64_t nb, uint32_t *offsets, MsmTotals *tot) {
+                                                                  uint64_t nb, uint32_t *offsets, uint32_t max_segments,
+                                                                  MsmTotals *tot) {
   __shared__ uint32_t chunk_total;
   uint32_t carry = 0;
   for (uint32_t b0 = 0; b0 < num_tiles; b0 += kScanThreads) {
@@ -287,6 +309,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(uint32_t *tile
   }
   if (threadIdx.x == 0) {
     tot->entries = carry;
+    // as many segments as the plan has room for (a whole number of waves),
+    // with at least 8 entries each: sparse scalars make fewer entries
+    tot->seg_len = max(8u, (uint32_t)(((uint64_t)carry + max_segments - 1) / max_segments));
     offsets[nb] = carry;
   }
 }
@@ -370,22 +395,44 @@ __device__ __forceinline__ void emit_piece(const Xyzz<T> &acc, uint32_t b, uint3
   else store_point_xyzz(pieces, 2 * (uint64_t)t + 1, acc);
 }
 
+// The next free index of a list: one atomic for the lanes that are here.
+__device__ __forceinline__ uint32_t list_slot(uint32_t *counter) {
+  const uint32_t mask = __activemask(), lane = threadIdx.x & 31u, leader = __ffs(mask) - 1;
+  uint32_t base = 0;
+  if (lane == leader) base = atomicAdd(counter, (uint32_t)__popc(mask));
+  return __shfl_sync(mask, base, leader) + __popc(mask & ((1u << lane) - 1u));
+}
+
+// Piece i of a bucket over `span` + 1 segments, in segment t: a node of every
+// level l of its tree for which i is a multiple of 4^(l + 1) and i + 4^l <=
+// span.
+__device__ __forceinline__ void push_items(MsmTotals *tot, const CombineLists &lists, uint32_t t, uint32_t i,
+                                           uint32_t span) {
+  if (span <= kShortSpan) return;
+  uint32_t step = 1;
+  for (int l = 0; l < kLongLevels && (i & (4 * step - 1)) == 0 && i + step <= span; ++l, step *= 4)
+    lists.items[lists.item_base[l] + list_slot(&tot->items[l])] = t | (i == 0 ? kSignBit : 0u);
+}
+
 // BA: segment t adds the points of sorted entries [t S, t S + S).
 template <class C>
 __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
     msm_accumulate_kernel(const uint4 *__restrict__ pts_m, const uint32_t *__restrict__ sorted,
-                          const uint32_t *__restrict__ offsets, uint64_t nb, uint32_t S, EcConst<typename C::T> k,
-                          MsmTotals *tot, uint2 *__restrict__ seg_ends, uint4 *bucket_sum, uint4 *pieces) {
+                          const uint32_t *__restrict__ offsets, uint64_t nb, EcConst<typename C::T> k,
+                          MsmTotals *tot, CombineLists lists, uint4 *bucket_sum, uint4 *pieces) {
   using T = typename C::T;
   constexpr int L = T::L;
-  const uint32_t n_entries = tot->entries;
+  const uint32_t n_entries = tot->entries, S = tot->seg_len;
   const uint32_t num_segs = (n_entries + S - 1) / S;
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < num_segs; t += gridDim.x * blockDim.x) {
     const uint32_t e0 = t * S, e1 = min(e0 + S, n_entries);
     uint32_t b = bucket_of_entry(offsets, nb, e0);
-    const uint32_t first = b;
     uint32_t end_b = __ldg(offsets + b + 1);
     bool started_before = __ldg(offsets + b) < e0;
+    if (started_before) {
+      const uint32_t t0 = __ldg(offsets + b) / S;
+      push_items(tot, lists, t, t - t0, (end_b - 1) / S - t0);
+    }
     Xyzz<T> acc;
     xyzz_set_inf(acc);
     for (uint32_t e = e0; e < e1; ++e) {
@@ -415,58 +462,89 @@ __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
     emit_piece(acc, b, t, started_before, continues, bucket_sum, pieces);
     if (continues && !started_before) {
       const uint32_t span = (end_b - 1) / S - t;  // segments after t that hold bucket b
-      atomicMax(&tot->max_span, span);
+      if (span <= kShortSpan) lists.crossing[list_slot(&tot->crossing)] = t | (uint32_t)(span - 1) << 28;
+      else push_items(tot, lists, t, 0, span);
     }
-    seg_ends[t] = make_uint2(first, b);
   }
 }
 
-// BA, combine round r.  The pieces of a bucket that crosses segments
-// t0 < t0+1 < ... < t1 form V[0] = head slot 2 t0 + 1, V[i] = slot 2 (t0 + i);
-// round r adds V[i + 2^r] into V[i] for i a multiple of 2^(r+1), so after
-// ceil(log2(t1 - t0 + 1)) rounds the bucket's sum is in V[0].
+// The pieces of a bucket that crosses the ends of segments t0 < t0 + 1 < ... <
+// t0 + span form V[0] = head slot 2 t0 + 1, V[i] = slot 2 (t0 + i); their sum
+// goes to V[0].  One thread per bucket, or, when there are too few buckets to
+// fill the grid, four lanes (an addition is then 4 products deep, not 14).
 template <class C>
 __global__ void __launch_bounds__(kEcThreads, C::kTreeMinBlocks)
-    msm_combine_kernel(const uint32_t *__restrict__ offsets, const uint2 *__restrict__ seg_ends, uint32_t S,
-                       const MsmTotals *tot, uint32_t r, uint4 *pieces) {
+    msm_combine_kernel(const MsmTotals *tot, const uint32_t *__restrict__ crossing, uint4 *pieces) {
   using T = typename C::T;
-  const uint32_t step = 1u << r;
-  if (step > tot->max_span) return;
-  const uint32_t n_entries = tot->entries;
-  const uint32_t num_segs = (n_entries + S - 1) / S;
-  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < num_segs; t += gridDim.x * blockDim.x) {
-    const uint2 ends = seg_ends[t];
-    const uint32_t e0 = t * S, e1 = min(e0 + S, n_entries);
-    // role of V[0]: the last bucket starts in this segment and continues
-    {
-      const uint32_t b = ends.y;
-      const uint32_t ob = __ldg(offsets + b), ob1 = __ldg(offsets + b + 1);
-      if (ob >= e0 && ob1 > e1) {
-        const uint32_t span = (ob1 - 1) / S - t;
-        if (step <= span) {
-          Xyzz<T> a, q;
-          load_point_xyzz(a, pieces, 2 * (uint64_t)t + 1);
-          load_point_xyzz(q, pieces, 2 * (uint64_t)(t + step));
-          xyzz_add<T, true>(a, q);
-          store_point_xyzz(pieces, 2 * (uint64_t)t + 1, a);
-        }
+  constexpr int L = T::L;
+  const uint32_t count = tot->crossing, threads = gridDim.x * blockDim.x;
+  const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (count <= threads / 4) {
+    for (uint32_t i0 = (id & ~31u) / 4; i0 < count; i0 += threads / 4) {   // uniform in a warp
+      const uint32_t i = i0 + (id & 31u) / 4;
+      const bool live = i < count;
+      const uint32_t item = crossing[live ? i : i0];
+      const uint32_t t = item & kSegMask, span = live ? (item >> 28) + 1 : 0u;
+      const uint32_t most = __reduce_max_sync(0xffffffffu, span);
+      uint32_t v[L], w[L];
+      quad_load<T>(v, pieces, 2 * (uint64_t)t + 1);
+#pragma unroll 1
+      for (uint32_t j = 1; j <= most; ++j) {
+        if (j <= span) quad_load<T>(w, pieces, 2 * (uint64_t)(t + j));
+        else fv_zero<L>(w);   // O
+        quad_add<T>(v, w);
       }
+      if (live) quad_store<T>(pieces, 2 * (uint64_t)t + 1, v);
     }
-    // role of V[i], i >= 1: the first bucket started in an earlier segment
-    {
-      const uint32_t b = ends.x;
-      const uint32_t ob = __ldg(offsets + b), ob1 = __ldg(offsets + b + 1);
-      if (ob < e0) {
-        const uint32_t t0 = ob / S, span = (ob1 - 1) / S - t0, i = t - t0;
-        if ((i & (2 * step - 1)) == 0 && i + step <= span) {
-          Xyzz<T> a, q;
-          load_point_xyzz(a, pieces, 2 * (uint64_t)t);
-          load_point_xyzz(q, pieces, 2 * (uint64_t)(t + step));
-          xyzz_add<T, true>(a, q);
-          store_point_xyzz(pieces, 2 * (uint64_t)t, a);
-        }
-      }
+    return;
+  }
+  for (uint32_t i = id; i < count; i += threads) {
+    const uint32_t item = crossing[i], t = item & kSegMask, span = (item >> 28) + 1;
+    Xyzz<T> a;
+    load_point_xyzz(a, pieces, 2 * (uint64_t)t + 1);
+#pragma unroll 1
+    for (uint32_t j = 1; j <= span; ++j) {
+      Xyzz<T> q;
+      load_point_xyzz(q, pieces, 2 * (uint64_t)(t + j));
+      xyzz_add<T, true>(a, q);
     }
+    store_point_xyzz(pieces, 2 * (uint64_t)t + 1, a);
+  }
+}
+
+// Level l of the long buckets' trees: V[i] += V[i + m 4^l], m = 1..3, for the
+// listed i (multiples of 4^(l + 1)); four lanes per item.
+template <class C>
+__global__ void __launch_bounds__(kEcThreads)
+    msm_combine_long_kernel(const uint32_t *__restrict__ offsets, uint64_t nb, const MsmTotals *tot,
+                            CombineLists lists, int level, uint4 *pieces) {
+  using T = typename C::T;
+  constexpr int L = T::L;
+  const uint32_t count = tot->items[level], threads = gridDim.x * blockDim.x, S = tot->seg_len;
+  const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t *items = lists.items + lists.item_base[level];
+  const uint32_t step = 1u << (2 * level);
+  for (uint32_t i0 = (id & ~31u) / 4; i0 < count; i0 += threads / 4) {   // uniform in a warp
+    const uint32_t i = i0 + (id & 31u) / 4;
+    const bool live = i < count;
+    const uint32_t item = items[live ? i : i0];
+    const uint32_t t = item & ~kSignBit;
+    const uint64_t slot = 2 * (uint64_t)t + (item & kSignBit ? 1u : 0u);
+    // segments of this bucket after t: up to the segment of its last entry
+    const uint32_t e = item & kSignBit ? min((t + 1) * S, tot->entries) - 1 : t * S;
+    const uint32_t b = bucket_of_entry(offsets, nb, e);
+    const uint32_t after = live ? (__ldg(offsets + b + 1) - 1) / S - t : 0u;
+    uint32_t v[L], w[L];
+    quad_load<T>(v, pieces, slot);
+#pragma unroll 1
+    for (uint32_t m = 1; m < 4; ++m) {
+      const bool add = after >= m * step;
+      if (!__any_sync(0xffffffffu, add)) break;
+      if (add) quad_load<T>(w, pieces, 2 * (uint64_t)(t + m * step));
+      else fv_zero<L>(w);
+      quad_add<T>(v, w);
+    }
+    if (live) quad_store<T>(pieces, slot, v);
   }
 }
 
@@ -487,9 +565,10 @@ __device__ __forceinline__ void load_bucket(Xyzz<T> &p, const uint4 *bucket_sum,
 template <class C>
 __global__ void __launch_bounds__(kEcThreads, C::kTreeMinBlocks)
     msm_reduce_level_kernel(uint32_t s, uint32_t lb, uint32_t kb, uint32_t nk, const uint4 *bucket_sum,
-                            const uint4 *pieces, const uint32_t *offsets, uint32_t S, uint4 *heap_w,
+                            const uint4 *pieces, const uint32_t *offsets, const MsmTotals *tot, uint4 *heap_w,
                             uint4 *heap_b) {
   using T = typename C::T;
+  const uint32_t S = tot->seg_len;
   const uint64_t per = 1ull << s, total = per * nk;  // windows kb .. kb + nk - 1
   for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total;
        t += (uint64_t)gridDim.x * blockDim.x) {
@@ -523,33 +602,103 @@ __global__ void __launch_bounds__(kEcThreads, C::kTreeMinBlocks)
   }
 }
 
+// Coordinate `lane` of bucket b's sum (load_bucket, four lanes per point).
+template <class T>
+__device__ __forceinline__ void quad_load_bucket(uint32_t v[T::L], const uint4 *bucket_sum, const uint4 *pieces,
+                                                 const uint32_t *offsets, uint32_t S, uint64_t b) {
+  const uint32_t ob = offsets[b], ob1 = offsets[b + 1];
+  if (ob1 == ob) fv_zero<T::L>(v);
+  else if (ob / S == (ob1 - 1) / S) quad_load<T>(v, bucket_sum, b);
+  else quad_load<T>(v, pieces, 2 * (uint64_t)(ob / S) + 1);
+}
+
+// The same level with eight lanes per node, four for W and four for B: a level
+// with few nodes takes the time of its dependent products, 8 deep this way
+// instead of 51 (BLS12-381: 65 us a level by one thread per node).
+template <class C>
+__global__ void __launch_bounds__(kEcThreads)
+    msm_reduce_level_quad_kernel(uint32_t s, uint32_t lb, uint32_t kb, uint32_t nk, const uint4 *bucket_sum,
+                                 const uint4 *pieces, const uint32_t *offsets, const MsmTotals *tot, uint4 *heap_w,
+                                 uint4 *heap_b) {
+  using T = typename C::T;
+  constexpr int L = T::L;
+  const uint32_t S = tot->seg_len;
+  const uint64_t per = 1ull << s, total = per * nk;
+  const uint64_t group = (uint64_t)gridDim.x * (blockDim.x / 8);
+  const uint64_t first = (uint64_t)blockIdx.x * (blockDim.x / 8) + (threadIdx.x / 8);
+  const bool is_b = (threadIdx.x & 4) != 0;
+  const bool leaves = s + 1 == lb;
+  // every lane of the warp takes part in each step; a node past the end is a
+  // copy of the last one that is not stored
+  for (uint64_t t0 = first - (threadIdx.x % 32) / 8; t0 < total; t0 += group) {
+    const uint64_t t = t0 + (threadIdx.x % 32) / 8;
+    const bool live = t < total;
+    const uint64_t tc = live ? t : total - 1;
+    const uint64_t k = kb + (tc >> s), b = tc & (per - 1);
+    const uint64_t heap0 = k << lb, node = heap0 + per + b;
+    uint32_t v[L], w[L], x[L];
+    if (leaves) {
+      quad_load_bucket<T>(v, bucket_sum, pieces, offsets, S, heap0 + 2 * b);
+      quad_load_bucket<T>(w, bucket_sum, pieces, offsets, S, heap0 + 2 * b + 1);
+      fv_copy<L>(x, w);                  // W = (B_L + B_R) + B_R
+    } else {
+      const uint64_t child = heap0 + 2 * per + 2 * b;
+      quad_load<T>(v, is_b ? heap_b : heap_w, child);
+      quad_load<T>(w, is_b ? heap_b : heap_w, child + 1);
+      quad_load<T>(x, heap_b, child + 1);   // W = W_L + W_R + B_R
+    }
+    quad_add<T>(v, w);
+    uint32_t y[L];
+    fv_copy<L>(y, v);
+    quad_add<T>(y, x);                   // the W lanes' result
+    quad_dbl<T>(v);                      // the B lanes': 2 (B_L + B_R)
+    if (live) {
+      if (!is_b) quad_store<T>(heap_w, node, y);
+      else if (s != 0) quad_store<T>(heap_b, node, v);   // the root's B is not needed
+    }
+  }
+}
+
 // WM: sum_{kb <= k < ke} 2^(k c) W_k by Horner (then kb c doublings), in
 // affine standard form; the whole MSM for [0, K).  With one bucket per
-// window (c = 1) W_k is that bucket.
+// window (c = 1) W_k is that bucket.  A chain of about 255 doublings: one warp
+// with four lanes per point (every group of four does the same).
 template <class C>
 __global__ void msm_merge_kernel(uint32_t c, uint32_t kb, uint32_t ke, const uint4 *heap_w, const uint4 *bucket_sum,
-                                 const uint4 *pieces, const uint32_t *offsets, uint32_t S,
+                                 const uint4 *pieces, const uint32_t *offsets, const MsmTotals *tot,
                                  EcConst<typename C::T> kc, uint4 *result) {
   using T = typename C::T;
   constexpr int L = T::L;
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  const uint32_t lb = c - 1;
-  Xyzz<T> acc;
-  xyzz_set_inf(acc);
+  if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+  const uint32_t lb = c - 1, S = tot->seg_len;
+  uint32_t v[L];
+  fv_zero<L>(v);
+  uint32_t doublings = 0;
   for (int k = (int)ke - 1; k >= (int)kb; --k) {
-    if (!xyzz_is_inf(acc))
-      for (uint32_t j = 0; j < c; ++j) xyzz_dbl(acc, acc);
-    Xyzz<T> w;
-    if (lb == 0) load_bucket(w, bucket_sum, pieces, offsets, S, (uint64_t)k);
-    else load_point_xyzz(w, heap_w, ((uint64_t)k << lb) + 1);
-    xyzz_add(acc, w);
+    uint32_t w[L];
+    if (lb == 0) quad_load_bucket<T>(w, bucket_sum, pieces, offsets, S, (uint64_t)k);
+    else quad_load<T>(w, heap_w, ((uint64_t)k << lb) + 1);
+#pragma unroll 1
+    for (uint32_t j = 0; j < doublings; ++j) quad_dbl<T>(v);
+    quad_add<T>(v, w);
+    doublings = c;
   }
-  if (!xyzz_is_inf(acc))
-    for (uint32_t j = 0; j < c * kb; ++j) xyzz_dbl(acc, acc);
-  uint32_t x[L], y[L];
-  xyzz_to_affine_std<T>(x, y, acc, kc.one);
-  T::store(result, 0, x);
-  T::store(result, 1, y);
+#pragma unroll 1
+  for (uint32_t j = 0; j < c * kb; ++j) quad_dbl<T>(v);
+  // affine: x = X ZZZ / (ZZ ZZZ), y = Y ZZ / (ZZ ZZZ)
+  uint32_t z[L], t[L];
+  quad_get<L>(z, v, 2);
+  quad_get<L>(t, v, 3);
+  const bool inf = fv_is_zero<L>(z);
+  uint32_t inv[L], p[L];
+  f_mul<T, true>(p, z, t);
+  f_inverse<T>(inv, p, kc.r2);           // 0 for O
+  quad_pick<L>(z, (threadIdx.x & 3) == 0, t, z);
+  f_mul<T, true>(z, inv, z);
+  f_mul<T, true>(z, z, v);
+  T::redc(z, z);
+  if (inf) fv_zero<L>(z);
+  if (threadIdx.x < 2) T::store(result, threadIdx.x, z);
 }
 
 // Precomputed bases (fixed points reused across calls): for every point P_i
@@ -613,7 +762,7 @@ __global__ void __launch_bounds__(kEcThreads) msm_bases_kernel(const uint4 *pts,
       T::mul(pre[k], pre[k - 1], z);  // prefix products of z_k = ZZ_k ZZZ_k
     }
     uint32_t inv[L];
-    f_inverse<T>(inv, pre[K - 1], kc.one);  // (z_0 ... z_{K-1})^-1
+    f_inverse<T>(inv, pre[K - 1], kc.r2);  // (z_0 ... z_{K-1})^-1
     for (int k = (int)K - 1; k >= 0; --k) {
       uint32_t ik[L], z[L], zi[L], ax[L], ay[L];
       if (k > 0) {
@@ -674,7 +823,7 @@ __global__ void __launch_bounds__(kEcThreads) fixed_base_affine_kernel(EcConst<t
   } else {
     uint32_t t[L], inv[L], zi[L];
     T::mul(t, p.ZZ, p.ZZZ);
-    f_inverse<T>(inv, t, kc.one);
+    f_inverse<T>(inv, t, kc.r2);
     T::mul(zi, inv, p.ZZZ);
     T::mul(x, p.X, zi);
     T::mul(zi, inv, p.ZZ);
@@ -705,7 +854,7 @@ __global__ void __launch_bounds__(kEcThreads) fixed_base_points_kernel(EcConst<t
       xyzz_madd<T>(acc, x, y, kc.one);
     }
     uint32_t x[L], y[L];
-    xyzz_to_affine_std<T>(x, y, acc, kc.one);
+    xyzz_to_affine_std<T>(x, y, acc, kc.r2);
     T::store(out, 2 * i, x);
     T::store(out, 2 * i + 1, y);
   }
@@ -863,13 +1012,27 @@ uint32_t default_window(uint64_t n, uint32_t scalar_bits) {
   return best;
 }
 
-// Entries per accumulation segment: enough segments to fill the GPU eight
-// times over (512 resident threads per SM), 8..128 additions each.  Longer
-// segments cut the buckets that cross a segment end, hence the combine work.
-uint32_t segment_length(uint64_t max_n, uint32_t K, int sms) {
-  const uint64_t entries = max_n * K;
-  const uint64_t want = (uint64_t)sms * 512 * 8;
-  return (uint32_t)std::max<uint64_t>(8, std::min<uint64_t>(128, entries / want));
+// Entries per accumulation segment: the segments of a full call fill the GPU a
+// whole number of times (1 to 8 times the threads that are resident, so that the
+// last wave is not nearly empty), with 64 additions or more each where there
+// are enough entries: longer segments cut the buckets that cross a segment end,
+// hence the combine work.
+uint32_t segment_length(uint64_t max_n, uint32_t K, int sms, int blocks_per_sm) {
+  const uint64_t entries = max_n * K, resident = (uint64_t)sms * blocks_per_sm * kEcThreads;
+  const uint64_t waves = std::max<uint64_t>(1, std::min<uint64_t>(8, entries / (resident * 64)));
+  return (uint32_t)std::max<uint64_t>(8, std::min<uint64_t>(128, (entries + waves * resident - 1) / (waves * resident)));
+}
+
+// Item list bases: level l of the long trees has at most segments / 4^(l + 1)
+// + one head per bucket; a long bucket covers more than kShortSpan segments.
+uint64_t item_bases(uint64_t segments, uint32_t base[kLongLevels]) {
+  uint64_t total = 0, per = 4;
+  for (int l = 0; l < kLongLevels; ++l) {
+    base[l] = (uint32_t)total;
+    total += segments / per + segments / kShortSpan + 1;
+    per *= 4;
+  }
+  return total;
 }
 
 uint32_t curve_scalar_bits(int curve) { return curve == MSM_CURVE_BLS12_381_G1 ? 255u : 254u; }
@@ -896,7 +1059,7 @@ struct msm_plan_s {
   uint32_t *counts = nullptr, *offsets = nullptr, *cursor = nullptr, *tile_sums = nullptr;
   MsmTotals *tot = nullptr;
   uint32_t *sorted = nullptr;
-  uint2 *seg_ends = nullptr;  // first and last bucket of each segment
+  CombineLists lists{};       // work lists of the combine kernels
   uint4 *bucket_sum = nullptr, *pieces = nullptr;   // nb and 2 max_segments XYZZ points
   uint4 *heap_w = nullptr, *heap_b = nullptr;       // nb XYZZ points each
   uint4 *bases = nullptr;     // precomputed window copies: K x max_n points (msm_plan_set_bases)
@@ -908,7 +1071,7 @@ namespace {
 
 void free_plan(msm_plan p) {
   void *bufs[] = {p->pts_m, p->counts, p->offsets, p->cursor, p->tile_sums, p->tot, p->sorted,
-                  p->seg_ends, p->bucket_sum, p->pieces, p->heap_w, p->heap_b, p->bases};
+                  p->lists.crossing, p->lists.items, p->bucket_sum, p->pieces, p->heap_w, p->heap_b, p->bases};
   for (void *b : bufs)
     if (b) cudaFree(b);
   delete p;
@@ -955,31 +1118,43 @@ ntt_status enqueue_msm(msm_plan p, const uint4 *sc, const uint4 *pt, uint64_t n,
     msm_count_kernel<C><<<grid_for(n, 256, sms, 8), 256, 0, st>>>(sc, n, p->c, kb, ke, flat, p->counts, p->tot);
   }
   scan_reduce_kernel<<<num_tiles, kScanThreads, 0, st>>>(p->counts, nb, p->tile_sums);
-  scan_tiles_kernel<<<1, kScanThreads, 0, st>>>(p->tile_sums, num_tiles, nb, p->offsets, p->tot);
+  scan_tiles_kernel<<<1, kScanThreads, 0, st>>>(p->tile_sums, num_tiles, nb, p->offsets,
+                                                (uint32_t)std::max<uint64_t>(1, p->max_segments - 1), p->tot);
   scan_apply_kernel<<<num_tiles, kScanThreads, 0, st>>>(p->counts, nb, p->tile_sums, p->offsets, p->cursor);
   if (n > 0) {
     msm_scatter_kernel<<<grid_for(n, 256, sms, 8), 256, 0, st>>>(sc, n, p->c, kb, ke,
                                                                  flat ? (uint32_t)p->max_n : 0u, p->cursor,
                                                                  p->sorted);
-    const uint64_t segs = (n * p->K + p->S - 1) / p->S;
+    const uint64_t segs = std::min<uint64_t>((n * p->K + 7) / 8, p->max_segments);
     const int g = grid_for(segs, kEcThreads, sms, C::kMinBlocks);
-    msm_accumulate_kernel<C><<<g, kEcThreads, 0, st>>>(pts, p->sorted, p->offsets, nb, p->S, k, p->tot,
-                                                       p->seg_ends, p->bucket_sum, p->pieces);
-    // a bucket holds at most n entries, so it crosses at most ceil(n / S)
-    // segment boundaries; rounds beyond the measured maximum exit at once
-    const uint64_t max_span = (n + p->S - 1) / p->S;
+    msm_accumulate_kernel<C><<<g, kEcThreads, 0, st>>>(pts, p->sorted, p->offsets, nb, k, p->tot, p->lists,
+                                                       p->bucket_sum, p->pieces);
     const int gt = grid_for(segs, kEcThreads, sms, C::kTreeMinBlocks);
-    for (uint32_t r = 0; (1ull << r) <= max_span; ++r)
-      msm_combine_kernel<C><<<gt, kEcThreads, 0, st>>>(p->offsets, p->seg_ends, p->S, p->tot, r, p->pieces);
+    msm_combine_kernel<C><<<gt, kEcThreads, 0, st>>>(p->tot, p->lists.crossing, p->pieces);
+    // a bucket holds at most n entries of one window (flat: of all of them), so
+    // it crosses at most this many segment ends; empty levels exit at once
+    // (segments of 8 entries at least, at most max_segments of them)
+    const uint64_t most = flat ? n * p->K : n;
+    const uint64_t max_span = std::min<uint64_t>((most + 7) / 8, p->max_segments);
+    uint64_t step = 1;
+    for (int l = 0; l < kLongLevels && max_span > kShortSpan && step <= max_span; ++l, step *= 4)
+      msm_combine_long_kernel<C><<<grid_for(4 * (max_span / (4 * step) + 1) * p->K, kEcThreads, sms, 4), kEcThreads, 0,
+                                   st>>>(p->offsets, nb, p->tot, p->lists, l, p->pieces);
   }
   for (int s = (int)lb - 1; s >= 0 && tree_ke > tree_kb; --s) {
     const uint64_t work = ((uint64_t)(tree_ke - tree_kb)) << s;
+    if (work <= (uint64_t)sms * kQuadNodesPerSm) {
+      msm_reduce_level_quad_kernel<C><<<grid_for(8 * work, kEcThreads, sms, 8), kEcThreads, 0, st>>>(
+          (uint32_t)s, lb, tree_kb, tree_ke - tree_kb, p->bucket_sum, p->pieces, p->offsets, p->tot, p->heap_w,
+          p->heap_b);
+      continue;
+    }
     msm_reduce_level_kernel<C><<<grid_for(work, kEcThreads, sms, C::kTreeMinBlocks), kEcThreads, 0, st>>>(
-        (uint32_t)s, lb, tree_kb, tree_ke - tree_kb, p->bucket_sum, p->pieces, p->offsets, p->S, p->heap_w,
+        (uint32_t)s, lb, tree_kb, tree_ke - tree_kb, p->bucket_sum, p->pieces, p->offsets, p->tot, p->heap_w,
         p->heap_b);
   }
   msm_merge_kernel<C><<<1, 32, 0, st>>>(p->c, tree_kb, tree_ke, p->heap_w, p->bucket_sum, p->pieces, p->offsets,
-                                        p->S, k, result);
+                                        p->tot, k, result);
   return cuda_st(cudaGetLastError());
 }
 
@@ -1057,7 +1232,8 @@ ntt_status msm_plan_create(msm_plan *out, msm_curve curve, uint64_t max_n, uint3
   p->max_n = max_n;
   p->c = c;
   p->K = num_windows(c, sbits);
-  p->S = segment_length(max_n, p->K, sms);
+  p->S = segment_length(max_n, p->K, sms,
+                        p->curve == MSM_CURVE_BLS12_381_G1 ? CurveBls381::kMinBlocks : CurveBn254::kMinBlocks);
   p->nb = (uint64_t)p->K << (c - 1);
   const uint64_t entries = max_n * p->K;
   p->max_segments = (entries + p->S - 1) / p->S + 1;
@@ -1074,7 +1250,8 @@ ntt_status msm_plan_create(msm_plan *out, msm_curve curve, uint64_t max_n, uint3
   if (s == NTT_OK) s = alloc(&p->tile_sums, (uint64_t)p->num_tiles * 4, &tb);
   if (s == NTT_OK) s = alloc(&p->tot, sizeof(MsmTotals), &tb);
   if (s == NTT_OK) s = alloc(&p->sorted, entries * 4, &tb);
-  if (s == NTT_OK) s = alloc(&p->seg_ends, p->max_segments * sizeof(uint2), &tb);
+  if (s == NTT_OK) s = alloc(&p->lists.crossing, p->max_segments * 4, &tb);
+  if (s == NTT_OK) s = alloc(&p->lists.items, item_bases(p->max_segments, p->lists.item_base) * 4, &tb);
   if (s == NTT_OK) s = alloc(&p->bucket_sum, p->nb * xb, &tb);
   if (s == NTT_OK) s = alloc(&p->pieces, 2 * p->max_segments * xb, &tb);
   if (s == NTT_OK) s = alloc(&p->heap_w, p->nb * xb, &tb);
