@@ -2,9 +2,9 @@
 //
 // The paper batches NTTs to keep its matrix units busy (Sec. 4.4, Fig. 7).
 // On GB300 a single small transform leaves most of the 152 SMs idle (a
-// 2^14-point pass has 8 tiles), so a batch is run as one persistent kernel
+// 2^14-point pass has 16 tiles), so a batch is run as one persistent kernel
 // per field: every (job, pass, tile) is an item in one queue ordered by pass
-// level, CTAs (3 per SM) claim items with an atomic counter, and an item of
+// level, CTAs (6 per SM) claim items with an atomic counter, and an item of
 // pass j waits (time-bounded) for the completion counter of pass j-1 of its
 // own job.  The segment table and counters of a job list are built once; the
 // launch sequence (counter reset + kernels) is captured into a CUDA graph and
@@ -52,6 +52,7 @@ struct Part {
   uint32_t *d_ctl = nullptr;  // [0] = head, [1 + s] = done tiles of segment s
   uint32_t num_segs = 0;
   uint32_t total_items = 0;
+  uint32_t tile_log = 10;
 };
 
 // How a job list is run: jobs of 2^split_log points and more (and matrix-path
@@ -171,12 +172,19 @@ namespace gb300ntt {
 
 // Segment table of the jobs of one field: every pass of every job, ordered
 // by pass level (larger jobs first within a level).  Pure host code.
-std::vector<BatchSeg> build_segments(const std::vector<BatchJobRef> &jobs, int field, uint32_t *total_items) {
+std::vector<BatchSeg> build_segments(const std::vector<BatchJobRef> &jobs, int field, uint32_t *total_items,
+                                     uint32_t *tile_log) {
   std::vector<BatchSeg> segs;
   std::vector<std::vector<int>> seg_of(jobs.size());  // [job][pass] -> segment index
   uint32_t max_passes = 0;
-  for (const BatchJobRef &j : jobs)
-    if (j.plan->field == field) max_passes = std::max(max_passes, j.plan->num_passes);
+  uint64_t elements = 0;
+  *tile_log = 10;
+  for (const BatchJobRef &j : jobs) {
+    if (j.plan->field != field) continue;
+    max_passes = std::max(max_passes, j.plan->num_passes);
+    elements += 1ull << j.plan->log_n;
+    *tile_log = std::max(*tile_log, batch_tile_log(j.plan));
+  }
   std::vector<size_t> order;
   for (size_t i = 0; i < jobs.size(); ++i)
     if (jobs[i].plan->field == field) order.push_back(i);
@@ -192,9 +200,12 @@ std::vector<BatchSeg> build_segments(const std::vector<BatchJobRef> &jobs, int f
       int mode = 0;
       build_pass_args(j.plan, j.kind, j.in, j.out, level, &s.a, &mode);
       s.logs = j.plan->pass_log[level];
-      s.mode = (uint32_t)mode;
+      s.mode = (uint16_t)mode;
+      const TileShape shape = batch_shape(elements, s.logs, *tile_log, j.plan->sm_count);
+      s.tl = (uint8_t)shape.tl;
+      s.pl = (uint8_t)shape.pl;
       s.first_item = item;
-      s.num_tiles = (uint32_t)pass_tiles(j.plan->log_n, s.logs, kTileLog);
+      s.num_tiles = (uint32_t)pass_tiles(j.plan->log_n, s.logs, shape.tl);
       if (level > 0) {
         s.dep_seg = seg_of[i][level - 1];
         s.dep_tiles = segs[s.dep_seg].num_tiles;
@@ -235,7 +246,7 @@ ntt_status build_part(const std::vector<JobKey> &jobs, const Policy &pol, int fi
   for (const JobKey &j : jobs)
     if (!runs_alone(j, pol)) refs.push_back(BatchJobRef{j.plan, j.kind, j.in, j.out});
   uint32_t item = 0;
-  std::vector<BatchSeg> segs = build_segments(refs, field, &item);
+  std::vector<BatchSeg> segs = build_segments(refs, field, &item, &part->tile_log);
   if (segs.empty()) return NTT_OK;
   if (g_stall) {
     // test hook: the last segment waits for one tile more than exists
@@ -303,7 +314,8 @@ ntt_status build_entry(Entry &e, int sm_count) {
       b.done = part.d_ctl + 1;
       b.err = err;
       b.wait_ns = g_wait_ns;
-      b.grid = (uint32_t)(sm_count * kPassCtasPerSm);
+      b.tile_log = part.tile_log;
+      b.sm_count = sm_count;
       launchers(part.field).batch(b, cs);
     }
     // join

@@ -40,12 +40,16 @@ struct StaticScratch {
 // kStaticMaxSegs), ordered by pass level, larger jobs first within a level.
 // Fixed-size arrays only.
 ntt_status static_segments(const ntt_job *jobs, size_t n, int field, BatchSeg *out, uint32_t *count,
-                           uint32_t *total_items) {
+                           uint32_t *total_items, uint32_t *tile_log) {
   uint32_t order[kStaticMaxJobs];
   int seg_of[kStaticMaxJobs][kMaxPasses];  // [job][pass] -> segment index
   uint32_t m = 0, max_passes = 0;
+  uint64_t elements = 0;
+  *tile_log = 10;
   for (size_t i = 0; i < n; ++i) {
     if (jobs[i].plan->field != field) continue;
+    elements += 1ull << jobs[i].plan->log_n;
+    *tile_log = std::max(*tile_log, batch_tile_log(jobs[i].plan));
     order[m++] = (uint32_t)i;
     max_passes = std::max(max_passes, jobs[i].plan->num_passes);
   }
@@ -62,9 +66,12 @@ ntt_status static_segments(const ntt_job *jobs, size_t n, int field, BatchSeg *o
       int mode = 0;
       build_pass_args(j.plan, j.kind, j.in, j.out, level, &s.a, &mode);
       s.logs = j.plan->pass_log[level];
-      s.mode = (uint32_t)mode;
+      s.mode = (uint16_t)mode;
+      const TileShape shape = batch_shape(elements, s.logs, *tile_log, j.plan->sm_count);
+      s.tl = (uint8_t)shape.tl;
+      s.pl = (uint8_t)shape.pl;
       s.first_item = item;
-      s.num_tiles = (uint32_t)pass_tiles(j.plan->log_n, s.logs, kTileLog);
+      s.num_tiles = (uint32_t)pass_tiles(j.plan->log_n, s.logs, shape.tl);
       s.dep_seg = level > 0 ? seg_of[i][level - 1] : -1;
       s.dep_tiles = level > 0 ? out[s.dep_seg].num_tiles : 0;
       seg_of[i][level] = (int)segs;
@@ -169,8 +176,8 @@ extern "C" ntt_status ntt_batch_submit_static(const ntt_job *jobs, size_t n, uin
   if (n == 0) return NTT_OK;
   BatchSeg host_segs[kStaticMaxSegs];
   for (int field = 0; field < 2; ++field) {
-    uint32_t count = 0, total = 0;
-    st = static_segments(jobs, n, field, host_segs, &count, &total);
+    uint32_t count = 0, total = 0, tile_log = 10;
+    st = static_segments(jobs, n, field, host_segs, &count, &total, &tile_log);
     if (st != NTT_OK) return st;
     if (count == 0) continue;
     // from pageable stack memory: the call returns once the bytes are staged
@@ -187,7 +194,8 @@ extern "C" ntt_status ntt_batch_submit_static(const ntt_job *jobs, size_t n, uin
     b.done = scratch->ctl[field] + 1;
     b.err = err;
     b.wait_ns = batch_wait_limit_ns();
-    b.grid = (uint32_t)(jobs[0].plan->sm_count * kPassCtasPerSm);
+    b.tile_log = tile_log;
+    b.sm_count = jobs[0].plan->sm_count;
     if (launchers(field).batch(b, s) != cudaSuccess) return NTT_ERR_CUDA;
   }
   return NTT_OK;

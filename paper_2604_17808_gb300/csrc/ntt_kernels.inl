@@ -12,12 +12,14 @@
 #include "../../include/ntt_gb300.h"
 #include "ntt_launch.h"
 
+#include <algorithm>
+
 namespace gb300ntt {
 namespace NTT_NS {
 
 // launchers defined by the other parts of this field
 cudaError_t prepare_pass();
-cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st);
+cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, int sms, cudaStream_t st);
 cudaError_t prepare_batch();
 cudaError_t batch(const BatchLaunch &b, cudaStream_t st);
 cudaError_t prepare_matrix();
@@ -71,18 +73,28 @@ namespace {
 template <int MODE>
 cudaError_t set_pass_attr() {
   cudaError_t e = cudaFuncSetAttribute(ntt_pass_kernel<F, MODE, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       128 * 8 * 32);
+                                       kGroupBytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(ntt_pass_kernel<F, MODE, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 256 * 8 * 32);
+    e = cudaFuncSetAttribute(ntt_pass_kernel<F, MODE, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             2 * kGroupBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(ntt_pass_kernel<F, MODE, 896>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kGroups * kGroupBytes);
   return e;
 }
 
 template <int MODE>
-cudaError_t pass_mode(const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  const dim3 grid((unsigned)tiles), block(1u << (s.tl - s.pl));
+cudaError_t pass_mode(const TileShape &s, const PassArgs &a, uint64_t tiles, int sms, cudaStream_t st) {
+  const uint32_t threads = 1u << (s.tl - s.pl);
   const int smem = 32 << s.tl;
-  if (block.x <= 128) return launch_pdl(ntt_pass_kernel<F, MODE, 128>, grid, block, smem, st, a, s);
-  return launch_pdl(ntt_pass_kernel<F, MODE, 256>, grid, block, smem, st, a, s);
+  const uint32_t n = (uint32_t)tiles;
+  // seven tiles per CTA where that makes the pass one wave that six do not
+  constexpr uint64_t kResident = TileBounds<128>::kMinBlocks;
+  if (s.tl == 10 && s.pl == 3 && tiles > kResident * sms && tiles <= (uint64_t)kGroups * sms)
+    return launch_pdl(ntt_pass_kernel<F, MODE, 896>, (n + kGroups - 1) / kGroups, kGroups * kGroupThreads,
+                      kGroups * kGroupBytes, st, a, s, n);
+  if (threads <= 128) return launch_pdl(ntt_pass_kernel<F, MODE, 128>, n, threads, smem, st, a, s, n);
+  return launch_pdl(ntt_pass_kernel<F, MODE, 256>, n, threads, smem, st, a, s, n);
 }
 
 }  // namespace
@@ -94,13 +106,13 @@ cudaError_t prepare_pass() {
   return e;
 }
 
-cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
+cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, int sms, cudaStream_t st) {
   if (s.pl < 1 || s.pl > 3 || s.tl > 11 || s.logs < 1 || s.logs > s.tl || s.tl - s.pl > 8)
     return cudaErrorInvalidValue;
   switch (mode) {
-    case kModeInner: return pass_mode<kModeInner>(s, a, tiles, st);
-    case kModeFirst: return pass_mode<kModeFirst>(s, a, tiles, st);
-    case kModeFirstPre: return pass_mode<kModeFirstPre>(s, a, tiles, st);
+    case kModeInner: return pass_mode<kModeInner>(s, a, tiles, sms, st);
+    case kModeFirst: return pass_mode<kModeFirst>(s, a, tiles, sms, st);
+    case kModeFirstPre: return pass_mode<kModeFirstPre>(s, a, tiles, sms, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -109,17 +121,18 @@ cudaError_t pass(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles
 
 namespace {
 
-// One tile of one segment (a non-inlined function per mode).
-template <int MODE>
-__device__ __noinline__ void batch_tile_fn(const BatchSeg &sg, uint64_t tile, uint4 *smem) {
-  pass_tile<F, MODE>(sg.a, TileShape{sg.logs, (uint32_t)kTileLog, 3u}, tile, smem);
+// One tile of one segment (a non-inlined function per mode and instance).
+template <int MODE, int MAXT>
+__device__ __noinline__ void batch_tile_fn(const BatchSeg &sg, uint64_t tile, uint32_t smem) {
+  pass_tile<Elem256<F>, MODE, false>(sg.a, TileShape{sg.logs, sg.tl, sg.pl}, tile, smem, threadIdx.x, 0);
 }
 
-__device__ __forceinline__ void batch_tile(const BatchSeg &sg, uint64_t tile, uint4 *smem) {
+template <int MAXT>
+__device__ __forceinline__ void batch_tile(const BatchSeg &sg, uint64_t tile, uint32_t smem) {
   switch (sg.mode) {
-    case kModeInner: batch_tile_fn<kModeInner>(sg, tile, smem); break;
-    case kModeFirst: batch_tile_fn<kModeFirst>(sg, tile, smem); break;
-    default: batch_tile_fn<kModeFirstPre>(sg, tile, smem); break;
+    case kModeInner: batch_tile_fn<kModeInner, MAXT>(sg, tile, smem); break;
+    case kModeFirst: batch_tile_fn<kModeFirst, MAXT>(sg, tile, smem); break;
+    default: batch_tile_fn<kModeFirstPre, MAXT>(sg, tile, smem); break;
   }
 }
 
@@ -130,17 +143,22 @@ __device__ __forceinline__ void batch_tile(const BatchSeg &sg, uint64_t tile, ui
 // is bounded by b.wait_ns (globaltimer); on timeout the CTA records
 // NTT_ERR_TIMEOUT in *b.err and returns, and every CTA stops claiming
 // items once *b.err is set.
-__global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) batch_kernel(const BatchLaunch b) {
+//
+// Two instances, as for the pass kernels: 128 threads and tiles of up to 1024
+// elements, 6 CTAs per SM, and 256 threads and 2048 elements, 3 CTAs per SM, for
+// lists with a 2^11-point pass.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, TileBounds<MAXT>::kMinBlocks) batch_kernel(const BatchLaunch b) {
   extern __shared__ uint4 smem[];
   __shared__ uint32_t s_item;
   __shared__ int32_t s_seg;
-  __shared__ int s_abort;
+  const uint32_t t = threadIdx.x;
+  const uint32_t tile_smem = (uint32_t)__cvta_generic_to_shared(smem);
   for (;;) {
-    if (threadIdx.x == 0) {
+    if (t == 0) {
       uint32_t item = atomicAdd(b.head, 1u);
       if (*(volatile uint32_t *)b.err != 0) item = b.total_items;
       int32_t seg = -1;
-      int abort = 0;
       if (item < b.total_items) {
         int lo = 0, hi = (int)b.num_segs - 1;
         while (lo < hi) {
@@ -156,7 +174,7 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) batch_kernel(con
           while (ld_acquire_gpu(b.done + dep) < need) {
             if (global_ns() - t0 > b.wait_ns) {
               atomicCAS(b.err, 0u, (uint32_t)NTT_ERR_TIMEOUT);
-              abort = 1;
+              item = b.total_items;   // stop
               break;
             }
             __nanosleep(128);
@@ -165,16 +183,17 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) batch_kernel(con
       }
       s_item = item;
       s_seg = seg;
-      s_abort = abort;
     }
     __syncthreads();
-    if (s_item >= b.total_items || s_abort) return;
-    const BatchSeg &sg = b.segs[s_seg];
-    batch_tile(sg, s_item - sg.first_item, smem);
+    const uint32_t item = s_item;
+    if (item >= b.total_items) return;
+    const int32_t seg = s_seg;
+    const BatchSeg &sg = b.segs[seg];
+    batch_tile<MAXT>(sg, item - sg.first_item, tile_smem);
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (t == 0) {
       __threadfence();
-      atomicAdd(b.done + s_seg, 1u);
+      atomicAdd(b.done + seg, 1u);
     }
   }
 }
@@ -182,13 +201,18 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) batch_kernel(con
 }  // namespace
 
 cudaError_t batch(const BatchLaunch &b, cudaStream_t st) {
-  batch_kernel<<<b.grid, kPassThreads, kTileBytes, st>>>(b);
+  if (b.tile_log <= 10)
+    batch_kernel<128><<<b.sm_count * TileBounds<128>::kMinBlocks, 128, kGroupBytes, st>>>(b);
+  else
+    batch_kernel<256><<<b.sm_count * TileBounds<256>::kMinBlocks, 256, 2 * kGroupBytes, st>>>(b);
   return cudaGetLastError();
 }
 
-
 cudaError_t prepare_batch() {
-  return cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes);
+  cudaError_t e = cudaFuncSetAttribute(batch_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(batch_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kGroupBytes);
+  return e;
 }
 
 #elif defined(NTT_PART_MATRIX)

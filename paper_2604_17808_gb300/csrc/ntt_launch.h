@@ -31,7 +31,8 @@ struct Pow2Table {
 struct BatchSeg {
   PassArgs a;
   uint32_t logs;        // log2 of the pass's sub-transform size
-  uint32_t mode;        // PassMode
+  uint16_t mode;        // PassMode
+  uint8_t tl, pl;       // tile of 2^tl elements, 2^pl per thread
   uint32_t first_item;  // index of the segment's first tile in the item space
   uint32_t num_tiles;
   int32_t dep_seg;      // segment that must be complete first, or -1
@@ -54,13 +55,14 @@ struct BatchLaunch {
   uint32_t *done;         // device: completed tiles per segment (zeroed)
   uint32_t *err;          // device: first error code (NTT_ERR_TIMEOUT)
   uint64_t wait_ns;       // bound of every dependency wait
-  uint32_t grid;          // CTAs (a multiple of the SM count)
+  uint32_t tile_log;      // largest tile of the segments: 10 (CTAs of 128 threads) or 11 (256)
+  int sm_count;
 };
 
 struct FieldLaunchers {
   cudaError_t (*prepare)();
-  // one pass over `tiles` tiles of the given shape
-  cudaError_t (*pass)(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, cudaStream_t st);
+  // one pass over `tiles` tiles of the given shape on a device of `sms` SMs
+  cudaError_t (*pass)(int mode, const TileShape &s, const PassArgs &a, uint64_t tiles, int sms, cudaStream_t st);
   // out[n * Mp + q] = init * fac[n] * base^(n*q)    (fac may be null)
   cudaError_t (*gen_2d)(uint4 *out, uint32_t log_s, uint32_t log_mp, const Pow2Table &pw, const uint4 *fac,
                         Fe32 init, cudaStream_t st);

@@ -20,7 +20,7 @@
 // After the last pass the buffer holds X in natural order.  Coset and
 // inverse scale factors are folded into the same per-element multipliers.
 //
-// Work split on the GPU: one CTA owns a tile of 2^tl elements in shared memory
+// Work split on the GPU: a group of threads owns a tile of 2^tl elements in shared memory
 // = 2^(tl - logs) sub-transforms with consecutive sub-transform index, and
 // each thread 2^pl of its elements at a time.  The DIF (Gentleman-Sande)
 // radix-2 network over every sub-transform of the tile runs in rounds of up to
@@ -62,19 +62,35 @@ struct TileShape {
   uint32_t logs, tl, pl;
 };
 
-// Launch bounds of the two kernel instances: up to 128 threads with 7 CTAs per
-// SM (1024-element tiles of 32 KiB with 8 elements per thread: 7168 resident
-// elements per SM, so a 2^20-point pass is one wave of 152 SMs), and 256
-// threads with 3 CTAs per SM (2048-element tiles).
+// A CTA runs one tile, or several independent ones side by side: `groups` of
+// 2^(tl - pl) threads, each with a tile of its own and a named barrier.  Three
+// kernel instances:
+//   up to 128 threads  one tile per CTA, 6 CTAs per SM for 1024-element tiles
+//                      (32 KiB and another KiB that each CTA reserves);
+//   896 threads        seven 1024-element tiles with 8 elements per thread,
+//                      one CTA per SM, for passes that are one wave this way:
+//                      the 1024 tiles of a 2^20-point pass took two waves of
+//                      six (99 and 80 us a pass against 90 and 75).  With many
+//                      waves the CTAs that come and go on their own are faster
+//                      (2^24: 2.9 against 3.1 ms);
+//   256 threads        one 2048-element tile, 3 CTAs per SM.
+constexpr uint32_t kGroups = 7;
+constexpr uint32_t kGroupThreads = 128;
+constexpr uint32_t kGroupBytes = 32u << 10;   // a 1024-element tile
+
 template <int MAXT>
 struct TileBounds {
-  static constexpr int kMinBlocks = MAXT == 256 ? 3 : 7;
+  static constexpr int kMinBlocks = MAXT == 896 ? 1 : MAXT == 256 ? 3 : 6;
 };
 
-constexpr int kPassThreads = 256;                  // batched kernel (tl = 11, pl = 3)
-constexpr int kPassCtasPerSm = 3;
-constexpr int kTileLog = 11;
-constexpr int kTileBytes = 32 << kTileLog;
+// Barrier of one group of `threads` threads; of the CTA where it has one group
+// only (a barrier number in a register would claim all sixteen for the CTA).
+template <bool GROUPED>
+__device__ __forceinline__ void group_sync(uint32_t group, uint32_t threads) {
+  if constexpr (GROUPED) asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(threads) : "memory");
+  else __syncthreads();
+}
+
 constexpr int kMaxPassLog = 11;                    // sub-transforms up to 2048 points
 
 enum PassMode : int {
@@ -118,11 +134,6 @@ __device__ __forceinline__ bool dbg_in(const PassArgs &a, uint64_t idx, uint64_t
 __device__ __forceinline__ constexpr bool dbg_in(const PassArgs &, uint64_t, uint64_t) { return true; }
 #endif
 
-__device__ __forceinline__ void fe_zero(uint32_t r[8]) {
-#pragma unroll
-  for (int j = 0; j < 8; ++j) r[j] = 0;
-}
-
 // Output row of pass 0 for untransformed digits d (their significance reversed).
 __device__ __forceinline__ uint64_t reverse_digits(const PassArgs &a, uint64_t d) {
   uint64_t rest = d, rev = 0;
@@ -157,52 +168,83 @@ __device__ __forceinline__ uint32_t swz(uint32_t e) {
   return ((kSwzLut0 >> (3 * x0)) ^ (kSwzLut1 >> (3 * x1)) ^ (kSwzLut2 >> (3 * x2))) & 7u;
 }
 
-// Byte offset in the tile of the low half of element e; the high half is at
-// the offset ^ 16.
-__device__ __forceinline__ uint32_t tile_offset(uint32_t e) { return ((e << 1) ^ swz(e)) << 4; }
+// What the tile routine asks of a field's elements (this one: 256-bit fields,
+// eight words): their place in the tile, moves, and arithmetic on values in
+// [0, 2p).  `tile` is the tile's shared-memory address, `off` a byte offset that
+// is linear over GF(2) in the bits of the element index; the accesses keep their
+// program order (a thread reads back what it wrote).
+template <class F>
+struct Elem256 {
+  static constexpr int W = 8;
+  static constexpr bool kPreByPosition = false;   // pass-0 multipliers are indexed by n_0
 
-// `tile`: shared-memory address of the tile.  (The accesses keep their program
-// order: no address is formed twice, and a thread reads back what it wrote.)
-__device__ __forceinline__ void tile_store(uint32_t tile, uint32_t off, const uint32_t a[8]) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + off), "r"(a[0]), "r"(a[1]), "r"(a[2]),
-               "r"(a[3])
-               : "memory");
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + (off ^ 16u)), "r"(a[4]), "r"(a[5]), "r"(a[6]),
-               "r"(a[7])
-               : "memory");
-}
+  // low half of element e; the high half is at the offset ^ 16
+  __device__ static __forceinline__ uint32_t tile_offset(uint32_t e) { return ((e << 1) ^ swz(e)) << 4; }
 
-__device__ __forceinline__ void tile_load(uint32_t r[8], uint32_t tile, uint32_t off) {
-  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(tile + off)
-               : "memory");
-  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(tile + (off ^ 16u))
-               : "memory");
-}
+  __device__ static __forceinline__ void tile_store(uint32_t tile, uint32_t off, uint32_t, const uint32_t a[8]) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + off), "r"(a[0]), "r"(a[1]), "r"(a[2]),
+                 "r"(a[3])
+                 : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + (off ^ 16u)), "r"(a[4]), "r"(a[5]),
+                 "r"(a[6]), "r"(a[7])
+                 : "memory");
+  }
 
-// Global -> shared copy of one element without registers, through L2 (data
-// that another CTA wrote earlier in the same launch is read coherently).
-__device__ __forceinline__ void tile_copy_async(uint32_t tile, uint32_t off, const uint4 *base, uint64_t elem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tile + off), "l"(base + 2 * elem) : "memory");
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tile + (off ^ 16u)), "l"(base + 2 * elem + 1)
-               : "memory");
-}
+  __device__ static __forceinline__ void tile_load(uint32_t r[8], uint32_t tile, uint32_t off, uint32_t) {
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(tile + off)
+                 : "memory");
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(tile + (off ^ 16u))
+                 : "memory");
+  }
+
+  // Global -> shared copy of one element without registers, through L2 (data
+  // that another CTA wrote earlier in the same launch is read coherently).
+  __device__ static __forceinline__ void copy_async(uint32_t tile, uint32_t off, uint32_t, const uint4 *base,
+                                                    uint64_t elem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tile + off), "l"(base + 2 * elem) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tile + (off ^ 16u)), "l"(base + 2 * elem + 1)
+                 : "memory");
+  }
+
+  // entry w of the DFT table: the residues of mul_split
+  __device__ static __forceinline__ void load_twiddle(uint32_t A[8], uint32_t B[8], const uint4 *dft_tw, uint32_t w) {
+    const char *p = reinterpret_cast<const char *>(dft_tw) + (w << 6);
+    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(A[0]), "=r"(A[1]), "=r"(A[2]), "=r"(A[3]), "=r"(A[4]), "=r"(A[5]), "=r"(A[6]), "=r"(A[7])
+        : "l"(p));
+    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8+32];"
+        : "=r"(B[0]), "=r"(B[1]), "=r"(B[2]), "=r"(B[3]), "=r"(B[4]), "=r"(B[5]), "=r"(B[6]), "=r"(B[7])
+        : "l"(p));
+  }
+  __device__ static __forceinline__ void load(uint32_t r[8], const uint4 *base, uint64_t e) {
+    fe_load_global(r, base, e);
+  }
+  __device__ static __forceinline__ void store(uint4 *base, uint64_t e, const uint32_t a[8]) {
+    fe_store_global(base, e, a);
+  }
+
+  __device__ static __forceinline__ void add(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
+    add_lazy<F>(r, a, b);
+  }
+  __device__ static __forceinline__ void sub(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
+    sub_lazy<F>(r, a, b);
+  }
+  __device__ static __forceinline__ void mul_twiddle(uint32_t r[8], const uint32_t x[8], const uint32_t A[8],
+                                                     const uint32_t B[8]) {
+    mul_split<F>(r, x, A, B);
+  }
+  // w: a table entry in Montgomery form; below 2p
+  __device__ static __forceinline__ void mul_in(uint32_t x[8], const uint32_t w[8]) { mont_mul_lazy<F>(x, w, x); }
+  // canonical results
+  __device__ static __forceinline__ void mul_out(uint32_t x[8], const uint32_t w[8]) { mont_mul<F>(x, w, x); }
+  __device__ static __forceinline__ void finish(uint32_t x[8]) { reduce_once<F>(x, x); }
+};
 
 __device__ __forceinline__ void tile_copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Twiddle entry w of the DFT table (mul_split's residues).
-__device__ __forceinline__ void load_twiddle(uint32_t A[8], uint32_t B[8], const uint4 *dft_tw, uint32_t w) {
-  const char *p = reinterpret_cast<const char *>(dft_tw) + (w << 6);
-  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=r"(A[0]), "=r"(A[1]), "=r"(A[2]), "=r"(A[3]), "=r"(A[4]), "=r"(A[5]), "=r"(A[6]), "=r"(A[7])
-      : "l"(p));
-  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8+32];"
-      : "=r"(B[0]), "=r"(B[1]), "=r"(B[2]), "=r"(B[3]), "=r"(B[4]), "=r"(B[5]), "=r"(B[6]), "=r"(B[7])
-      : "l"(p));
-}
 
 // ----------------------------------------------------------- butterflies
 
@@ -219,20 +261,21 @@ __device__ __forceinline__ uint32_t private_offset(const Private &v, uint32_t j)
 
 // Private bits: the r round bits T .. T + r - 1 and, when r < pl, the top pl -
 // r bits of the tile index.
+template <class El>
 __device__ __forceinline__ Private private_set(const TileShape &s, uint32_t e, uint32_t T, uint32_t r) {
   const uint32_t top = s.tl - s.pl;   // private bit k >= r is index bit top + k
   Private v;
-  v.base = tile_offset(e);
-  v.d0 = tile_offset(1u << (r > 0 ? T : top));
-  v.d1 = tile_offset(1u << (r > 1 ? T + 1 : top + 1));
-  v.d2 = tile_offset(1u << (r > 2 ? T + 2 : top + 2));
+  v.base = El::tile_offset(e);
+  v.d0 = El::tile_offset(1u << (r > 0 ? T : top));
+  v.d1 = El::tile_offset(1u << (r > 1 ? T + 1 : top + 1));
+  v.d2 = El::tile_offset(1u << (r > 2 ? T + 2 : top + 2));
   return v;
 }
 
 // Private stages T + hi - 1 down to T + lo: pairs that differ in private bit
 // b, twiddle omega_S^((p mod h) S / 2h) with h = 2^(T + b), p the position in
 // the sub-transform; low = its bits below T.
-template <class F>
+template <class El>
 __device__ __forceinline__ void private_stages(uint32_t tile, const uint4 *dft_tw, const TileShape &s, const Private &v,
                                                uint32_t T, int hi, int lo, uint32_t low) {
 #pragma unroll 1
@@ -244,42 +287,42 @@ __device__ __forceinline__ void private_stages(uint32_t tile, const uint4 *dft_t
       const uint32_t j = (i & mask) | ((i & ~mask) << 1);
       const uint32_t c = private_offset(v, j);
       const uint32_t w = (low | ((j & mask) << T)) << sh;
-      uint32_t x[8], y[8], d[8];
+      uint32_t x[El::W], y[El::W], d[El::W];
       if (T == 0 && (j & mask) == 0) {   // twiddle 1, for every thread
-        tile_load(x, tile, c);
-        tile_load(y, tile, c ^ db);
-        sub_lazy<F>(d, x, y);
-        add_lazy<F>(x, x, y);
-        tile_store(tile, c, x);
-        tile_store(tile, c ^ db, d);
+        El::tile_load(x, tile, c, s.tl);
+        El::tile_load(y, tile, c ^ db, s.tl);
+        El::sub(d, x, y);
+        El::add(x, x, y);
+        El::tile_store(tile, c, s.tl, x);
+        El::tile_store(tile, c ^ db, s.tl, d);
         continue;
       }
-      uint32_t A[8], B[8];
-      load_twiddle(A, B, dft_tw, w);
-      tile_load(x, tile, c);
-      tile_load(y, tile, c ^ db);
-      sub_lazy<F>(d, x, y);
-      add_lazy<F>(x, x, y);
-      tile_store(tile, c, x);
-      mul_split<F>(d, d, A, B);
-      tile_store(tile, c ^ db, d);
+      uint32_t A[El::W], B[El::W];
+      El::load_twiddle(A, B, dft_tw, w);
+      El::tile_load(x, tile, c, s.tl);
+      El::tile_load(y, tile, c ^ db, s.tl);
+      El::sub(d, x, y);
+      El::add(x, x, y);
+      El::tile_store(tile, c, s.tl, x);
+      El::mul_twiddle(d, d, A, B);
+      El::tile_store(tile, c ^ db, s.tl, d);
     }
   }
 }
 
 // One output element: canonical, times the output multiplier where there is
 // one.
-template <class F>
-__device__ __forceinline__ void store_output(const PassArgs &a, uint64_t pos, uint32_t x[8]) {
+template <class El>
+__device__ __forceinline__ void store_output(const PassArgs &a, uint64_t pos, uint32_t x[El::W]) {
   if (!dbg_in(a, pos, a.n_vec)) return;
   if (a.post) {   // uniform across the grid
-    uint32_t w[8];
-    fe_load_global(w, a.post, pos);
-    mont_mul<F>(x, w, x);
+    uint32_t w[El::W];
+    El::load(w, a.post, pos);
+    El::mul_out(x, w);
   } else {
-    reduce_once<F>(x, x);
+    El::finish(x);
   }
-  fe_store_global(a.dst, pos, x);
+  El::store(a.dst, pos, x);
 }
 
 // Global position of element n of sub-transform d (pass input; the in-place
@@ -294,12 +337,13 @@ __device__ __forceinline__ uint64_t elem_pos(const PassArgs &a, uint32_t logs, u
   }
 }
 
-// Process tile `tile` of one pass.  All threads of the CTA call this; the
-// caller separates two tiles on the same shared memory with a barrier.
-template <class F, int MODE>
-__device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, uint64_t tile, uint4 *smem_tile) {
-  const uint32_t smem = (uint32_t)__cvta_generic_to_shared(smem_tile);
-  const uint32_t t = threadIdx.x, logs = s.logs, pl = s.pl;
+// Process tile `tile` of one pass.  All threads of the group call this (t: index
+// in the group); the caller separates two tiles on the same shared memory with a
+// barrier.
+template <class El, int MODE, bool GROUPED>
+__device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, uint64_t tile, uint32_t smem,
+                                          uint32_t t, uint32_t group) {
+  const uint32_t logs = s.logs, pl = s.pl, threads = 1u << (s.tl - pl);
   const uint32_t logg = s.tl - logs;                 // log2 of the tile's sub-transforms
   const uint64_t d0 = tile << logg;
   const uint32_t last = min(pl, logs);               // stages of the last round
@@ -312,7 +356,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     T -= r;
     const uint32_t gbits = logg - (pl - r);
     const uint32_t dl = t & ((1u << gbits) - 1u), low = t >> gbits;
-    const Private v = private_set(s, (dl << logs) | low, T, r);
+    const Private v = private_set<El>(s, (dl << logs) | low, T, r);
     const uint32_t count = 1u << pl, rmask = (1u << r) - 1u;
     // element j is input low + ((j mod 2^r) << T) of sub-transform d; with r =
     // pl (all but sub-transforms of 2 and 4 points) its position is linear in j
@@ -327,27 +371,31 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
       if (d >= a.num_sub) continue;
       const uint32_t c = private_offset(v, j);
       if (dbg_in(a, pos, a.n_vec)) {
-        tile_copy_async(smem, c, a.src, pos);
+        El::copy_async(smem, c, s.tl, a.src, pos);
       } else {
-        uint32_t z[8];
-        fe_zero(z);
-        tile_store(smem, c, z);
+        uint32_t z[El::W] = {};
+        El::tile_store(smem, c, s.tl, z);
       }
     }
     if constexpr (MODE != kModeFirst) {
       // the multiplier of the next element is on its way during a product
       const uint64_t q_mask = (1ull << a.log_mp) - 1;
       auto mul_of = [&](uint64_t d, uint32_t n) {
-        return MODE == kModeInner ? ((uint64_t)n << a.log_mp) + (d & q_mask) : (uint64_t)n;
+        if constexpr (MODE == kModeInner) return ((uint64_t)n << a.log_mp) + (d & q_mask);
+        else return El::kPreByPosition ? elem_pos<MODE>(a, logs, d, n) : (uint64_t)n;
       };
-      const uint64_t wstep = MODE == kModeInner ? step : 1ull << T;
+      const uint64_t wstep = MODE == kModeInner || El::kPreByPosition ? step : 1ull << T;
       uint64_t wi = mul_of(dfirst, low);
-      uint32_t w[8], next[8];
-      auto load_mul = [&](uint32_t x[8], uint32_t j) {
+      uint32_t w[El::W], next[El::W];
+      auto load_mul = [&](uint32_t *x, uint32_t j) {
         const uint64_t d = linear ? dfirst : sub_of(j);
         if (!linear) wi = mul_of(d, low | ((j & rmask) << T));
-        if (d < a.num_sub && dbg_in(a, wi, a.n_mul)) fe_load_global(x, a.mul, wi);
-        else fe_zero(x);
+        if (d < a.num_sub && dbg_in(a, wi, a.n_mul)) {
+          El::load(x, a.mul, wi);
+        } else {
+#pragma unroll
+          for (int k = 0; k < El::W; ++k) x[k] = 0;
+        }
         wi += wstep;
       };
       load_mul(next, 0);
@@ -355,17 +403,18 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
 #pragma unroll 1
       for (uint32_t j = 0; j < count; ++j) {
         const uint32_t c = private_offset(v, j);
-        fe_copy(w, next);
+#pragma unroll
+        for (int k = 0; k < El::W; ++k) w[k] = next[k];
         if (j + 1 < count) load_mul(next, j + 1);
-        uint32_t x[8];
-        tile_load(x, smem, c);
-        mont_mul_lazy<F>(x, w, x);
-        tile_store(smem, c, x);
+        uint32_t x[El::W];
+        El::tile_load(x, smem, c, s.tl);
+        El::mul_in(x, w);
+        El::tile_store(smem, c, s.tl, x);
       }
     } else {
       tile_copy_wait();
     }
-    if (T > 0) private_stages<F>(smem, a.dft_tw, s, v, T, (int)r, 0, low);
+    if (T > 0) private_stages<El>(smem, a.dft_tw, s, v, T, (int)r, 0, low);
   }
 
   // ---- middle rounds
@@ -373,26 +422,26 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
   while (T > last) {
     const uint32_t r = min(pl, T - last);
     T -= r;
-    __syncthreads();
+    group_sync<GROUPED>(group, threads);
     const uint32_t low = t & ((1u << T) - 1u);
-    const Private v = private_set(s, low | ((t >> T) << (T + r)), T, r);
-    private_stages<F>(smem, a.dft_tw, s, v, T, (int)r, 0, low);
+    const Private v = private_set<El>(s, low | ((t >> T) << (T + r)), T, r);
+    private_stages<El>(smem, a.dft_tw, s, v, T, (int)r, 0, low);
   }
 
   // ---- last round: stages last - 1 .. 0; inner passes vary sub-transforms
   // fastest across threads (consecutive q), pass 0 the output index: either
   // way a warp writes runs of consecutive elements
-  if (T > 0) __syncthreads();
+  if (T > 0) group_sync<GROUPED>(group, threads);
   const uint32_t tbits = logs - last, gbits = logg - (pl - last);
   const uint32_t dl = MODE == kModeInner ? t & ((1u << gbits) - 1u) : t >> tbits;
   const uint32_t tt = MODE == kModeInner ? t >> gbits : t & ((1u << tbits) - 1u);
   const uint32_t p0 = tbits ? (__brev(tt) >> (32 - tbits)) << last : 0u;
-  const Private v = private_set(s, (dl << logs) | p0, 0, last);
+  const Private v = private_set<El>(s, (dl << logs) | p0, 0, last);
   const uint32_t lmask = (1u << last) - 1u, half = 1u << (logs - 1);
-  private_stages<F>(smem, a.dft_tw, s, v, 0, (int)last, last >= 2 ? 2 : 1, 0);
-  const uint32_t group = last >= 2 ? 4u : 2u;
+  private_stages<El>(smem, a.dft_tw, s, v, 0, (int)last, last >= 2 ? 2 : 1, 0);
+  const uint32_t unit = last >= 2 ? 4u : 2u;
 #pragma unroll 1
-  for (uint32_t j = 0; j < (1u << pl); j += group) {
+  for (uint32_t j = 0; j < (1u << pl); j += unit) {
     const uint64_t d = d0 + dl + ((uint64_t)(j >> last) << gbits);
     const uint32_t c = private_offset(v, j);
     const uint32_t k = __brev(p0 | (j & lmask)) >> (32 - logs);   // output of the group's first position
@@ -404,37 +453,37 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     } else if (d < a.num_sub) {
       out = reverse_digits(a, d) << logs;
     }
-    uint32_t x0[8], x1[8], y[8];
+    uint32_t x0[El::W], x1[El::W], y[El::W];
     if (last >= 2) {
-      uint32_t x2[8], x3[8];
+      uint32_t x2[El::W], x3[El::W];
       {
-        uint32_t A[8], B[8];   // omega_4 = omega_S^(S/4)
-        load_twiddle(A, B, a.dft_tw, half >> 1);
-        tile_load(x1, smem, c ^ v.d0);
-        tile_load(x3, smem, c ^ v.d0 ^ v.d1);
-        sub_lazy<F>(y, x1, x3);
-        add_lazy<F>(x1, x1, x3);
-        mul_split<F>(x3, y, A, B);
+        uint32_t A[El::W], B[El::W];   // omega_4 = omega_S^(S/4)
+        El::load_twiddle(A, B, a.dft_tw, half >> 1);
+        El::tile_load(x1, smem, c ^ v.d0, s.tl);
+        El::tile_load(x3, smem, c ^ v.d0 ^ v.d1, s.tl);
+        El::sub(y, x1, x3);
+        El::add(x1, x1, x3);
+        El::mul_twiddle(x3, y, A, B);
       }
-      tile_load(x0, smem, c);
-      tile_load(x2, smem, c ^ v.d1);
-      sub_lazy<F>(y, x0, x2);
-      add_lazy<F>(x0, x0, x2);
-      add_lazy<F>(x2, y, x3);
-      sub_lazy<F>(x3, y, x3);
+      El::tile_load(x0, smem, c, s.tl);
+      El::tile_load(x2, smem, c ^ v.d1, s.tl);
+      El::sub(y, x0, x2);
+      El::add(x0, x0, x2);
+      El::add(x2, y, x3);
+      El::sub(x3, y, x3);
       if (d < a.num_sub) {
-        store_output<F>(a, out + ((uint64_t)(k + (half >> 1)) << sh), x2);
-        store_output<F>(a, out + ((uint64_t)(k + (half >> 1) + half) << sh), x3);
+        store_output<El>(a, out + ((uint64_t)(k + (half >> 1)) << sh), x2);
+        store_output<El>(a, out + ((uint64_t)(k + (half >> 1) + half) << sh), x3);
       }
     } else {
-      tile_load(x0, smem, c);
-      tile_load(x1, smem, c ^ v.d0);
+      El::tile_load(x0, smem, c, s.tl);
+      El::tile_load(x1, smem, c ^ v.d0, s.tl);
     }
-    sub_lazy<F>(y, x0, x1);
-    add_lazy<F>(x0, x0, x1);
+    El::sub(y, x0, x1);
+    El::add(x0, x0, x1);
     if (d < a.num_sub) {
-      store_output<F>(a, out + ((uint64_t)k << sh), x0);
-      store_output<F>(a, out + ((uint64_t)(k + half) << sh), y);
+      store_output<El>(a, out + ((uint64_t)k << sh), x0);
+      store_output<El>(a, out + ((uint64_t)(k + half) << sh), y);
     }
   }
 }
@@ -455,10 +504,17 @@ __device__ __forceinline__ void pdl_wait_and_trigger() {
 
 template <class F, int MODE, int MAXT>
 __global__ void __launch_bounds__(MAXT, TileBounds<MAXT>::kMinBlocks)
-    ntt_pass_kernel(const __grid_constant__ PassArgs a, const TileShape s) {
+    ntt_pass_kernel(const __grid_constant__ PassArgs a, const TileShape s, uint32_t tiles) {
   extern __shared__ uint4 smem[];
   pdl_wait_and_trigger();
-  pass_tile<F, MODE>(a, s, blockIdx.x, smem);
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+  if constexpr (MAXT == 896) {
+    const uint32_t group = threadIdx.x / kGroupThreads, tile = blockIdx.x * kGroups + group;
+    if (tile < tiles)
+      pass_tile<Elem256<F>, MODE, true>(a, s, tile, base + group * kGroupBytes, threadIdx.x % kGroupThreads, group);
+  } else {
+    pass_tile<Elem256<F>, MODE, false>(a, s, blockIdx.x, base, threadIdx.x, 0);
+  }
 }
 
 }  // namespace gb300ntt

@@ -1,6 +1,6 @@
 // ntt_plan.cu -- plans, resident twiddle tables and the C ABI.
 //
-// A plan fixes (field, log_n), splits N into passes of at most 2^8 points
+// A plan fixes (field, log_n), splits N into passes of at most 2^10 points
 // (the four-step / six-step decomposition of ntt_pass.cuh), and builds on
 // the device every constant the passes multiply by, in Montgomery form:
 //   * per distinct pass size S: omega_S^i and omega_S^-i, i < S/2 (two
@@ -83,13 +83,16 @@ ntt_status cuda_status(cudaError_t e) {
 }
 
 // Default split of log_n into passes of at most kDefaultPassLog bits, as
-// equal as possible, larger ones first.  (Sub-transforms of up to 2^10
-// points keep at least two per tile, so the strided reads of a pass still
-// touch two adjacent elements; the autotuner may pick other splits.)
+// equal as possible, larger ones first; one pass more where that is faster
+// because a smaller sub-transform takes fewer elements per thread (GB300, us,
+// BLS12-381 Fr): 2^9 (5, 4) 9.4 against 10.7, 2^10 (5, 5) 10.1 against 20.3,
+// 2^19 (7, 6, 6) 90 against 106 for (10, 9); not at 2^8 (8.2 against 6.6), 2^18
+// (54 against 51) or 2^20 (177 against 170).  (The autotuner may pick others.)
 constexpr uint32_t kDefaultPassLog = 10;
 
 std::vector<uint32_t> split_passes(uint32_t log_n) {
-  const uint32_t P = (log_n + kDefaultPassLog - 1) / kDefaultPassLog;
+  uint32_t P = (log_n + kDefaultPassLog - 1) / kDefaultPassLog;
+  if (log_n == 9 || log_n == 10 || log_n == 19) P += 1;
   std::vector<uint32_t> s(P, log_n / P);
   for (uint32_t i = 0; i < log_n % P; ++i) s[i] += 1;
   return s;
@@ -280,7 +283,7 @@ void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j
 }
 
 // Tile of a pass launch.  Elements per thread (2^pl) trade parallelism for
-// barriers: as few as still fit the GPU at once (7 CTAs of 128 threads per SM)
+// barriers: as few as still fit the GPU at once (7 groups of 128 threads per SM)
 // while a sub-transform fits 128 threads, so that a small transform is spread
 // over as many warps as there are and its serial chain is short: 2 up to 2^18
 // points, 4 at 2^19, 8 from 2^20 on (and for sub-transforms of 2^9 and 2^10
@@ -288,12 +291,29 @@ void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j
 // one warp).
 TileShape pass_shape(ntt_plan p, uint32_t logs, uint32_t tl) {
   if (tl != 10) return TileShape{logs, tl, 3};
-  const uint64_t slots = (uint64_t)p->sm_count * 128u * (uint64_t)TileBounds<128>::kMinBlocks;
+  const uint64_t slots = (uint64_t)p->sm_count * kGroupThreads * kGroups;
   for (uint32_t pl = 1; pl < 3; ++pl) {
     const uint32_t t = std::max(logs, pl + 5);
     if (t - pl <= 7 && (1ull << p->log_n) >> pl <= slots) return TileShape{logs, t, pl};
   }
   return TileShape{logs, tl, 3};
+}
+
+// Tiles of a batched launch over `elements` points: the same rule with the whole
+// list in place of one transform (all tiles of a launch have the same number of
+// threads: 2^(tl - pl) = 128, or 256 where a pass needs a 2048-element tile).
+uint32_t batch_tile_log(ntt_plan p) {
+  uint32_t t = 10;
+  for (uint32_t j = 0; j < p->num_passes; ++j) t = std::max(t, p->pass_log[j]);
+  return t;
+}
+
+TileShape batch_shape(uint64_t elements, uint32_t logs, uint32_t tile_log, int sm_count) {
+  if (tile_log > 10) return TileShape{logs, 11, 3};
+  const uint64_t slots = (uint64_t)sm_count * kGroupThreads * kGroups;
+  for (uint32_t pl = 1; pl < 3; ++pl)
+    if (logs <= 7 + pl && elements >> pl <= slots) return TileShape{logs, 7 + pl, pl};
+  return TileShape{logs, 10, 3};
 }
 
 // Enqueue one transform: one kernel launch per pass.
@@ -309,7 +329,7 @@ ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cu
     const uint32_t logs = p->pass_log[j];
     cudaError_t e = timing_begin(p, (int)j, st);
     const TileShape shape = pass_shape(p, logs, p->pass_tl[j]);
-    if (e == cudaSuccess) e = L.pass(mode, shape, a, pass_tiles(p->log_n, logs, shape.tl), st);
+    if (e == cudaSuccess) e = L.pass(mode, shape, a, pass_tiles(p->log_n, logs, shape.tl), p->sm_count, st);
     if (e == cudaSuccess) e = timing_end(p, st);
     if (e != cudaSuccess) return cuda_status(e);
   }

@@ -129,7 +129,10 @@ struct BatchJobRef {
   const void *in;
   void *out;
 };
-std::vector<BatchSeg> build_segments(const std::vector<BatchJobRef> &jobs, int field, uint32_t *total_items);
+std::vector<BatchSeg> build_segments(const std::vector<BatchJobRef> &jobs, int field, uint32_t *total_items,
+                                     uint32_t *tile_log);
+uint32_t batch_tile_log(ntt_plan p);   // 11 when a pass of the plan needs a 2048-element tile, else 10
+TileShape batch_shape(uint64_t elements, uint32_t logs, uint32_t tile_log, int sm_count);
 uint64_t batch_wait_limit_ns();
 bool batch_debug_stall();  // the ntt_batch_debug_stall test hook is on
 ntt_status batch_error_word(uint32_t **out);

@@ -184,8 +184,8 @@ void dispatch(ntt_server_s *s, Slot *sl) {
   uint32_t *err = nullptr;
   batch_error_word(&err);
   for (int field = 0; field < 2; ++field) {
-    uint32_t total = 0;
-    std::vector<BatchSeg> segs = build_segments(jobs, field, &total);
+    uint32_t total = 0, tile_log = 10;
+    std::vector<BatchSeg> segs = build_segments(jobs, field, &total, &tile_log);
     if (segs.empty()) continue;
     if (segs.size() > sl->cap) {  // cannot happen with the configured limits
       s->error = NTT_ERR_INVALID_ARG;
@@ -203,7 +203,8 @@ void dispatch(ntt_server_s *s, Slot *sl) {
     b.done = sl->d_ctl[field] + 1;
     b.err = err;
     b.wait_ns = batch_wait_limit_ns();
-    b.grid = (uint32_t)(s->sm_count * kPassCtasPerSm);
+    b.tile_log = tile_log;
+    b.sm_count = s->sm_count;
     if (launchers(field).batch(b, st) != cudaSuccess) s->error = NTT_ERR_CUDA;
   }
   for (uint64_t t : sl->tickets) {

@@ -3,12 +3,13 @@
 //
 // The moduli (the smallest primes c 2^32 + 1, c odd, above floor(pi
 // 2^(b-2)) for b = 377 and 753; generators 7 and 11, the smallest quadratic
-// non-residues) are public constants of this library, written out below.
-// The host derives R mod p, R^2 mod p and (p - 1) / 2^32 from them with a
-// small fixed-width arithmetic; every root of unity, inverse and table is
-// computed on the device (wide_constants_kernel, wide_table_kernel).
+// non-residues) are public constants of this library (fp_wide.cuh).  The host
+// derives R mod p and R^2 mod p from them with a small fixed-width arithmetic;
+// every root of unity, inverse and table is computed on the device
+// (wide_constants_kernel, wide_table_kernel).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <map>
 #include <new>
@@ -22,13 +23,6 @@
 
 namespace gb300ntt {
 namespace {
-
-const uint32_t kP377[12] = {0x00000001u, 0xBBDF2BD5u, 0xF31C6809u, 0x44A29410u, 0x4C762736u, 0xE804177Du,
-                            0x1114CF98u, 0xA252049Cu, 0x1701B839u, 0x69898CC5u, 0x4442D184u, 0x01921FB5u};
-const uint32_t kP753[24] = {0x00000001u, 0x6FDBDCD3u, 0xB96DE80Du, 0xDAD617FEu, 0x85D34C6Fu, 0xFD8DE898u,
-                            0x6AECC4BCu, 0x848BC90Bu, 0x6ADADAA3u, 0x286E9FC2u, 0x14DBE4BEu, 0x86366056u,
-                            0x33679A74u, 0x09BBDF2Au, 0x10F31C68u, 0x3644A294u, 0x7D4C7627u, 0x98E80417u,
-                            0x9C1114CFu, 0x39A25204u, 0xC51701B8u, 0x8469898Cu, 0xB54442D1u, 0x0001921Fu};
 
 #define NTT_TRY_W(expr)                \
   do {                                 \
@@ -64,34 +58,26 @@ void host_double_mod(uint32_t x[NL], const uint32_t p[NL]) {
   }
 }
 
-template <int NL32>
-WideConst<NL32> make_const(const uint32_t p[NL32], uint32_t gen) {
-  constexpr int L = WideShape<NL32>::L;
-  WideConst<NL32> c{};
-  std::memcpy(c.p32, p, sizeof c.p32);
-  auto to29 = [&](uint32_t out[L], const uint32_t x[NL32]) {
-    for (int j = 0; j < L; ++j) {
-      const int bit = 29 * j, w = bit >> 5, sh = bit & 31;
-      const uint64_t lo = w < NL32 ? x[w] : 0u, hi = w + 1 < NL32 ? x[w + 1] : 0u;
-      out[j] = (uint32_t)(((hi << 32) | lo) >> sh) & kM29;
-    }
-  };
-  to29(c.p, p);
-  uint32_t inv = 1;   // p^-1 mod 2^32 by Newton's iteration
-  for (int t = 0; t < 5; ++t) inv *= 2u - p[0] * inv;
-  c.ninv = (0u - inv) & kM29;
-  uint32_t x[NL32] = {1};
-  for (int b = 0; b < 29 * L; ++b) host_double_mod<NL32>(x, p);   // R mod p, R = 2^(29 L)
-  to29(c.one, x);
-  for (int b = 0; b < 29 * L; ++b) host_double_mod<NL32>(x, p);   // R^2 mod p
-  to29(c.r2, x);
-  for (int j = 0; j < NL32; ++j) c.exp_c[j] = j + 1 < NL32 ? p[j + 1] : 0u;   // (p - 1) >> 32 (p0 = 1)
-  c.gen = gen;
+template <class F>
+WideConst<F> make_const() {
+  constexpr int L = F::L;
+  WideConst<F> c{};
+  uint32_t p[L], x[L] = {1};
+  for (int j = 0; j < L; ++j) p[j] = F::p(j);
+  for (int b = 0; b < 32 * L; ++b) host_double_mod<L>(x, p);   // R mod p, R = 2^(32 L)
+  std::memcpy(c.one, x, sizeof c.one);
+  for (int b = 0; b < 32 * L; ++b) host_double_mod<L>(x, p);   // R^2 mod p
+  std::memcpy(c.r2, x, sizeof c.r2);
+  return c;
+}
+
+template <class F>
+const WideConst<F> &wide_const() {
+  static const WideConst<F> c = make_const<F>();
   return c;
 }
 
 int limbs_of(int field) { return field == NTT_FIELD_W377 ? 12 : 24; }
-int tile_log(int field) { return field == NTT_FIELD_W377 ? WideShape<12>::kLog : WideShape<24>::kLog; }
 
 struct WidePlan {
   uint32_t log_n = 0, num_passes = 0;
@@ -110,20 +96,22 @@ struct WidePlan {
 
 std::mutex g_wide_mu;
 bool g_wide_ready[8] = {};
+int g_wide_sms[8] = {};   // multiprocessors of each device
 std::map<std::tuple<int, int, uint32_t>, WidePlan *> g_wide_plans;   // (device, field, log_n)
 
 ntt_status cuda_w(cudaError_t e) { return cuda_status(e); }
 
-template <int NL32>
+template <class F>
 ntt_status gen_table(uint4 *out, uint32_t log_m, int dir, bool use_m_inv, uint32_t log_mp, uint64_t count, int two_d,
-                     bool constant, uint32_t *kbuf, cudaStream_t st) {
-  constexpr int L = WideShape<NL32>::L;
-  wide_constants_kernel<NL32><<<1, 1, 0, st>>>(kbuf, log_m);
+                     bool constant, bool split, uint32_t *kbuf, cudaStream_t st) {
+  constexpr int L = F::L;
+  wide_constants_kernel<F><<<1, 1, 0, st>>>(kbuf, log_m, wide_const<F>());
   const uint32_t *ladder = constant ? nullptr : kbuf + (dir ? 32 : 0) * L;
   const uint32_t *init = kbuf + (use_m_inv ? 64 : 65) * L;
   uint64_t blocks = (count + 255) / 256;
   if (blocks > 152ull * 32) blocks = 152ull * 32;
-  wide_table_kernel<NL32><<<(unsigned)(blocks ? blocks : 1), 256, 0, st>>>(out, log_mp, ladder, init, count, two_d);
+  wide_table_kernel<F><<<(unsigned)(blocks ? blocks : 1), 256, 0, st>>>(out, log_mp, ladder, init, count, two_d,
+                                                                         split ? 1 : 0);
   return cuda_w(cudaGetLastError());
 }
 
@@ -139,16 +127,23 @@ ntt_status alloc_w(WidePlan *w, uint4 **out, uint64_t bytes) {
   return NTT_OK;
 }
 
-template <int NL32>
-ntt_status build_wide(int field, uint32_t log_n, WidePlan *w) {
-  constexpr int L = WideShape<NL32>::L, LP = WideShape<NL32>::LP;
-  const uint32_t TL = (uint32_t)tile_log(field);
-  const uint32_t P = (log_n + TL - 1) / TL;
+// Passes of a transform: up to 2^8 points one (2 or 4 elements per thread hold
+// them in one CTA), else as few as the largest tile allows, at least two (one
+// CTA with a 2^10-point sub-transform is slower than two passes over several).
+uint32_t wide_passes(uint32_t log_n, uint32_t tile_log) {
+  if (log_n <= 8) return 1;
+  return std::max<uint32_t>(2, (log_n + tile_log - 1) / tile_log);
+}
+
+template <class F>
+ntt_status build_wide(uint32_t log_n, WidePlan *w) {
+  constexpr int L = F::L;
+  const uint32_t P = wide_passes(log_n, (uint32_t)WideShape<F>::kLog);
   if (P > (uint32_t)kMaxPasses) return NTT_ERR_UNSUPPORTED;
   w->log_n = log_n;
   w->num_passes = P;
   for (uint32_t j = 0; j < P; ++j) w->pass_log[j] = log_n / P + (j < log_n % P ? 1 : 0);
-  const uint64_t eb = 4ull * LP;   // table entry: LP words of 29-bit limbs
+  const uint64_t eb = 4ull * L;   // table entry
   uint32_t *kbuf = nullptr;
   if (cudaMalloc(&kbuf, 66 * 4 * L) != cudaSuccess) return NTT_ERR_OOM;
   w->allocs.push_back(kbuf);
@@ -159,8 +154,8 @@ ntt_status build_wide(int field, uint32_t log_n, WidePlan *w) {
     for (int dir = 0; dir < 2; ++dir) {
       if (w->dft_tw[dir][logs]) continue;
       const uint64_t cnt = logs ? (1ull << (logs - 1)) : 1;
-      NTT_TRY_W(alloc_w(w, &w->dft_tw[dir][logs], cnt * eb));
-      NTT_TRY_W(gen_table<NL32>(w->dft_tw[dir][logs], logs, dir, false, 0, cnt, 0, false, kbuf, st));
+      NTT_TRY_W(alloc_w(w, &w->dft_tw[dir][logs], cnt * 2 * eb));
+      NTT_TRY_W(gen_table<F>(w->dft_tw[dir][logs], logs, dir, false, 0, cnt, 0, false, true, kbuf, st));
     }
   }
   uint32_t log_m = w->pass_log[0];
@@ -169,26 +164,26 @@ ntt_status build_wide(int field, uint32_t log_n, WidePlan *w) {
     log_m += logs;
     for (int dir = 0; dir < 2; ++dir) {
       NTT_TRY_W(alloc_w(w, &w->tw[dir][j], (1ull << log_m) * eb));
-      NTT_TRY_W(gen_table<NL32>(w->tw[dir][j], log_m, dir, dir == 1 && j == P - 1, log_mp, 1ull << log_m, 1, false,
-                                kbuf, st));
+      NTT_TRY_W(gen_table<F>(w->tw[dir][j], log_m, dir, dir == 1 && j == P - 1, log_mp, 1ull << log_m, 1, false, false,
+                             kbuf, st));
     }
   }
   if (P == 1) {   // single-pass inverse: N^-1 as the pass-0 multiplier
     NTT_TRY_W(alloc_w(w, &w->pre_inv, (1ull << log_n) * eb));
-    NTT_TRY_W(gen_table<NL32>(w->pre_inv, log_n, 0, true, 0, 1ull << log_n, 0, true, kbuf, st));
+    NTT_TRY_W(gen_table<F>(w->pre_inv, log_n, 0, true, 0, 1ull << log_n, 0, true, false, kbuf, st));
   }
-  if (P > 1) NTT_TRY_W(alloc_w(w, &w->scratch, (1ull << log_n) * 4ull * NL32));   // memory-layout elements
+  if (P > 1) NTT_TRY_W(alloc_w(w, &w->scratch, (1ull << log_n) * eb));
   return cuda_w(cudaDeviceSynchronize());
 }
 
-// The coset tables of shift s (NL32 words, 0 < s < p), s^i and s^-i for
+// The coset tables of shift s (L words, 0 < s < p), s^i and s^-i for
 // i < N: allocated on the first coset call for this (device, field, size),
 // rewritten in place when a call brings another shift (after the device is
 // idle: transforms enqueued earlier may still read the old tables).
-template <int NL32>
+template <class F>
 ntt_status build_wide_coset(WidePlan *w, const uint32_t *shift) {
-  constexpr int L = WideShape<NL32>::L, LP = WideShape<NL32>::LP;
-  const uint64_t n = 1ull << w->log_n, eb = 4ull * LP;
+  constexpr int L = F::L;
+  const uint64_t n = 1ull << w->log_n, eb = 4ull * L;
   if (!w->coset_post) {
     const size_t kept = w->allocs.size();
     uint4 *pre = nullptr, *post = nullptr;
@@ -207,81 +202,71 @@ ntt_status build_wide_coset(WidePlan *w, const uint32_t *shift) {
   w->coset_ready = false;   // until the tables below are written
   uint4 *pre = w->coset_pre, *post = w->coset_post;
   cudaStream_t st = nullptr;
-  NTT_TRY_W(cuda_w(cudaMemcpy(w->kbuf + 64 * L, shift, 4 * NL32, cudaMemcpyHostToDevice)));
-  wide_coset_constants_kernel<NL32><<<1, 1, 0, st>>>(w->kbuf);
+  NTT_TRY_W(cuda_w(cudaMemcpy(w->kbuf + 64 * L, shift, 4 * L, cudaMemcpyHostToDevice)));
+  wide_coset_constants_kernel<F><<<1, 1, 0, st>>>(w->kbuf, wide_const<F>());
   uint64_t blocks = (n + 255) / 256;
   if (blocks > 152ull * 32) blocks = 152ull * 32;
-  wide_table_kernel<NL32><<<(unsigned)blocks, 256, 0, st>>>(pre, 0, w->kbuf, w->kbuf + 65 * L, n, 0);
-  wide_table_kernel<NL32><<<(unsigned)blocks, 256, 0, st>>>(post, 0, w->kbuf + 32 * L, w->kbuf + 65 * L, n, 0);
+  wide_table_kernel<F><<<(unsigned)blocks, 256, 0, st>>>(pre, 0, w->kbuf, w->kbuf + 65 * L, n, 0, 0);
+  wide_table_kernel<F><<<(unsigned)blocks, 256, 0, st>>>(post, 0, w->kbuf + 32 * L, w->kbuf + 65 * L, n, 0, 0);
   NTT_TRY_W(cuda_w(cudaGetLastError()));
   NTT_TRY_W(cuda_w(cudaDeviceSynchronize()));
-  std::memcpy(w->coset_shift, shift, 4 * NL32);
+  std::memcpy(w->coset_shift, shift, 4 * L);
   w->coset_ready = true;
   return NTT_OK;
 }
 
-template <int NL, int LOGS>
-cudaError_t wide_launch(int mode, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  const int smem = WideShape<NL>::kBytes;
+// Tile of a pass launch, by the rule of the 256-bit passes (pass_shape in
+// ntt_plan.cu): as few elements per thread as still fit the GPU at once.
+template <class F>
+TileShape wide_shape(uint32_t log_n, uint32_t logs, int sms) {
+  using W = WideShape<F>;
+  const uint64_t slots = (uint64_t)sms * W::kThreads * W::kMinBlocks;
+  for (uint32_t pl = 1; pl < 3; ++pl) {
+    const uint32_t t = std::max(logs, pl + 5);
+    if ((1u << (t - pl)) <= (uint32_t)W::kThreads && (1ull << log_n) >> pl <= slots) return TileShape{logs, t, pl};
+  }
+  return TileShape{logs, (uint32_t)W::kLog, 3};
+}
+
+template <class F, int MODE>
+cudaError_t wide_launch(const PassArgs &a, const TileShape &s, cudaStream_t st) {
+  const uint64_t g = 1ull << (s.tl - s.logs), tiles = (a.num_sub + g - 1) / g;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)tiles);
+  cfg.blockDim = dim3(1u << (s.tl - s.pl));
+  cfg.dynamicSmemBytes = (size_t)(4 * F::L) << s.tl;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];   // see pdl_wait_and_trigger
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, wide_pass_kernel<F, MODE>, a, s);
+}
+
+template <class F>
+cudaError_t wide_pass(int mode, const PassArgs &a, uint32_t log_n, uint32_t logs, int sms, cudaStream_t st) {
+  const TileShape s = wide_shape<F>(log_n, logs, sms);
   switch (mode) {
-    case kModeInner: wide_pass_kernel<NL, LOGS, kModeInner><<<(unsigned)tiles, 256, smem, st>>>(a); break;
-    case kModeFirst: wide_pass_kernel<NL, LOGS, kModeFirst><<<(unsigned)tiles, 256, smem, st>>>(a); break;
-    default: wide_pass_kernel<NL, LOGS, kModeFirstPre><<<(unsigned)tiles, 256, smem, st>>>(a); break;
+    case kModeInner: return wide_launch<F, kModeInner>(a, s, st);
+    case kModeFirst: return wide_launch<F, kModeFirst>(a, s, st);
+    default: return wide_launch<F, kModeFirstPre>(a, s, st);
   }
-  return cudaGetLastError();
 }
 
-template <int NL, int LOGS>
-cudaError_t wide_attr() {
-  const int smem = WideShape<NL>::kBytes;
-  cudaError_t e = cudaFuncSetAttribute(wide_pass_kernel<NL, LOGS, kModeInner>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(wide_pass_kernel<NL, LOGS, kModeFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(wide_pass_kernel<NL, LOGS, kModeFirstPre>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem);
-  return e;
-}
-
-template <int NL>
+template <class F>
 cudaError_t wide_set_attrs() {
-  cudaError_t e = wide_attr<NL, 1>();
-  if (e == cudaSuccess) e = wide_attr<NL, 2>();
-  if (e == cudaSuccess) e = wide_attr<NL, 3>();
-  if (e == cudaSuccess) e = wide_attr<NL, 4>();
-  if (e == cudaSuccess) e = wide_attr<NL, 5>();
-  if (e == cudaSuccess) e = wide_attr<NL, 6>();
-  if (e == cudaSuccess) e = wide_attr<NL, 7>();
-  if (e == cudaSuccess) e = wide_attr<NL, 8>();
-  if (e == cudaSuccess) e = wide_attr<NL, 9>();
-  if constexpr (WideShape<NL>::kLog >= 10) {
-    if (e == cudaSuccess) e = wide_attr<NL, 10>();
-  }
+  constexpr int smem = WideShape<F>::kBytes;
+  cudaError_t e = cudaFuncSetAttribute(wide_pass_kernel<F, kModeInner>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(wide_pass_kernel<F, kModeFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(wide_pass_kernel<F, kModeFirstPre>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return e;
-}
-
-template <int NL>
-cudaError_t wide_dispatch(int logs, int mode, const PassArgs &a, uint64_t tiles, cudaStream_t st) {
-  switch (logs) {
-    case 1: return wide_launch<NL, 1>(mode, a, tiles, st);
-    case 2: return wide_launch<NL, 2>(mode, a, tiles, st);
-    case 3: return wide_launch<NL, 3>(mode, a, tiles, st);
-    case 4: return wide_launch<NL, 4>(mode, a, tiles, st);
-    case 5: return wide_launch<NL, 5>(mode, a, tiles, st);
-    case 6: return wide_launch<NL, 6>(mode, a, tiles, st);
-    case 7: return wide_launch<NL, 7>(mode, a, tiles, st);
-    case 8: return wide_launch<NL, 8>(mode, a, tiles, st);
-    case 9: return wide_launch<NL, 9>(mode, a, tiles, st);
-    case 10:
-      if constexpr (WideShape<NL>::kLog >= 10) return wide_launch<NL, 10>(mode, a, tiles, st);
-      return cudaErrorInvalidValue;
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 // The (device, field, size) tables, built on first use; with a shift
-// (NL32 words), also the coset tables of that shift.  The caller holds
+// (L words), also the coset tables of that shift.  The caller holds
 // g_wide_mu until its transform is enqueued, so no other call can rewrite
 // the coset tables in between.
 ntt_status wide_plan(int field, uint32_t log_n, const uint32_t *shift, WidePlan **out) {
@@ -289,12 +274,9 @@ ntt_status wide_plan(int field, uint32_t log_n, const uint32_t *shift, WidePlan 
   if (cudaGetDevice(&dev) != cudaSuccess) return NTT_ERR_NO_DEVICE;
   if (dev < 0 || dev >= 8) return NTT_ERR_UNSUPPORTED;
   if (!g_wide_ready[dev]) {
-    const WideConst<12> c12 = make_const<12>(kP377, 7);
-    const WideConst<24> c24 = make_const<24>(kP753, 11);
-    NTT_TRY_W(cuda_w(cudaMemcpyToSymbol(c_wide12, &c12, sizeof c12)));
-    NTT_TRY_W(cuda_w(cudaMemcpyToSymbol(c_wide24, &c24, sizeof c24)));
-    NTT_TRY_W(cuda_w(wide_set_attrs<12>()));
-    NTT_TRY_W(cuda_w(wide_set_attrs<24>()));
+    NTT_TRY_W(cuda_w(wide_set_attrs<FieldW377>()));
+    NTT_TRY_W(cuda_w(wide_set_attrs<FieldW753>()));
+    NTT_TRY_W(cuda_w(cudaDeviceGetAttribute(&g_wide_sms[dev], cudaDevAttrMultiProcessorCount, dev)));
     g_wide_ready[dev] = true;
   }
   auto key = std::make_tuple(dev, field, log_n);
@@ -305,7 +287,7 @@ ntt_status wide_plan(int field, uint32_t log_n, const uint32_t *shift, WidePlan 
   } else {
     w = new (std::nothrow) WidePlan();
     if (!w) return NTT_ERR_OOM;
-    const ntt_status s = limbs_of(field) == 12 ? build_wide<12>(field, log_n, w) : build_wide<24>(field, log_n, w);
+    const ntt_status s = limbs_of(field) == 12 ? build_wide<FieldW377>(log_n, w) : build_wide<FieldW753>(log_n, w);
     if (s != NTT_OK) {
       for (void *p : w->allocs) cudaFree(p);
       delete w;
@@ -316,16 +298,17 @@ ntt_status wide_plan(int field, uint32_t log_n, const uint32_t *shift, WidePlan 
   if (shift && (!w->coset_ready || std::memcmp(w->coset_shift, shift, 4 * limbs_of(field)) != 0)) {
     // a failure leaves forward and inverse usable and the coset tables
     // marked unwritten (the next coset call writes them again)
-    NTT_TRY_W(limbs_of(field) == 12 ? build_wide_coset<12>(w, shift) : build_wide_coset<24>(w, shift));
+    NTT_TRY_W(limbs_of(field) == 12 ? build_wide_coset<FieldW377>(w, shift) : build_wide_coset<FieldW753>(w, shift));
   }
   *out = w;
   return NTT_OK;
 }
 
-// 0 < s < p for a shift of NL32 little-endian words.
+// 0 < s < p for a shift of 12 or 24 little-endian words.
 bool shift_in_range(ntt_field field, const uint32_t *sw) {
   const int nl = limbs_of((int)field);
-  const uint32_t *p = field == NTT_FIELD_W377 ? kP377 : kP753;
+  uint32_t p[24];
+  for (int j = 0; j < nl; ++j) p[j] = nl == 12 ? FieldW377::p(j) : FieldW753::p(j);
   bool zero = true;
   for (int j = 0; j < nl; ++j) zero = zero && sw[j] == 0;
   if (zero) return false;
@@ -334,7 +317,7 @@ bool shift_in_range(ntt_field field, const uint32_t *sw) {
   return false;   // s == p
 }
 
-// One transform; `shift` (NL32 words, checked by the caller) is used by the
+// One transform; `shift` (L words, checked by the caller) is used by the
 // coset kinds only.  The table lock is held until every pass is enqueued.
 ntt_status wide_transform(ntt_field field, ntt_kind kind, uint32_t log_n, const uint32_t *shift, const void *d_in,
                           void *d_out, ntt_stream stream) {
@@ -344,7 +327,8 @@ ntt_status wide_transform(ntt_field field, ntt_kind kind, uint32_t log_n, const 
   const ntt_status s = wide_plan((int)field, log_n, coset ? shift : nullptr, &w);
   if (s != NTT_OK) return s;
   const int NL = limbs_of((int)field);
-  const uint32_t TL = (uint32_t)tile_log((int)field);
+  int dev = 0;
+  NTT_TRY_W(cuda_w(cudaGetDevice(&dev)));   // below 8 (wide_plan)
   const int dir = (kind == NTT_KIND_INVERSE || kind == NTT_KIND_COSET_INVERSE) ? 1 : 0;
   const uint32_t P = w->num_passes;
   uint4 *work = (P > 1 && d_in == d_out) ? w->scratch : (uint4 *)d_out;
@@ -377,10 +361,10 @@ ntt_status wide_transform(ntt_field field, ntt_kind kind, uint32_t log_n, const 
       mode = kModeInner;
     }
     if (j == P - 1 && kind == NTT_KIND_COSET_INVERSE) a.post = w->coset_post;
-    const uint64_t g = 1ull << (TL - logs);
-    const uint64_t tiles = (a.num_sub + g - 1) / g;
-    const cudaError_t e = NL == 12 ? wide_dispatch<12>((int)logs, mode, a, tiles, (cudaStream_t)stream)
-                                   : wide_dispatch<24>((int)logs, mode, a, tiles, (cudaStream_t)stream);
+    a.n_vec = 1ull << log_n;
+    a.n_mul = a.mul ? (j == 0 ? 1ull << log_n : 1ull << (a.log_mp + logs)) : 0;
+    const cudaError_t e = NL == 12 ? wide_pass<FieldW377>(mode, a, log_n, logs, g_wide_sms[dev], (cudaStream_t)stream)
+                                   : wide_pass<FieldW753>(mode, a, log_n, logs, g_wide_sms[dev], (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_status(e);
   }
   return NTT_OK;
