@@ -602,6 +602,38 @@ __global__ void __launch_bounds__(kEcThreads, C::kTreeMinBlocks)
   }
 }
 
+// BR, the lowest levels at once where there are many buckets: one thread takes
+// 2^j adjacent leaves of a window by running sums (W = sum (i + 1) B_i, B = 2^j
+// sum B_i), 2 additions a bucket (28 products) where the tree's levels take 51
+// products per node.
+template <class C>
+__global__ void __launch_bounds__(kEcThreads, C::kTreeMinBlocks)
+    msm_reduce_chunk_kernel(uint32_t j, uint32_t lb, uint32_t kb, uint32_t nk, const uint4 *bucket_sum,
+                            const uint4 *pieces, const uint32_t *offsets, const MsmTotals *tot, uint4 *heap_w,
+                            uint4 *heap_b) {
+  using T = typename C::T;
+  const uint32_t S = tot->seg_len, s = lb - j;
+  const uint64_t per = 1ull << s, total = per * nk;
+  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total;
+       t += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t heap0 = (kb + (t >> s)) << lb, b = t & (per - 1);
+    Xyzz<T> w, run, q;
+    xyzz_set_inf(w);
+    xyzz_set_inf(run);
+#pragma unroll 1
+    for (int i = (1 << j) - 1; i >= 0; --i) {
+      load_bucket(q, bucket_sum, pieces, offsets, S, heap0 + (b << j) + i);
+      xyzz_add<T, true>(run, q);
+      xyzz_add<T, true>(w, run);
+    }
+    const uint64_t node = heap0 + per + b;
+    store_point_xyzz(heap_w, node, w);
+#pragma unroll 1
+    for (uint32_t i = 0; i < j; ++i) xyzz_dbl<T, true>(run, run);
+    store_point_xyzz(heap_b, node, run);
+  }
+}
+
 // Coordinate `lane` of bucket b's sum (load_bucket, four lanes per point).
 template <class T>
 __device__ __forceinline__ void quad_load_bucket(uint32_t v[T::L], const uint4 *bucket_sum, const uint4 *pieces,
@@ -1141,7 +1173,20 @@ ntt_status enqueue_msm(msm_plan p, const uint4 *sc, const uint4 *pt, uint64_t n,
       msm_combine_long_kernel<C><<<grid_for(4 * (max_span / (4 * step) + 1) * p->K, kEcThreads, sms, 4), kEcThreads, 0,
                                    st>>>(p->offsets, nb, p->tot, p->lists, l, p->pieces);
   }
-  for (int s = (int)lb - 1; s >= 0 && tree_ke > tree_kb; --s) {
+  // leaves of the tree that one thread takes at once: while that still fills
+  // the GPU about once
+  int s = (int)lb - 1;
+  if (tree_ke > tree_kb) {
+    const uint64_t leaves = ((uint64_t)(tree_ke - tree_kb)) << lb;
+    uint32_t j = 0;
+    while (j + 1 < lb && (leaves >> (j + 1)) * 4 >= (uint64_t)sms * C::kTreeMinBlocks * kEcThreads * 3) ++j;
+    if (j >= 2) {
+      msm_reduce_chunk_kernel<C><<<grid_for(leaves >> j, kEcThreads, sms, C::kTreeMinBlocks), kEcThreads, 0, st>>>(
+          j, lb, tree_kb, tree_ke - tree_kb, p->bucket_sum, p->pieces, p->offsets, p->tot, p->heap_w, p->heap_b);
+      s = (int)(lb - j) - 1;
+    }
+  }
+  for (; s >= 0 && tree_ke > tree_kb; --s) {
     const uint64_t work = ((uint64_t)(tree_ke - tree_kb)) << s;
     if (work <= (uint64_t)sms * kQuadNodesPerSm) {
       msm_reduce_level_quad_kernel<C><<<grid_for(8 * work, kEcThreads, sms, 8), kEcThreads, 0, st>>>(
