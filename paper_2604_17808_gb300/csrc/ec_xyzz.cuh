@@ -487,14 +487,14 @@ __device__ __forceinline__ void quad_pick(uint32_t r[L], bool first, const uint3
 }
 
 // v = 2 v (dbl-2008-s-1, a = 0); O stays O.
-template <class T>
+template <class T, bool kCall = true>
 __device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
   constexpr int L = T::L;
   const int lane = threadIdx.x & 3;
   uint32_t a[L], b[L], p[L], V[L], M[L], q[L], g[L], h[L];
   T::add(a, v, v);
   quad_pick<L>(a, lane == 1, a, v);       // lane 1: U = 2 Y; lane 0: X
-  f_mul<T, true>(p, a, a);                // lane 0: X^2, lane 1: V = U^2
+  f_mul<T, kCall>(p, a, a);                // lane 0: X^2, lane 1: V = U^2
   quad_get<L>(V, p, 1);
   quad_get<L>(g, p, 0);
   T::add(M, g, g);
@@ -502,7 +502,7 @@ __device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
   quad_pick<L>(a, lane == 3, M, a);
   quad_pick<L>(a, lane == 2, v, a);
   quad_pick<L>(b, lane == 3, M, V);
-  f_mul<T, true>(q, a, b);                // S = X V, W = U V, ZZ3 = ZZ V, M^2
+  f_mul<T, kCall>(q, a, b);                // S = X V, W = U V, ZZ3 = ZZ V, M^2
   quad_get<L>(g, q, lane == 0 ? 3 : 1);   // lane 0: M^2, lane 3: W
   uint32_t x3[L];
   T::sub(x3, g, q);
@@ -511,7 +511,7 @@ __device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
   quad_pick<L>(a, lane == 0, M, q);
   quad_pick<L>(a, lane == 3, g, a);
   quad_pick<L>(b, lane == 0, b, v);
-  f_mul<T, true>(h, a, b);                // lane 0: M (S - X3), lane 1: W Y, lane 3: W ZZZ
+  f_mul<T, kCall>(h, a, b);                // lane 0: M (S - X3), lane 1: W Y, lane 3: W ZZZ
   quad_get<L>(g, h, 0);
   T::sub(g, g, h);                        // lane 1: Y3
   quad_pick<L>(v, lane == 0, x3, q);

@@ -711,12 +711,12 @@ __global__ void msm_merge_kernel(uint32_t c, uint32_t kb, uint32_t ke, const uin
     if (lb == 0) quad_load_bucket<T>(w, bucket_sum, pieces, offsets, S, (uint64_t)k);
     else quad_load<T>(w, heap_w, ((uint64_t)k << lb) + 1);
 #pragma unroll 1
-    for (uint32_t j = 0; j < doublings; ++j) quad_dbl<T>(v);
+    for (uint32_t j = 0; j < doublings; ++j) quad_dbl<T, false>(v);
     quad_add<T>(v, w);
     doublings = c;
   }
 #pragma unroll 1
-  for (uint32_t j = 0; j < c * kb; ++j) quad_dbl<T>(v);
+  for (uint32_t j = 0; j < c * kb; ++j) quad_dbl<T, false>(v);
   // affine: x = X ZZZ / (ZZ ZZZ), y = Y ZZ / (ZZ ZZZ)
   uint32_t z[L], t[L];
   quad_get<L>(z, v, 2);
