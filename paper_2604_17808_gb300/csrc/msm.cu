@@ -644,9 +644,9 @@ __device__ __forceinline__ void quad_load_bucket(uint32_t v[T::L], const uint4 *
   else quad_load<T>(v, pieces, 2 * (uint64_t)(ob / S) + 1);
 }
 
-// The same level with eight lanes per node, four for W and four for B: a level
-// with few nodes takes the time of its dependent products, 8 deep this way
-// instead of 51 (BLS12-381: 65 us a level by one thread per node).
+// The same level with four lanes for a node's W and four, of another warp, for
+// its B: a level with few nodes takes the time of its dependent products, 8 or 7
+// deep this way instead of 51 (BLS12-381: 65 us a level by one thread per node).
 template <class C>
 __global__ void __launch_bounds__(kEcThreads)
     msm_reduce_level_quad_kernel(uint32_t s, uint32_t lb, uint32_t kb, uint32_t nk, const uint4 *bucket_sum,
@@ -656,38 +656,34 @@ __global__ void __launch_bounds__(kEcThreads)
   constexpr int L = T::L;
   const uint32_t S = tot->seg_len;
   const uint64_t per = 1ull << s, total = per * nk;
-  const uint64_t group = (uint64_t)gridDim.x * (blockDim.x / 8);
-  const uint64_t first = (uint64_t)blockIdx.x * (blockDim.x / 8) + (threadIdx.x / 8);
-  const bool is_b = (threadIdx.x & 4) != 0;
-  const bool leaves = s + 1 == lb;
+  // warp pairs: eight nodes' W and B
+  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, warps = gridDim.x * (blockDim.x / 32);
+  const bool is_b = warp & 1u, leaves = s + 1 == lb;
+  if (is_b && s == 0) return;   // the root's B is not needed
   // every lane of the warp takes part in each step; a node past the end is a
   // copy of the last one that is not stored
-  for (uint64_t t0 = first - (threadIdx.x % 32) / 8; t0 < total; t0 += group) {
-    const uint64_t t = t0 + (threadIdx.x % 32) / 8;
+  for (uint64_t t0 = 8ull * (warp / 2); t0 < total; t0 += 8ull * (warps / 2)) {
+    const uint64_t t = t0 + (threadIdx.x % 32) / 4;
     const bool live = t < total;
     const uint64_t tc = live ? t : total - 1;
     const uint64_t k = kb + (tc >> s), b = tc & (per - 1);
-    const uint64_t heap0 = k << lb, node = heap0 + per + b;
-    uint32_t v[L], w[L], x[L];
+    const uint64_t heap0 = k << lb, node = heap0 + per + b, child = heap0 + 2 * per + 2 * b;
+    uint32_t v[L], w[L];
     if (leaves) {
       quad_load_bucket<T>(v, bucket_sum, pieces, offsets, S, heap0 + 2 * b);
       quad_load_bucket<T>(w, bucket_sum, pieces, offsets, S, heap0 + 2 * b + 1);
-      fv_copy<L>(x, w);                  // W = (B_L + B_R) + B_R
     } else {
-      const uint64_t child = heap0 + 2 * per + 2 * b;
       quad_load<T>(v, is_b ? heap_b : heap_w, child);
       quad_load<T>(w, is_b ? heap_b : heap_w, child + 1);
-      quad_load<T>(x, heap_b, child + 1);   // W = W_L + W_R + B_R
     }
     quad_add<T>(v, w);
-    uint32_t y[L];
-    fv_copy<L>(y, v);
-    quad_add<T>(y, x);                   // the W lanes' result
-    quad_dbl<T>(v);                      // the B lanes': 2 (B_L + B_R)
-    if (live) {
-      if (!is_b) quad_store<T>(heap_w, node, y);
-      else if (s != 0) quad_store<T>(heap_b, node, v);   // the root's B is not needed
+    if (is_b) {
+      quad_dbl<T>(v);                               // B = 2 (B_L + B_R)
+    } else {
+      if (!leaves) quad_load<T>(w, heap_b, child + 1);
+      quad_add<T>(v, w);                            // W = W_L + W_R + B_R (leaves: W_j = B_j)
     }
+    if (live) quad_store<T>(is_b ? heap_b : heap_w, node, v);
   }
 }
 

@@ -25,12 +25,16 @@ def _case(name, n, r):
         return [5] * n, [(3 if i % 2 else r - 3) for i in range(n)]
     if name == "sparse":         # one point in a hundred
         return [int(rng.randint(1, 2**30)) * 2**190 % r if i % 100 == 0 else 0 for i in range(n)], ts
+    if name == "repeated":       # many equal and opposite neighbours, points at infinity, dense scalars
+        return [int(v) * 2**220 % r + int(v) for v in rng.randint(1, 2**31 - 1, n)], [(0, 1, r - 1, 2)[int(v)] for v in
+                                                                                     rng.randint(0, 4, n)]
     return [int(v) for v in rng.randint(0, 2, n)], ts   # bits
 
 
 @pytest.mark.parametrize("curve", ["bn254_g1", "bls12_381_g1"])
-@pytest.mark.parametrize("name", ["constant", "cancel", "sparse", "bits"])
-@pytest.mark.parametrize("n,flat", [(9, False), (300, True), (20_000, False), (20_000, True)])
+@pytest.mark.parametrize("name", ["constant", "cancel", "sparse", "bits", "repeated"])
+@pytest.mark.parametrize("n,flat", [(9, False), (300, True), (20_000, False), (20_000, True), (90_001, False),
+                                    (90_001, True)])
 def test_pieces(curve, name, n, flat):
     import paper_2604_17808_gb300 as lib
 
