@@ -49,6 +49,7 @@ constexpr uint32_t neg_inv_u32(uint32_t p0) {
 // BLS12-381 scalar field r (255 bits, 2-adicity 32, generator 7).
 struct FieldBls12381Fr {
   static constexpr int kId = 0;
+  static constexpr uint32_t kLazy = 2;       // values inside a transform pass stay below kLazy p
   static constexpr bool kSubtract = true;   // redc_row subtracts T_0 r
   static constexpr uint32_t P0 = 0x00000001u, P1 = 0xffffffffu, P2 = 0xfffe5bfeu, P3 = 0x53bda402u,
                             P4 = 0x09a1d805u, P5 = 0x3339d808u, P6 = 0x299d7d48u, P7 = 0x73eda753u;
@@ -58,6 +59,7 @@ struct FieldBls12381Fr {
 // BN254 scalar field r (254 bits, 2-adicity 28, generator 5).
 struct FieldBn254Fr {
   static constexpr int kId = 1;
+  static constexpr uint32_t kLazy = 3;
   static constexpr bool kSubtract = false;
   static constexpr uint32_t P0 = 0xf0000001u, P1 = 0x43e1f593u, P2 = 0x79b97091u, P3 = 0x2833e848u,
                             P4 = 0x8181585du, P5 = 0xb85045b6u, P6 = 0xe131a029u, P7 = 0x30644e72u;
@@ -350,23 +352,26 @@ __device__ __forceinline__ void sub_mod(uint32_t r[8], const uint32_t a[8], cons
   for (int j = 0; j < 8; ++j) r[j] = d[j];
 }
 
-// ------------------------------------------------ lazy values in [0, 2p)
-// Inside a transform pass values stay in [0, 2p), which fits 256 bits for both
-// fields.
+// ------------------------------------------- lazy values in [0, kLazy p)
+// Inside a transform pass values stay in [0, 2p) (BLS12-381 Fr) or [0, 3p) (BN254
+// Fr, where 3p < 2^256 and mul_split then ends below 3p without a subtraction).
 
-// Limb j of 2p.
+// Limb j of kLazy p.
 template <class F>
-struct TwoP {
-  static constexpr uint32_t W0 = F::P0 << 1, W1 = F::P1 << 1 | F::P0 >> 31, W2 = F::P2 << 1 | F::P1 >> 31,
-                            W3 = F::P3 << 1 | F::P2 >> 31, W4 = F::P4 << 1 | F::P3 >> 31,
-                            W5 = F::P5 << 1 | F::P4 >> 31, W6 = F::P6 << 1 | F::P5 >> 31,
-                            W7 = F::P7 << 1 | F::P6 >> 31;
+struct LazyP {
+  static constexpr uint64_t k = F::kLazy;
+  static constexpr uint64_t C0 = k * F::P0, C1 = k * F::P1 + (C0 >> 32), C2 = k * F::P2 + (C1 >> 32),
+                            C3 = k * F::P3 + (C2 >> 32), C4 = k * F::P4 + (C3 >> 32), C5 = k * F::P5 + (C4 >> 32),
+                            C6 = k * F::P6 + (C5 >> 32), C7 = k * F::P7 + (C6 >> 32);
+  static_assert(C7 >> 32 == 0, "kLazy p < 2^256");
+  static constexpr uint32_t W0 = (uint32_t)C0, W1 = (uint32_t)C1, W2 = (uint32_t)C2, W3 = (uint32_t)C3,
+                            W4 = (uint32_t)C4, W5 = (uint32_t)C5, W6 = (uint32_t)C6, W7 = (uint32_t)C7;
 };
 
-// r = a + b mod 2p for a, b < 2p (the sum may need 257 bits).
+// r = a + b mod kLazy p for a, b < kLazy p (the sum may need 257 bits).
 template <class F>
 __device__ __forceinline__ void add_lazy(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
-  using P = TwoP<F>;
+  using P = LazyP<F>;
   uint32_t s[8], d[8], c;
   asm("add.cc.u32  %0, %9,  %17;\n\t"
       "addc.cc.u32 %1, %10, %18;\n\t"
@@ -394,15 +399,15 @@ __device__ __forceinline__ void add_lazy(uint32_t r[8], const uint32_t a[8], con
         "+&r"(c)
       : "r"(s[0]), "r"(s[1]), "r"(s[2]), "r"(s[3]), "r"(s[4]), "r"(s[5]), "r"(s[6]), "r"(s[7]), "n"(P::W0),
         "n"(P::W1), "n"(P::W2), "n"(P::W3), "n"(P::W4), "n"(P::W5), "n"(P::W6), "n"(P::W7));
-  // c: all ones when a + b < 2p, zero otherwise
+  // c: all ones when a + b < kLazy p, zero otherwise
 #pragma unroll
   for (int j = 0; j < 8; ++j) r[j] = c ? s[j] : d[j];
 }
 
-// r = a - b mod 2p for a, b < 2p.
+// r = a - b mod kLazy p for a, b < kLazy p.
 template <class F>
 __device__ __forceinline__ void sub_lazy(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) {
-  using P = TwoP<F>;
+  using P = LazyP<F>;
   asm("{\n\t.reg .pred q;\n\t.reg .u32 c;\n\t"
       "sub.cc.u32  %0, %8,  %16;\n\t"
       "subc.cc.u32 %1, %9,  %17;\n\t"
@@ -522,8 +527,8 @@ __device__ __forceinline__ void redc_row_s(uint32_t E[8], uint32_t O[8], uint32_
 // 2^256 mod p: x w = (x_lo A + x_hi B) 2^-128 with the 128-bit halves of x, a
 // sum of 12 words instead of 16, so half of the reduction rows fall away (64 +
 // 32 products instead of 64 + 64; BLS12-381 Fr 64 + 24 instead of 64 + 48).
-// x < 2p; r = x w mod p, left below 2p: (x_lo A + x_hi B + M p) 2^-128 < (1 +
-// 2p 2^-256 + 1) p, which is below 2.4 p for BN254 (one subtraction of p); for
+// x < kLazy p; r = x w mod p, left below kLazy p: (x_lo A + x_hi B + M p) 2^-128
+// < (1 + x 2^-256 + 1) p, which is below 2.57 p for BN254 and x < 3p; for
 // BLS12-381 the subtracted rows give (-p, 1.91 p) (p added to a negative
 // value).  Measured, dependent products: 93 G/s (BLS12-381 Fr) and 88 G/s
 // (BN254 Fr) against 74 and 66 G/s for mont_mul.
@@ -576,10 +581,15 @@ __device__ __forceinline__ void mul_split(uint32_t r[8], const uint32_t x[8], co
           "r"(E[2]), "r"(E[3]), "r"(E[4]), "r"(E[5]), "r"(E[6]), "r"(E[7]));
     add_p_if<F>(r, s);
   } else {
-    uint32_t t[8];
-    pairs_merge(t, O, E);
-    reduce_once<F>(r, t);
+    pairs_merge(r, O, E);
   }
+}
+
+// r = t mod p for t < kLazy p.
+template <class F>
+__device__ __forceinline__ void reduce_lazy(uint32_t r[8], const uint32_t t[8]) {
+  reduce_once<F>(r, t);
+  if constexpr (F::kLazy == 3) reduce_once<F>(r, r);
 }
 
 // ------------------------------------------- warp-cooperative variant

@@ -41,7 +41,8 @@
 // bounds a pass is the IMAD pipe: a butterfly is one mul_split (fp256.cuh; 90
 // or 100 IMAD-pipe instructions of four cycles) beside which additions, shared
 // memory (8 128-bit accesses) and twiddle loads (64 bytes) are issued.
-// Values stay in [0, 2p) from the first butterfly to the last store.
+// Values stay in [0, 2p) or [0, 3p) (fp256.cuh) from the first butterfly to the
+// last store.
 //
 // The tile is XOR-swizzled on 16-byte chunks: chunk 2e + h of element e is
 // stored at (2e + h) ^ swz(e), linear over GF(2) in the bits of e.  For every
@@ -172,10 +173,10 @@ __device__ __forceinline__ uint32_t swz(uint32_t e) {
 }
 
 // What the tile routine asks of a field's elements (this one: 256-bit fields,
-// eight words): their place in the tile, moves, and arithmetic on values in
-// [0, 2p).  `tile` is the tile's shared-memory address, `off` a byte offset that
-// is linear over GF(2) in the bits of the element index; the accesses keep their
-// program order (a thread reads back what it wrote).
+// eight words): their place in the tile, moves, and arithmetic on lazy values.
+// `tile` is the tile's shared-memory address, `off` a byte offset that is linear
+// over GF(2) in the bits of the element index; the accesses keep their program
+// order (a thread reads back what it wrote).
 template <class F>
 struct Elem256 {
   static constexpr int W = 8;
@@ -247,7 +248,7 @@ struct Elem256 {
   __device__ static __forceinline__ void mul_in(uint32_t x[8], const uint32_t w[8]) { mont_mul_lazy<F>(x, w, x); }
   // canonical results
   __device__ static __forceinline__ void mul_out(uint32_t x[8], const uint32_t w[8]) { mont_mul<F>(x, w, x); }
-  __device__ static __forceinline__ void finish(uint32_t x[8]) { reduce_once<F>(x, x); }
+  __device__ static __forceinline__ void finish(uint32_t x[8]) { reduce_lazy<F>(x, x); }
 };
 
 __device__ __forceinline__ void tile_copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
