@@ -41,7 +41,7 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
-// Launch with programmatic stream serialisation (see pdl_wait_and_trigger):
+// Launch with programmatic stream serialisation (see pdl_wait):
 // consecutive passes overlap their launch latency and CTA scheduling.
 template <class K, class... A>
 cudaError_t launch_pdl(K kernel, dim3 grid, dim3 block, int smem, cudaStream_t st, const A &...a) {

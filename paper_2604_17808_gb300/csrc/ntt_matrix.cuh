@@ -520,7 +520,10 @@ __global__ void __launch_bounds__(kMatThreads, 1)
     load_e(tile_q(u_begin));
     e_issued = 1;
   }
-  pdl_wait_and_trigger();
+  // the next pass may start at once (one CTA per SM, whatever its SM): its
+  // barriers, TMEM and E are ready when this one ends
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------ MMA issuer

@@ -516,22 +516,20 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
 // ------------------------------------------------------------ pass kernel
 
 // Programmatic dependent launch (the passes are launched with it): each thread
-// waits here until the previous launch has completed and its memory is visible,
-// and only then lets the next launch start (its CTAs take SM slots as ours
-// retire, and wait in turn).  Triggering before the wait let a whole queue of
-// launches become resident, waiting; each new one was then placed on the few
-// SMs that the oldest had just left (2^17 points: 125 us a transform back to
-// back, 62 us alone).  Without the launch attribute both are no-ops.
-__device__ __forceinline__ void pdl_wait_and_trigger() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// waits here until the previous launch has completed and its memory is visible.
+// No launch is released early (no griddepcontrol.launch_dependents): the next
+// one's CTAs then start as ours retire.  A release at the start let waiting CTAs
+// of the next launches fill the free slots of the SMs, unevenly, so that every
+// launch after ran on few of them: 2^17 points 125 us a transform back to back
+// and 62 alone with the release before this wait, 2^18 points 69 us with it after
+// the wait and 50 without.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class F, int MODE, int MAXT>
 __global__ void __launch_bounds__(MAXT, TileBounds<MAXT>::kMinBlocks)
     ntt_pass_kernel(const __grid_constant__ PassArgs a, const TileShape s, uint32_t tiles) {
   extern __shared__ uint4 smem[];
-  pdl_wait_and_trigger();
+  pdl_wait();
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
   if constexpr (MAXT == 896) {
     const uint32_t group = threadIdx.x / kGroupThreads, tile = blockIdx.x * kGroups + group;

@@ -236,7 +236,7 @@ cudaError_t wide_launch(const PassArgs &a, const TileShape &s, cudaStream_t st) 
   cfg.blockDim = dim3(1u << (s.tl - s.pl));
   cfg.dynamicSmemBytes = (size_t)(4 * F::L) << s.tl;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];   // see pdl_wait_and_trigger
+  cudaLaunchAttribute attr[1];   // see pdl_wait
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;

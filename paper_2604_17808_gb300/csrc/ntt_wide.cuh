@@ -110,7 +110,7 @@ template <class F, int MODE>
 __global__ void __launch_bounds__(WideShape<F>::kThreads, WideShape<F>::kMinBlocks)
     wide_pass_kernel(const __grid_constant__ PassArgs a, const TileShape s) {
   extern __shared__ uint4 wide_smem[];
-  pdl_wait_and_trigger();
+  pdl_wait();
   pass_tile<ElemWide<F>, MODE, false>(a, s, blockIdx.x, (uint32_t)__cvta_generic_to_shared(wide_smem), threadIdx.x, 0);
 }
 
