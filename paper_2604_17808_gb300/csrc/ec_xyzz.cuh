@@ -20,6 +20,7 @@
 
 #include "fp256.cuh"
 #include "fp384.cuh"
+#include "fp_square.cuh"
 
 namespace gb300ntt {
 
@@ -42,6 +43,7 @@ struct FqBn254 {
   __device__ static void add(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) { add_mod<F>(r, a, b); }
   __device__ static void sub(uint32_t r[8], const uint32_t a[8], const uint32_t b[8]) { sub_mod<F>(r, a, b); }
   __device__ static void redc(uint32_t r[8], const uint32_t a[8]) { mont_redc<F>(r, a); }
+  __device__ static void reduce(uint32_t r[8], const uint32_t t[8]) { reduce_once<F>(r, t); }   // t < 2p
   __device__ static bool canonical(const uint32_t a[8]) {
     const uint32_t p[8] = {F::P0, F::P1, F::P2, F::P3, F::P4, F::P5, F::P6, F::P7};
 #pragma unroll
@@ -64,6 +66,7 @@ struct FqBls381 {
   __device__ static void add(uint32_t r[12], const uint32_t a[12], const uint32_t b[12]) { fp384::add_mod(r, a, b); }
   __device__ static void sub(uint32_t r[12], const uint32_t a[12], const uint32_t b[12]) { fp384::sub_mod(r, a, b); }
   __device__ static void redc(uint32_t r[12], const uint32_t a[12]) { fp384::mont_redc(r, a); }
+  __device__ static void reduce(uint32_t r[12], const uint32_t t[12]) { fp384::reduce_once(r, t); }   // t < 2p
   __device__ static bool canonical(const uint32_t a[12]) { return fp384::is_canonical(a); }
   __device__ static constexpr uint32_t modulus(int j) {
     return j == 0 ? F::P0 : j == 1 ? F::P1 : j == 2 ? F::P2 : j == 3 ? F::P3 : j == 4 ? F::P4 : j == 5 ? F::P5
@@ -140,6 +143,37 @@ __device__ __forceinline__ void f_mul(uint32_t r[T::L], const uint32_t a[T::L], 
   }
 }
 
+// r = a^2
+template <class T>
+__device__ __noinline__ FeV<T> f_sqr_call(FeV<T> a) {
+  FeV<T> r;
+  field_square<T>(r.v, a.v);
+  return r;
+}
+
+template <class T, bool kCall>
+__device__ __forceinline__ void f_sqr(uint32_t r[T::L], const uint32_t a[T::L]) {
+  if constexpr (kCall) {
+    FeV<T> x;
+    fv_copy<T::L>(x.v, a);
+    const FeV<T> z = f_sqr_call<T>(x);
+    fv_copy<T::L>(r, z.v);
+  } else {
+    field_square<T>(r, a);
+  }
+}
+
+// r = a b - c d
+template <class T>
+__device__ __forceinline__ void f_mul_sub(uint32_t r[T::L], const uint32_t a[T::L], const uint32_t b[T::L],
+                                          const uint32_t c[T::L], const uint32_t d[T::L]) {
+  uint32_t p[T::L], n[T::L];
+#pragma unroll
+  for (int j = 0; j < T::L; ++j) p[j] = T::modulus(j);
+  words_sub<T::L>(n, p, c);   // p - c, p for c = 0
+  field_mul2<T>(r, a, b, n, d);
+}
+
 template <class T>
 struct Xyzz {
   uint32_t X[T::L], Y[T::L], ZZ[T::L], ZZZ[T::L];
@@ -187,21 +221,19 @@ __device__ __forceinline__ void xyzz_dbl(Xyzz<T> &r, const Xyzz<T> &p) {
   constexpr int L = T::L;
   uint32_t U[L], V[L], W[L], S[L], M[L];
   T::add(U, p.Y, p.Y);            // U = 2 Y1
-  f_mul<T, kCall>(V, U, U);       // V = U^2
+  f_sqr<T, kCall>(V, U);         // V = U^2
   f_mul<T, kCall>(W, U, V);       // W = U V
   f_mul<T, kCall>(S, p.X, V);     // S = X1 V
-  f_mul<T, kCall>(M, p.X, p.X);
+  f_sqr<T, kCall>(M, p.X);
   T::add(U, M, M);
   T::add(M, U, M);                // M = 3 X1^2
   f_mul<T, kCall>(r.ZZ, V, p.ZZ);    // ZZ3 = V ZZ1
   f_mul<T, kCall>(r.ZZZ, W, p.ZZZ);  // ZZZ3 = W ZZZ1
-  f_mul<T, kCall>(W, W, p.Y);        // W Y1
-  f_mul<T, kCall>(U, M, M);
+  f_sqr<T, kCall>(U, M);
   T::sub(U, U, S);
   T::sub(U, U, S);                // X3 = M^2 - 2 S
   T::sub(S, S, U);
-  f_mul<T, kCall>(S, M, S);
-  T::sub(r.Y, S, W);              // Y3 = M (S - X3) - W Y1
+  f_mul_sub<T>(r.Y, M, S, W, p.Y);   // Y3 = M (S - X3) - W Y1
   fv_copy<L>(r.X, U);
 }
 
@@ -227,19 +259,17 @@ __device__ __forceinline__ void xyzz_madd(Xyzz<T> &acc, const uint32_t x2[T::L],
     else xyzz_set_inf(acc);                          // opposite points
     return;
   }
-  f_mul<T, true>(PP, P, P);
+  f_sqr<T, true>(PP, P);
   f_mul<T, true>(PPP, P, PP);
   f_mul<T, true>(acc.ZZ, acc.ZZ, PP);     // ZZ3 = ZZ1 PP
   f_mul<T, true>(acc.ZZZ, acc.ZZZ, PPP);  // ZZZ3 = ZZZ1 PPP
   f_mul<T, true>(Q, acc.X, PP);           // Q = X1 PP
-  f_mul<T, true>(P, R, R);
+  f_sqr<T, true>(P, R);
   T::sub(P, P, PPP);
   T::sub(P, P, Q);
   T::sub(P, P, Q);                        // X3 = R^2 - PPP - 2 Q
   T::sub(Q, Q, P);
-  f_mul<T, true>(Q, R, Q);                // R (Q - X3)
-  f_mul<T, true>(PPP, acc.Y, PPP);
-  T::sub(acc.Y, Q, PPP);                  // Y3 = R (Q - X3) - Y1 PPP
+  f_mul_sub<T>(acc.Y, R, Q, acc.Y, PPP);  // Y3 = R (Q - X3) - Y1 PPP
   fv_copy<L>(acc.X, P);
 }
 
@@ -264,21 +294,19 @@ __device__ __forceinline__ void xyzz_add(Xyzz<T> &acc, const Xyzz<T> &q) {
     else xyzz_set_inf(acc);
     return;
   }
-  f_mul<T, kCall>(PP, P, P);
+  f_sqr<T, kCall>(PP, P);
   f_mul<T, kCall>(PPP, P, PP);
   f_mul<T, kCall>(acc.ZZ, acc.ZZ, q.ZZ);
   f_mul<T, kCall>(acc.ZZ, acc.ZZ, PP);    // ZZ3 = ZZ1 ZZ2 PP
   f_mul<T, kCall>(acc.ZZZ, acc.ZZZ, q.ZZZ);
   f_mul<T, kCall>(acc.ZZZ, acc.ZZZ, PPP); // ZZZ3 = ZZZ1 ZZZ2 PPP
   f_mul<T, kCall>(U1, U1, PP);            // Q = U1 PP
-  f_mul<T, kCall>(P, R, R);
+  f_sqr<T, kCall>(P, R);
   T::sub(P, P, PPP);
   T::sub(P, P, U1);
   T::sub(P, P, U1);                       // X3 = R^2 - PPP - 2 Q
   T::sub(U1, U1, P);
-  f_mul<T, kCall>(U1, R, U1);             // R (Q - X3)
-  f_mul<T, kCall>(S1, S1, PPP);
-  T::sub(acc.Y, U1, S1);                  // Y3 = R (Q - X3) - S1 PPP
+  f_mul_sub<T>(acc.Y, R, U1, S1, PPP);    // Y3 = R (Q - X3) - S1 PPP
   fv_copy<L>(acc.X, P);
 }
 
@@ -486,19 +514,25 @@ __device__ __forceinline__ void quad_pick(uint32_t r[L], bool first, const uint3
   for (int j = 0; j < L; ++j) r[j] = first ? a[j] : b[j];
 }
 
-// v = 2 v (dbl-2008-s-1, a = 0); O stays O.
+// v = 2 v (dbl-2008-s-1, a = 0); O stays O.  On the chain between two products
+// sums are left unreduced where the product allows it: factors a p and b p give
+// a result below 2p while a b < 2^(32 L) / p, which is 9.8 for the 381-bit and
+// 5.2 for the 254-bit field (U < 2p, M < 3p or 2p, S - X3 < 3p or 2p).
 template <class T, bool kCall = true>
 __device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
   constexpr int L = T::L;
+  constexpr bool kWide = T::modulus(L - 1) < 0x1c71c71cu;   // 9 p < 2^(32 L)
+  static_assert(T::modulus(L - 1) < 0x3fffffffu, "4 p < 2^(32 L)");
   const int lane = threadIdx.x & 3;
   uint32_t a[L], b[L], p[L], V[L], M[L], q[L], g[L], h[L];
-  T::add(a, v, v);
+  words_add<L>(a, v, v);
   quad_pick<L>(a, lane == 1, a, v);       // lane 1: U = 2 Y; lane 0: X
-  f_mul<T, kCall>(p, a, a);                // lane 0: X^2, lane 1: V = U^2
+  f_sqr<T, kCall>(p, a);                  // lane 0: X^2, lane 1: V = U^2
   quad_get<L>(V, p, 1);
   quad_get<L>(g, p, 0);
-  T::add(M, g, g);
-  T::add(M, M, g);                        // M = 3 X^2
+  if constexpr (kWide) words_add<L>(M, g, g);
+  else T::add(M, g, g);
+  words_add<L>(M, M, g);                  // M = 3 X^2
   quad_pick<L>(a, lane == 3, M, a);
   quad_pick<L>(a, lane == 2, v, a);
   quad_pick<L>(b, lane == 3, M, V);
@@ -507,7 +541,13 @@ __device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
   uint32_t x3[L];
   T::sub(x3, g, q);
   T::sub(x3, x3, q);                      // lane 0: X3 = M^2 - 2 S
-  T::sub(b, q, x3);                       // lane 0: S - X3
+  T::add(b, q, q);
+  if constexpr (kWide) words_add<L>(b, b, q);
+  else T::add(b, b, q);
+#pragma unroll
+  for (int j = 0; j < L; ++j) a[j] = T::modulus(j);
+  words_sub<L>(a, a, g);
+  words_add<L>(b, b, a);                  // lane 0: S - X3 = 3 S - M^2
   quad_pick<L>(a, lane == 0, M, q);
   quad_pick<L>(a, lane == 3, g, a);
   quad_pick<L>(b, lane == 0, b, v);
