@@ -75,11 +75,16 @@ constexpr int kScanPer = 8;
 constexpr int kScanTile = kScanThreads * kScanPer;
 constexpr int kEcThreads = 128;
 constexpr uint32_t kSignBit = 0x80000000u;
-// A bucket that crosses at most this many segment ends is added up by one
-// thread (or four lanes); longer ones by a tree of radix 4 over their pieces
-// (three additions a level; radix 8 took 154 us instead of the tree's 100 for
-// 1300 pieces of BLS12-381, radix 2 needs twice the launches).
-constexpr uint32_t kShortSpan = 8;
+// A bucket that crosses few segment ends is added up by one thread (or four
+// lanes); longer ones by a tree of radix 4 over their pieces (three additions a
+// level; radix 8 took 154 us instead of the tree's 100 for 1300 pieces of
+// BLS12-381, radix 2 needs twice the launches).  Where the average bucket is
+// shorter than a segment the longer ones are few, the tree runs for the longest
+// anyway, and the limit is the additions of one level (50,000 witness scalars of
+// BLS12-381: 1531 us a call with 3, 1604 with 8).  Where the average bucket
+// crosses several ends nearly all of them do, and one thread for each fills the
+// GPU (BLS12-381 commitment, 2^20 points: 6655 us with 8, 6713 with 3).
+constexpr uint32_t kShortSpan = 3, kShortSpanLongBuckets = 8;
 constexpr uint32_t kSegMask = (1u << 28) - 1u;   // a segment index (span - 1 above it in a crossing item)
 constexpr int kLongLevels = 14;    // 4^14 pieces
 // Tree levels of at most this many nodes per SM take eight lanes per node.
@@ -131,7 +136,7 @@ struct EcConst {
 struct MsmTotals {
   uint32_t entries;                // points placed in buckets (digit != 0)
   uint32_t seg_len;                // S, entries per segment (from the entries there are)
-  uint32_t crossing;               // buckets over 2 .. kShortSpan + 1 segments
+  uint32_t crossing;               // buckets over few segments (short_span)
   uint32_t items[kLongLevels];     // work items of the levels of the long buckets' trees
   uint32_t err;                    // MSM_ERR_* bits
 };
@@ -403,12 +408,16 @@ __device__ __forceinline__ uint32_t list_slot(uint32_t *counter) {
   return __shfl_sync(mask, base, leader) + __popc(mask & ((1u << lane) - 1u));
 }
 
+__device__ __forceinline__ uint32_t short_span(const MsmTotals *tot, uint64_t nb) {
+  return tot->entries >= nb * tot->seg_len ? kShortSpanLongBuckets : kShortSpan;
+}
+
 // Piece i of a bucket over `span` + 1 segments, in segment t: a node of every
 // level l of its tree for which i is a multiple of 4^(l + 1) and i + 4^l <=
 // span.
 __device__ __forceinline__ void push_items(MsmTotals *tot, const CombineLists &lists, uint32_t t, uint32_t i,
-                                           uint32_t span) {
-  if (span <= kShortSpan) return;
+                                           uint32_t span, uint32_t limit) {
+  if (span <= limit) return;
   uint32_t step = 1;
   for (int l = 0; l < kLongLevels && (i & (4 * step - 1)) == 0 && i + step <= span; ++l, step *= 4)
     lists.items[lists.item_base[l] + list_slot(&tot->items[l])] = t | (i == 0 ? kSignBit : 0u);
@@ -423,7 +432,7 @@ __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
   using T = typename C::T;
   constexpr int L = T::L;
   const uint32_t n_entries = tot->entries, S = tot->seg_len;
-  const uint32_t num_segs = (n_entries + S - 1) / S;
+  const uint32_t num_segs = (n_entries + S - 1) / S, limit = short_span(tot, nb);
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < num_segs; t += gridDim.x * blockDim.x) {
     const uint32_t e0 = t * S, e1 = min(e0 + S, n_entries);
     uint32_t b = bucket_of_entry(offsets, nb, e0);
@@ -431,7 +440,7 @@ __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
     bool started_before = __ldg(offsets + b) < e0;
     if (started_before) {
       const uint32_t t0 = __ldg(offsets + b) / S;
-      push_items(tot, lists, t, t - t0, (end_b - 1) / S - t0);
+      push_items(tot, lists, t, t - t0, (end_b - 1) / S - t0, limit);
     }
     Xyzz<T> acc;
     xyzz_set_inf(acc);
@@ -462,8 +471,8 @@ __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
     emit_piece(acc, b, t, started_before, continues, bucket_sum, pieces);
     if (continues && !started_before) {
       const uint32_t span = (end_b - 1) / S - t;  // segments after t that hold bucket b
-      if (span <= kShortSpan) lists.crossing[list_slot(&tot->crossing)] = t | (uint32_t)(span - 1) << 28;
-      else push_items(tot, lists, t, 0, span);
+      if (span <= limit) lists.crossing[list_slot(&tot->crossing)] = t | (uint32_t)(span - 1) << 28;
+      else push_items(tot, lists, t, 0, span, limit);
     }
   }
 }
@@ -1052,12 +1061,13 @@ uint32_t segment_length(uint64_t max_n, uint32_t K, int sms, int blocks_per_sm) 
 }
 
 // Item list bases: level l of the long trees has at most segments / 4^(l + 1)
-// + one head per bucket; a long bucket covers more than kShortSpan segments.
+// + one head per bucket; a bucket with a node there crosses more than kShortSpan
+// segment ends, and 4^l at least.
 uint64_t item_bases(uint64_t segments, uint32_t base[kLongLevels]) {
   uint64_t total = 0, per = 4;
   for (int l = 0; l < kLongLevels; ++l) {
     base[l] = (uint32_t)total;
-    total += segments / per + segments / kShortSpan + 1;
+    total += segments / per + segments / std::max<uint64_t>(kShortSpan, per / 4) + 1;
     per *= 4;
   }
   return total;
