@@ -400,27 +400,21 @@ __device__ __forceinline__ void emit_piece(const Xyzz<T> &acc, uint32_t b, uint3
   else store_point_xyzz(pieces, 2 * (uint64_t)t + 1, acc);
 }
 
-// The next free index of a list: one atomic for the lanes that are here.
-__device__ __forceinline__ uint32_t list_slot(uint32_t *counter) {
-  const uint32_t mask = __activemask(), lane = threadIdx.x & 31u, leader = __ffs(mask) - 1;
-  uint32_t base = 0;
-  if (lane == leader) base = atomicAdd(counter, (uint32_t)__popc(mask));
-  return __shfl_sync(mask, base, leader) + __popc(mask & ((1u << lane) - 1u));
-}
-
 __device__ __forceinline__ uint32_t short_span(const MsmTotals *tot, uint64_t nb) {
   return tot->entries >= nb * tot->seg_len ? kShortSpanLongBuckets : kShortSpan;
 }
 
 // Piece i of a bucket over `span` + 1 segments, in segment t: a node of every
 // level l of its tree for which i is a multiple of 4^(l + 1) and i + 4^l <=
-// span.
+// span.  One atomic per item: the lanes of a warp that are here together may be
+// at different levels, so that one atomic for all of them would take a slot of
+// one level's list for an item of another's.
 __device__ __forceinline__ void push_items(MsmTotals *tot, const CombineLists &lists, uint32_t t, uint32_t i,
                                            uint32_t span, uint32_t limit) {
   if (span <= limit) return;
   uint32_t step = 1;
   for (int l = 0; l < kLongLevels && (i & (4 * step - 1)) == 0 && i + step <= span; ++l, step *= 4)
-    lists.items[lists.item_base[l] + list_slot(&tot->items[l])] = t | (i == 0 ? kSignBit : 0u);
+    lists.items[lists.item_base[l] + atomicAdd(&tot->items[l], 1u)] = t | (i == 0 ? kSignBit : 0u);
 }
 
 // BA: segment t adds the points of sorted entries [t S, t S + S).
@@ -471,7 +465,7 @@ __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
     emit_piece(acc, b, t, started_before, continues, bucket_sum, pieces);
     if (continues && !started_before) {
       const uint32_t span = (end_b - 1) / S - t;  // segments after t that hold bucket b
-      if (span <= limit) lists.crossing[list_slot(&tot->crossing)] = t | (uint32_t)(span - 1) << 28;
+      if (span <= limit) lists.crossing[atomicAdd(&tot->crossing, 1u)] = t | (uint32_t)(span - 1) << 28;
       else push_items(tot, lists, t, 0, span, limit);
     }
   }
