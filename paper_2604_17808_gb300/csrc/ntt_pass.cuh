@@ -107,9 +107,6 @@ constexpr int kMaxPasses = 12;
 struct PassArgs {
   const uint4 *src;      // input elements (2 x uint4 each)
   uint4 *dst;            // output elements
-  uint4 *dst2;           // a second place for the outputs, or nullptr (host buffer of a
-                         // host-to-host transform: last pass only)
-  uint32_t src_host;     // first pass: src is host memory
   const uint4 *mul;      // input multipliers (Montgomery form) or nullptr
   const uint4 *dft_tw;   // omega_S^i, i < S/2, 64 bytes each: the residues A, B of mul_split
   const uint4 *post;     // output multipliers indexed by output position, or nullptr
@@ -227,9 +224,6 @@ struct Elem256 {
   __device__ static __forceinline__ void load(uint32_t r[8], const uint4 *base, uint64_t e) {
     fe_load_global(r, base, e);
   }
-  __device__ static __forceinline__ void load_coherent(uint32_t r[8], const uint4 *base, uint64_t e) {
-    fe_load_global_cg(r, base, e);
-  }
   __device__ static __forceinline__ void store(uint4 *base, uint64_t e, const uint32_t a[8]) {
     fe_store_global(base, e, a);
   }
@@ -330,7 +324,6 @@ __device__ __forceinline__ void store_output(const PassArgs &a, uint64_t pos, ui
     El::finish(x);
   }
   El::store(a.dst, pos, x);
-  if (a.dst2) El::store(a.dst2, pos, x);
 }
 
 // Global position of element n of sub-transform d (pass input; the in-place
@@ -372,23 +365,6 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     const bool linear = r == pl;
     auto sub_of = [&](uint32_t j) { return dfirst + ((uint64_t)(j >> r) << gbits); };
     uint64_t pos = elem_pos<MODE>(a, logs, dfirst, low);
-    if (MODE != kModeInner && El::W == 8 && linear && a.src_host) {
-      // whole elements over the bus, four on their way at a time (copies in
-      // 16-byte halves ask for every 32-byte sector twice)
-      if (dfirst < a.num_sub && dbg_in(a, pos + (count - 1) * step, a.n_vec)) {
-#pragma unroll 1
-        for (uint32_t j = 0; j < count; j += 4) {
-          uint32_t x[4][El::W];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (j + i < count) El::load_coherent(x[i], a.src, pos + i * step);
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (j + i < count) El::tile_store(smem, private_offset(v, j + i), s.tl, x[i]);
-          pos += 4 * step;
-        }
-      }
-    } else
 #pragma unroll 1
     for (uint32_t j = 0; j < count; ++j, pos += step) {
       const uint64_t d = linear ? dfirst : sub_of(j);

@@ -316,22 +316,8 @@ TileShape batch_shape(uint64_t elements, uint32_t logs, uint32_t tile_log, int s
   return TileShape{logs, 10, 3};
 }
 
-// Tile of a pass that reads or writes host memory.  From 2^18 points on the bus
-// is the bound (2^18: 42 us each way) and tiles hold two sub-transforms at least,
-// for requests of 64 bytes (measured, 8 MiB: 57 / 64 us for reads / writes of 32
-// bytes, 47 / 53 of 64, 45 / 47 of 128 and of a copy engine; whole transforms:
-// 2^18 150 us against 165, 2^20 473 against 610).  Below, the shapes of the device
-// transform are faster (2^16: 55 us against 70).
-TileShape host_shape(ntt_plan p, uint32_t logs, uint32_t tl) {
-  if (p->log_n < 18) return pass_shape(p, logs, tl);
-  return TileShape{logs, logs < 10 ? 10u : 11u, 3};
-}
-
-// Enqueue one transform: one kernel launch per pass.  With host_in the first
-// pass reads `in` from host memory, with out2 the last one also writes its
-// outputs there (host memory, device addresses).
-ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st, bool host_in,
-                             void *out2) {
+// Enqueue one transform: one kernel launch per pass.
+ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st) {
   const FieldLaunchers &L = launchers(p->field);
   const bool shrink = p->debug_shrink;   // debug-build test hook (see ntt_debug_shrink_next_extent)
   p->debug_shrink = false;
@@ -340,51 +326,13 @@ ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cu
     int mode;
     build_pass_args(p, kind, in, out, j, &a, &mode);
     if (shrink) a.n_vec >>= 1;
-    const bool to_host = out2 && j == p->num_passes - 1;
-    if (to_host) a.dst2 = (uint4 *)out2;
-    a.src_host = host_in && j == 0;
     const uint32_t logs = p->pass_log[j];
     cudaError_t e = timing_begin(p, (int)j, st);
-    const TileShape shape =
-        to_host || (host_in && j == 0) ? host_shape(p, logs, p->pass_tl[j]) : pass_shape(p, logs, p->pass_tl[j]);
+    const TileShape shape = pass_shape(p, logs, p->pass_tl[j]);
     if (e == cudaSuccess) e = L.pass(mode, shape, a, pass_tiles(p->log_n, logs, shape.tl), p->sm_count, st);
     if (e == cudaSuccess) e = timing_end(p, st);
     if (e != cudaSuccess) return cuda_status(e);
   }
-  return NTT_OK;
-}
-
-// The device address of a page-locked, mapped host buffer whose elements the
-// kernels can move with 256-bit accesses, or nullptr (pageable, misaligned, or
-// locked in part: copied instead).
-static void *mapped_host(const void *h, size_t bytes) {
-  if ((uintptr_t)h % 32) return nullptr;
-  cudaPointerAttributes first, last;
-  if (cudaPointerGetAttributes(&first, h) != cudaSuccess ||
-      cudaPointerGetAttributes(&last, (const char *)h + bytes - 1) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer) return nullptr;
-  if ((char *)last.devicePointer != (char *)first.devicePointer + bytes - 1) return nullptr;
-  if ((uintptr_t)first.devicePointer % 32) return nullptr;
-  return first.devicePointer;
-}
-
-// Host buffers in and out by way of d_work, on `st`.  The butterfly passes read
-// page-locked input and write page-locked output themselves, so the transfers
-// overlap the first and the last pass (copies on both sides -> this, us: 2^12 30 ->
-// 24, 2^16 70 -> 55, 2^18 174 -> 150, 2^21 1110 -> 868).
-static ntt_status enqueue_host_transform(ntt_plan plan, ntt_kind kind, const void *h_in, void *h_out, void *d_work,
-                                         cudaStream_t st) {
-  if (!kind_is_valid((int)kind, plan->has_coset)) return NTT_ERR_INVALID_ARG;
-  const size_t bytes = (size_t)32 << plan->log_n;
-  const bool direct = plan->path != NTT_PATH_MATRIX;
-  void *in = direct ? mapped_host(h_in, bytes) : nullptr, *out = direct ? mapped_host(h_out, bytes) : nullptr;
-  if (!in) NTT_CUDA(cudaMemcpyAsync(d_work, h_in, bytes, cudaMemcpyHostToDevice, st));
-  if (direct) NTT_TRY(enqueue_transform(plan, (int)kind, in ? in : d_work, d_work, st, in != nullptr, out));
-  else NTT_TRY(ntt_execute(plan, kind, d_work, d_work, (ntt_stream)st));
-  if (!out) NTT_CUDA(cudaMemcpyAsync(h_out, d_work, bytes, cudaMemcpyDeviceToHost, st));
   return NTT_OK;
 }
 
@@ -518,7 +466,7 @@ ntt_status ntt_execute(ntt_plan plan, ntt_kind kind, const void *d_in, void *d_o
   NTT_TRY(check_buffer(d_in));
   NTT_TRY(check_buffer(d_out));
   if (plan->path == NTT_PATH_MATRIX) return enqueue_matrix_transform(plan, (int)kind, d_in, d_out, (cudaStream_t)stream);
-  return enqueue_transform(plan, (int)kind, d_in, d_out, (cudaStream_t)stream, false, nullptr);
+  return enqueue_transform(plan, (int)kind, d_in, d_out, (cudaStream_t)stream);
 }
 
 ntt_status ntt_forward(ntt_plan plan, const void *d_in, void *d_out, ntt_stream stream) {
@@ -538,8 +486,11 @@ ntt_status ntt_transform_host(ntt_plan plan, ntt_kind kind, const void *h_in, vo
                               ntt_stream stream) {
   if (!plan || !h_in || !h_out) return NTT_ERR_INVALID_ARG;
   NTT_TRY(check_buffer(d_work));
+  const size_t bytes = (size_t)32 << plan->log_n;
   cudaStream_t st = (cudaStream_t)stream;
-  NTT_TRY(enqueue_host_transform(plan, kind, h_in, h_out, d_work, st));
+  NTT_CUDA(cudaMemcpyAsync(d_work, h_in, bytes, cudaMemcpyHostToDevice, st));
+  NTT_TRY(ntt_execute(plan, kind, d_work, d_work, stream));
+  NTT_CUDA(cudaMemcpyAsync(h_out, d_work, bytes, cudaMemcpyDeviceToHost, st));
   NTT_CUDA(cudaStreamSynchronize(st));
   return NTT_OK;
 }
@@ -548,7 +499,12 @@ ntt_status ntt_transform_host_async(ntt_plan plan, ntt_kind kind, const void *h_
                                     ntt_stream stream) {
   if (!plan || !h_in || !h_out) return NTT_ERR_INVALID_ARG;
   NTT_TRY(check_buffer(d_work));
-  return enqueue_host_transform(plan, kind, h_in, h_out, d_work, (cudaStream_t)stream);
+  const size_t bytes = (size_t)32 << plan->log_n;
+  cudaStream_t st = (cudaStream_t)stream;
+  NTT_CUDA(cudaMemcpyAsync(d_work, h_in, bytes, cudaMemcpyHostToDevice, st));
+  NTT_TRY(ntt_execute(plan, kind, d_work, d_work, stream));
+  NTT_CUDA(cudaMemcpyAsync(h_out, d_work, bytes, cudaMemcpyDeviceToHost, st));
+  return NTT_OK;
 }
 
 ntt_status ntt_plan_describe(ntt_plan plan, ntt_plan_desc *out) {

@@ -87,8 +87,7 @@ std::vector<uint32_t> split_passes_max(uint32_t log_n, uint32_t max_log);
 // has_coset, sm_count set) for the given pass split (nullptr = default).
 ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *forced_split);
 uint64_t pass_tiles(uint32_t log_n, uint32_t logs, uint32_t tl);
-ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st, bool host_in = false,
-                             void *out2 = nullptr);
+ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st);
 ntt_status cuda_status(cudaError_t e);
 struct PassArgs;
 void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j, PassArgs *a, int *mode);

@@ -81,7 +81,6 @@ struct ElemWide {
       r[4 * k] = v.x; r[4 * k + 1] = v.y; r[4 * k + 2] = v.z; r[4 * k + 3] = v.w;
     }
   }
-  __device__ static __forceinline__ void load_coherent(uint32_t *r, const uint4 *base, uint64_t e) { load(r, base, e); }
   __device__ static __forceinline__ void store(uint4 *base, uint64_t e, const uint32_t *a) {
 #pragma unroll
     for (int k = 0; k < W / 4; ++k)
