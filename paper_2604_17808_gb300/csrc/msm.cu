@@ -36,9 +36,14 @@
 //                                      B_b = 2 (B_2b + B_2b+1); the leaves
 //                                      start at W_j = B_j, so the root holds
 //                                      sum_j (j + 1) B_j
+//                msm_reduce_chunk_kernel  its lowest levels at once where there
+//                                      are many buckets
+//                msm_reduce_level_quad_kernel  levels of few nodes: four lanes
+//                                      for a W, four for a B
 //   WM           msm_merge_kernel      Horner over the windows, top one first
-//                                      (MSM = 2^c MSM + W_k), then the affine
-//                                      standard-form result.
+//                                      (MSM = 2^c MSM + W_k), four lanes per
+//                                      point, then the affine standard-form
+//                                      result.
 //
 // The paper streams the sorted points straight into bucket accumulation on
 // the TPU; here the sort moves 4-byte point indices and the accumulation

@@ -20,9 +20,9 @@
 // After the last pass the buffer holds X in natural order.  Coset and
 // inverse scale factors are folded into the same per-element multipliers.
 //
-// Work split on the GPU: a group of threads owns a tile of 2^tl elements in shared memory
-// = 2^(tl - logs) sub-transforms with consecutive sub-transform index, and
-// each thread 2^pl of its elements at a time.  The DIF (Gentleman-Sande)
+// Work split on the GPU: a group of threads owns a tile of 2^tl elements in
+// shared memory = 2^(tl - logs) sub-transforms with consecutive sub-transform
+// index, and each thread 2^pl of its elements at a time.  The DIF (Gentleman-Sande)
 // radix-2 network over every sub-transform of the tile runs in rounds of up to
 // pl stages: in a round a thread owns the 2^pl elements that differ in the
 // round's index bits, so its stages need no barrier between them; barriers

@@ -104,7 +104,7 @@ uint64_t pass_tiles(uint32_t log_n, uint32_t logs, uint32_t tl) {
   return (num_sub + g - 1) / g;
 }
 
-// Default tile shape of a pass: the 1024-element tile (7 CTAs per SM) when
+// Largest default tile of a pass: 1024 elements (6 CTAs per SM, 32 KiB each) when
 // the sub-transform fits in it, else the 2048-element tile.
 uint32_t default_tile_log(uint32_t logs) { return logs <= 10 ? 10 : 11; }
 

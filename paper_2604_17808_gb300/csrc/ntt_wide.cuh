@@ -9,10 +9,10 @@
 // x c.
 //
 // Tile: 2^10 (377) or 2^9 (753) elements, 48 KiB, up to 8 elements per thread,
-// 4 CTAs of 128 (377) or 64 threads (753: 200 registers each) per SM.  The 16-byte chunks of an element lie one
-// tile length apart; within a chunk row the elements are XOR-swizzled by the
-// same columns as the 256-bit tile, so eight consecutive lanes never meet in a
-// bank.
+// 4 CTAs of 128 (377) or 64 threads (753: 200 registers each) per SM.  The
+// 16-byte chunks of an element lie one tile length apart; within a chunk row the
+// elements are XOR-swizzled by the same columns as the 256-bit tile, so eight
+// consecutive lanes never meet in a bank.
 //
 // Multipliers: the first pass's table (mode kModeFirstPre) is indexed by
 // the input position (the coset factors s^i, or N^-1 for a one-pass
