@@ -33,8 +33,8 @@ def _case(name, n, r):
 
 @pytest.mark.parametrize("curve", ["bn254_g1", "bls12_381_g1"])
 @pytest.mark.parametrize("name", ["constant", "cancel", "sparse", "bits", "repeated"])
-@pytest.mark.parametrize("n,flat", [(9, False), (300, True), (20_000, False), (20_000, True), (90_001, False),
-                                    (90_001, True)])
+@pytest.mark.parametrize("n,flat", [(9, False), (60, False), (300, True), (20_000, False), (20_000, True),
+                                    (90_001, False), (90_001, True)])
 def test_pieces(curve, name, n, flat):
     import paper_2604_17808_gb300 as lib
 
