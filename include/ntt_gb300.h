@@ -38,7 +38,11 @@
  * (in != out) on one plan may run concurrently on several streams.  In-place
  * transforms (in == out) with more than one pass use the plan's scratch
  * vector, so concurrent in-place transforms on one plan race: order them on
- * one stream or use one plan per stream.
+ * one stream or use one plan per stream.  Up to 2^10 points an in-place
+ * transform is one pass and does not use the scratch, whatever the number of
+ * passes out of place, unless ntt_plan_set_passes or the autotuner chose the
+ * plan's passes.  ntt_transform_host and ntt_transform_host_async transform
+ * in place.
  *
  * Errors: every call returns an ntt_status; NTT_ERR_INVALID_ARG for a NULL
  * plan or buffer, a misaligned buffer or an unknown enum value;
@@ -165,7 +169,8 @@ ntt_status ntt_transform_host(ntt_plan plan, ntt_kind kind, const void *h_in, vo
  * and returns without synchronising.  h_in, h_out and d_work must stay
  * valid (and h_in unmodified) until the stream has passed this work; with
  * page-locked host buffers, transforms on different streams overlap their
- * copies with each other's kernels.
+ * copies with each other's kernels (one plan per stream: the transform is in
+ * place, see Concurrency above).
  */
 ntt_status ntt_transform_host_async(ntt_plan plan, ntt_kind kind, const void *h_in, void *h_out, void *d_work,
                                     ntt_stream stream);
@@ -174,7 +179,7 @@ ntt_status ntt_transform_host_async(ntt_plan plan, ntt_kind kind, const void *h_
  * Read back the plan's structure: number of passes and the log2 size of each
  * pass's sub-transforms (of the path selected: on the matrix path its own
  * split into passes of at most 2^3 points), the number of kernel launches one
- * transform makes and, on the matrix path, how many of its passes
+ * out-of-place transform makes and, on the matrix path, how many of its passes
  * (passes 1 .. matrix_folded_passes) take their input factors folded into
  * per-q byte matrices (so that the pass before them ends in a Barrett
  * reduction instead of a Montgomery product).

@@ -140,6 +140,8 @@ void release_plan_tables(ntt_plan p) {
   std::memset(p->tw, 0, sizeof p->tw);
   std::memset(p->pre, 0, sizeof p->pre);
   std::memset(p->fac_coset, 0, sizeof p->fac_coset);
+  std::memset(p->pre_one, 0, sizeof p->pre_one);
+  p->in_place_one = false;
   p->post_coset_inv = nullptr;
   p->scratch = nullptr;
 }
@@ -176,6 +178,10 @@ ntt_status build_coset_tables(ntt_plan p, const U256 &s, cudaStream_t st) {
       NTT_CUDA(L.gen_2d(p->tw[kCoset][j], logs, log_mp, make_ladder(F, w), p->fac_coset[j], one, st));
     }
   }
+  if (p->in_place_one) {
+    if (!p->pre_one[kCoset]) NTT_TRY(alloc_tab(p, &p->pre_one[kCoset], 1ull << log_n));
+    NTT_CUDA(L.gen_1d(p->pre_one[kCoset], 1ull << log_n, make_ladder(F, s), one, st));
+  }
   // coset inverse: x_n *= s^-n on the output of the last pass
   if (!p->post_coset_inv) NTT_TRY(alloc_tab(p, &p->post_coset_inv, 1ull << log_n));
   NTT_CUDA(L.gen_1d(p->post_coset_inv, 1ull << log_n, make_ladder(F, F.inv(s)), one, st));
@@ -195,6 +201,11 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
     p->pass_tl[j] = default_tile_log(passes[j]);
   }
   const uint32_t P = p->num_passes;
+  // A default plan whose vector fits one CTA's tile does not need the scratch in
+  // place, so that such calls on several streams do not meet in it: one pass
+  // over the whole vector.  2^9 and 2^10 points, us, one pass against two through
+  // the scratch: 9.8 against 9.1 and 15.1 against 9.9.
+  p->in_place_one = !forced_split && P > 1 && log_n <= kDefaultPassLog;
 
   p->omega = F.root_of_unity(log_n);
   p->omega_inv = F.inv(p->omega);
@@ -203,8 +214,8 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
   const Fe32 n_inv_m = to_fe32(F.to_mont(n_inv));
 
   // DFT twiddles per distinct pass size
-  for (uint32_t j = 0; j < P; ++j) {
-    const uint32_t logs = passes[j];
+  for (uint32_t j = 0; j < P + (p->in_place_one ? 1 : 0); ++j) {
+    const uint32_t logs = j < P ? passes[j] : log_n;
     for (int dir = 0; dir < 2; ++dir) {
       if (p->dft_tw[dir][logs]) continue;
       const U256 w = square_times(F, dir ? p->omega_inv : p->omega, log_n - logs);
@@ -231,21 +242,29 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
     NTT_TRY(alloc_tab(p, &p->pre[kInverse], 1ull << passes[0]));
     NTT_CUDA(L.gen_1d(p->pre[kInverse], 1ull << passes[0], make_ladder(F, u256(1)), n_inv_m, st));
   }
+  if (p->in_place_one) {
+    NTT_TRY(alloc_tab(p, &p->pre_one[kInverse], 1ull << log_n));
+    NTT_CUDA(L.gen_1d(p->pre_one[kInverse], 1ull << log_n, make_ladder(F, u256(1)), n_inv_m, st));
+  }
   if (p->has_coset) NTT_TRY(build_coset_tables(p, F.reduce_small(F.generator), st));
-  if (P > 1) NTT_TRY(alloc_tab(p, &p->scratch, 1ull << log_n));
+  if (P > 1 && !p->in_place_one) NTT_TRY(alloc_tab(p, &p->scratch, 1ull << log_n));
   p->launches = P;
   return NTT_OK;
 }
+
+// Whether a call runs as the plan's single in-place pass.
+static bool runs_one_pass(ntt_plan p, const void *in, const void *out) { return in == out && p->in_place_one; }
 
 // Arguments of pass j of one transform: pass 0 reads `in`; every later pass
 // works in place on `work` (out, or the plan's scratch for in-place calls);
 // the last pass writes `out`.
 void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j, PassArgs *a, int *mode) {
-  const uint32_t P = p->num_passes, log_n = p->log_n;
+  const bool one = runs_one_pass(p, in, out);
+  const uint32_t P = one ? 1 : p->num_passes, log_n = p->log_n;
   const int tk = table_kind(kind);
   const int dir = tk == kInverse ? 1 : 0;
   uint4 *work = (P > 1 && in == out) ? p->scratch : (uint4 *)out;
-  const uint32_t logs = p->pass_log[j];
+  const uint32_t logs = one ? log_n : p->pass_log[j];
   *a = PassArgs{};
   a->dft_tw = p->dft_tw[dir][logs];
   a->num_sub = 1ull << (log_n - logs);
@@ -260,7 +279,7 @@ void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j
       a->digit_shift[d - 1] = (uint8_t)shift;
       shift += p->pass_log[d];
     }
-    a->mul = p->pre[tk];
+    a->mul = one ? p->pre_one[tk] : p->pre[tk];
     *mode = a->mul ? kModeFirstPre : kModeFirst;
   } else {
     uint32_t log_mp = 0;
@@ -288,13 +307,16 @@ void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j
 // over as many warps as there are and its serial chain is short: 2 up to 2^18
 // points, 4 at 2^19, 8 from 2^20 on (and for sub-transforms of 2^9 and 2^10
 // points 4 and 8).  Tiles of the small shapes hold one sub-transform (at least
-// one warp).
+// one warp).  A sub-transform that is the whole transform has a single CTA,
+// which then gets 256 threads (2^10 points: 15.1 us against 20.0 with 128, and
+// 17.0 with 512; 2^9: 9.8 against 10.4).
 TileShape pass_shape(ntt_plan p, uint32_t logs, uint32_t tl) {
   if (tl != 10) return TileShape{logs, tl, 3};
   const uint64_t slots = (uint64_t)p->sm_count * kGroupThreads * kGroups;
+  const uint32_t max_threads_log = logs == p->log_n ? 8 : 7;
   for (uint32_t pl = 1; pl < 3; ++pl) {
     const uint32_t t = std::max(logs, pl + 5);
-    if (t - pl <= 7 && (1ull << p->log_n) >> pl <= slots) return TileShape{logs, t, pl};
+    if (t - pl <= max_threads_log && (1ull << p->log_n) >> pl <= slots) return TileShape{logs, t, pl};
   }
   return TileShape{logs, tl, 3};
 }
@@ -321,14 +343,15 @@ ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cu
   const FieldLaunchers &L = launchers(p->field);
   const bool shrink = p->debug_shrink;   // debug-build test hook (see ntt_debug_shrink_next_extent)
   p->debug_shrink = false;
-  for (uint32_t j = 0; j < p->num_passes; ++j) {
+  const bool one = runs_one_pass(p, in, out);
+  for (uint32_t j = 0; j < (one ? 1 : p->num_passes); ++j) {
     PassArgs a;
     int mode;
     build_pass_args(p, kind, in, out, j, &a, &mode);
     if (shrink) a.n_vec >>= 1;
-    const uint32_t logs = p->pass_log[j];
+    const uint32_t logs = one ? p->log_n : p->pass_log[j];
     cudaError_t e = timing_begin(p, (int)j, st);
-    const TileShape shape = pass_shape(p, logs, p->pass_tl[j]);
+    const TileShape shape = pass_shape(p, logs, one ? default_tile_log(logs) : p->pass_tl[j]);
     if (e == cudaSuccess) e = L.pass(mode, shape, a, pass_tiles(p->log_n, logs, shape.tl), p->sm_count, st);
     if (e == cudaSuccess) e = timing_end(p, st);
     if (e != cudaSuccess) return cuda_status(e);

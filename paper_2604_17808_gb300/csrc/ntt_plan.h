@@ -46,6 +46,10 @@ struct ntt_plan_s {
   uint4 *fac_coset[gb300ntt::kMaxPasses] = {};  // [pass >= 1]: s^(n N / M_j), n < S_j
   uint4 *post_coset_inv = nullptr;  // s^-n, n < N: output multipliers of the coset inverse
   uint4 *scratch = nullptr;      // N elements (in-place transforms with > 1 pass)
+  // in-place transforms run as one pass, without the scratch, although the plan
+  // has more (see build_plan); its pass-0 multipliers [N] by kind
+  bool in_place_one = false;
+  uint4 *pre_one[3] = {};
   uint32_t *d_err = nullptr;     // device error word
   bool debug_shrink = false;     // debug builds: next transform with its vector extent halved
   std::vector<void *> allocations;
