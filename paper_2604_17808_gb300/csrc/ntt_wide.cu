@@ -101,13 +101,15 @@ std::map<std::tuple<int, int, uint32_t>, WidePlan *> g_wide_plans;   // (device,
 
 ntt_status cuda_w(cudaError_t e) { return cuda_status(e); }
 
+// A table of the transform size 2^log_n from the constants in kbuf, which hold
+// omega_N^(2^b): the powers of omega_M, M = 2^log_m, are those from b = log_n -
+// log_m on.
 template <class F>
-ntt_status gen_table(uint4 *out, uint32_t log_m, int dir, bool use_m_inv, uint32_t log_mp, uint64_t count, int two_d,
-                     bool constant, bool split, uint32_t *kbuf, cudaStream_t st) {
+ntt_status gen_table(uint4 *out, uint32_t log_n, uint32_t log_m, int dir, bool use_n_inv, uint32_t log_mp,
+                     uint64_t count, int two_d, bool constant, bool split, const uint32_t *kbuf, cudaStream_t st) {
   constexpr int L = F::L;
-  wide_constants_kernel<F><<<1, 1, 0, st>>>(kbuf, log_m, wide_const<F>());
-  const uint32_t *ladder = constant ? nullptr : kbuf + (dir ? 32 : 0) * L;
-  const uint32_t *init = kbuf + (use_m_inv ? 64 : 65) * L;
+  const uint32_t *ladder = constant ? nullptr : kbuf + ((dir ? 32 : 0) + log_n - log_m) * L;
+  const uint32_t *init = kbuf + (use_n_inv ? 64 : 65) * L;
   uint64_t blocks = (count + 255) / 256;
   if (blocks > 152ull * 32) blocks = 152ull * 32;
   wide_table_kernel<F><<<(unsigned)(blocks ? blocks : 1), 256, 0, st>>>(out, log_mp, ladder, init, count, two_d,
@@ -149,13 +151,16 @@ ntt_status build_wide(uint32_t log_n, WidePlan *w) {
   w->allocs.push_back(kbuf);
   w->kbuf = kbuf;
   cudaStream_t st = nullptr;
+  // once for the size: one thread, 0.3 ms (377 bits) or 4.2 ms (753)
+  wide_constants_kernel<F><<<1, 1, 0, st>>>(kbuf, log_n, wide_const<F>());
+  NTT_TRY_W(cuda_w(cudaGetLastError()));
   for (uint32_t j = 0; j < P; ++j) {
     const uint32_t logs = w->pass_log[j];
     for (int dir = 0; dir < 2; ++dir) {
       if (w->dft_tw[dir][logs]) continue;
       const uint64_t cnt = logs ? (1ull << (logs - 1)) : 1;
       NTT_TRY_W(alloc_w(w, &w->dft_tw[dir][logs], cnt * 2 * eb));
-      NTT_TRY_W(gen_table<F>(w->dft_tw[dir][logs], logs, dir, false, 0, cnt, 0, false, true, kbuf, st));
+      NTT_TRY_W(gen_table<F>(w->dft_tw[dir][logs], log_n, logs, dir, false, 0, cnt, 0, false, true, kbuf, st));
     }
   }
   uint32_t log_m = w->pass_log[0];
@@ -164,13 +169,13 @@ ntt_status build_wide(uint32_t log_n, WidePlan *w) {
     log_m += logs;
     for (int dir = 0; dir < 2; ++dir) {
       NTT_TRY_W(alloc_w(w, &w->tw[dir][j], (1ull << log_m) * eb));
-      NTT_TRY_W(gen_table<F>(w->tw[dir][j], log_m, dir, dir == 1 && j == P - 1, log_mp, 1ull << log_m, 1, false, false,
-                             kbuf, st));
+      NTT_TRY_W(gen_table<F>(w->tw[dir][j], log_n, log_m, dir, dir == 1 && j == P - 1, log_mp, 1ull << log_m, 1, false,
+                             false, kbuf, st));
     }
   }
   if (P == 1) {   // single-pass inverse: N^-1 as the pass-0 multiplier
     NTT_TRY_W(alloc_w(w, &w->pre_inv, (1ull << log_n) * eb));
-    NTT_TRY_W(gen_table<F>(w->pre_inv, log_n, 0, true, 0, 1ull << log_n, 0, true, false, kbuf, st));
+    NTT_TRY_W(gen_table<F>(w->pre_inv, log_n, log_n, 0, true, 0, 1ull << log_n, 0, true, false, kbuf, st));
   }
   if (P > 1) NTT_TRY_W(alloc_w(w, &w->scratch, (1ull << log_n) * eb));
   return cuda_w(cudaDeviceSynchronize());
