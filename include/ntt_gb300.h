@@ -494,7 +494,8 @@ ntt_status ntt_pointwise_quotient(ntt_field field, const void *d_a, const void *
  * both synchronous, kept until the process exits.  Stream-ordered.  The
  * tables and an in-place call's scratch vector belong to the (device,
  * field, log_n), not to the caller: two in-place calls of the same field
- * and size must not run at the same time on different streams.
+ * and size must not run at the same time on different streams (up to 2^10
+ * points at 377 bits and 2^9 at 753 they may: no scratch is used there).
  * NTT_ERR_INVALID_ARG for another field or kind, or unaligned or null
  * buffers; NTT_ERR_UNSUPPORTED for other sizes.
  */
