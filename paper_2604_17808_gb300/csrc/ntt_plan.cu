@@ -47,10 +47,14 @@ Fe32 to_fe32(const U256 &a) {
 
 U256 from_limbs(const uint64_t *l) { return U256{{l[0], l[1], l[2], l[3]}}; }
 
-Pow2Table make_ladder(const HostField &F, const U256 &base) {
-  Pow2Table t;
+// base^(2^i) for the exponents of a table, which are below 2^bits.  (The host's
+// products are much of what creating a small plan takes: 2^9 points 4.4 ms with
+// 32 powers for every table and a full exponentiation for every pass's coset
+// step, 3.0 without.)
+Pow2Table make_ladder(const HostField &F, const U256 &base, uint32_t bits) {
+  Pow2Table t{};
   U256 b = base;
-  for (int i = 0; i < 32; ++i) {
+  for (uint32_t i = 0; i < bits; ++i) {
     t.v[i] = to_fe32(F.to_mont(b));
     b = F.mul(b, b);
   }
@@ -165,26 +169,26 @@ ntt_status build_coset_tables(ntt_plan p, const U256 &s, cudaStream_t st) {
     const uint32_t logs = p->pass_log[j];
     log_m += logs;
     // s^(N/M_j): the coset factor of one step of digit j
-    const U256 step = F.pow(s, 1ull << (log_n - log_m));
+    const U256 step = square_times(F, s, log_n - log_m);
     if (j == 0) {
       if (!p->pre[kCoset]) NTT_TRY(alloc_tab(p, &p->pre[kCoset], 1ull << logs));
-      NTT_CUDA(L.gen_1d(p->pre[kCoset], 1ull << logs, make_ladder(F, step), one, st));
+      NTT_CUDA(L.gen_1d(p->pre[kCoset], 1ull << logs, make_ladder(F, step, logs), one, st));
     } else {
       if (!p->fac_coset[j]) NTT_TRY(alloc_tab(p, &p->fac_coset[j], 1ull << logs));
-      NTT_CUDA(L.gen_1d(p->fac_coset[j], 1ull << logs, make_ladder(F, step), one, st));
+      NTT_CUDA(L.gen_1d(p->fac_coset[j], 1ull << logs, make_ladder(F, step, logs), one, st));
       const uint32_t log_mp = log_m - logs;
       const U256 w = square_times(F, p->omega, log_n - log_m);
       if (!p->tw[kCoset][j]) NTT_TRY(alloc_tab(p, &p->tw[kCoset][j], 1ull << log_m));
-      NTT_CUDA(L.gen_2d(p->tw[kCoset][j], logs, log_mp, make_ladder(F, w), p->fac_coset[j], one, st));
+      NTT_CUDA(L.gen_2d(p->tw[kCoset][j], logs, log_mp, make_ladder(F, w, log_m), p->fac_coset[j], one, st));
     }
   }
   if (p->in_place_one) {
     if (!p->pre_one[kCoset]) NTT_TRY(alloc_tab(p, &p->pre_one[kCoset], 1ull << log_n));
-    NTT_CUDA(L.gen_1d(p->pre_one[kCoset], 1ull << log_n, make_ladder(F, s), one, st));
+    NTT_CUDA(L.gen_1d(p->pre_one[kCoset], 1ull << log_n, make_ladder(F, s, log_n), one, st));
   }
   // coset inverse: x_n *= s^-n on the output of the last pass
   if (!p->post_coset_inv) NTT_TRY(alloc_tab(p, &p->post_coset_inv, 1ull << log_n));
-  NTT_CUDA(L.gen_1d(p->post_coset_inv, 1ull << log_n, make_ladder(F, F.inv(s)), one, st));
+  NTT_CUDA(L.gen_1d(p->post_coset_inv, 1ull << log_n, make_ladder(F, F.inv(s), log_n), one, st));
   p->coset_shift = s;
   return NTT_OK;
 }
@@ -221,7 +225,7 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
       const U256 w = square_times(F, dir ? p->omega_inv : p->omega, log_n - logs);
       const uint64_t count = std::max<uint64_t>(1, (1ull << logs) / 2);
       NTT_TRY(alloc_tab(p, &p->dft_tw[dir][logs], 2 * count));
-      NTT_CUDA(L.gen_split(p->dft_tw[dir][logs], count, make_ladder(F, w), one, st));
+      NTT_CUDA(L.gen_split(p->dft_tw[dir][logs], count, make_ladder(F, w, logs - 1), one, st));
     }
   }
   // inter-pass tables (forward, inverse)
@@ -234,17 +238,17 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
       const U256 w = square_times(F, dir ? p->omega_inv : p->omega, log_n - log_m);
       const Fe32 init = (dir == 1 && j == P - 1) ? n_inv_m : one;
       NTT_TRY(alloc_tab(p, &p->tw[dir][j], 1ull << log_m));
-      NTT_CUDA(L.gen_2d(p->tw[dir][j], logs, log_mp, make_ladder(F, w), nullptr, init, st));
+      NTT_CUDA(L.gen_2d(p->tw[dir][j], logs, log_mp, make_ladder(F, w, log_m), nullptr, init, st));
     }
   }
   // single-pass inverse: N^-1 as a pass-0 multiplier
   if (P == 1) {
     NTT_TRY(alloc_tab(p, &p->pre[kInverse], 1ull << passes[0]));
-    NTT_CUDA(L.gen_1d(p->pre[kInverse], 1ull << passes[0], make_ladder(F, u256(1)), n_inv_m, st));
+    NTT_CUDA(L.gen_1d(p->pre[kInverse], 1ull << passes[0], make_ladder(F, u256(1), log_n), n_inv_m, st));
   }
   if (p->in_place_one) {
     NTT_TRY(alloc_tab(p, &p->pre_one[kInverse], 1ull << log_n));
-    NTT_CUDA(L.gen_1d(p->pre_one[kInverse], 1ull << log_n, make_ladder(F, u256(1)), n_inv_m, st));
+    NTT_CUDA(L.gen_1d(p->pre_one[kInverse], 1ull << log_n, make_ladder(F, u256(1), log_n), n_inv_m, st));
   }
   if (p->has_coset) NTT_TRY(build_coset_tables(p, F.reduce_small(F.generator), st));
   if (P > 1 && !p->in_place_one) NTT_TRY(alloc_tab(p, &p->scratch, 1ull << log_n));
