@@ -87,16 +87,18 @@ ntt_status cuda_status(cudaError_t e) {
 }
 
 // Default split of log_n into passes of at most kDefaultPassLog bits, as
-// equal as possible, larger ones first; one pass more where that is faster
-// because a smaller sub-transform takes fewer elements per thread (GB300, us,
-// BLS12-381 Fr): 2^9 (5, 4) 9.4 against 10.7, 2^10 (5, 5) 10.1 against 20.3,
-// 2^19 (7, 6, 6) 90 against 106 for (10, 9); not at 2^8 (8.2 against 6.6), 2^18
-// (54 against 51) or 2^20 (177 against 170).  (The autotuner may pick others.)
-constexpr uint32_t kDefaultPassLog = 10;
+// equal as possible, larger ones first.  A transform that would be one pass of one
+// CTA gets two where 128 threads with 2 elements each do not hold it: a second
+// launch costs less than the longer chain of stages in one CTA.  GB300, us back to
+// back, both fields alike: 2^9 (5, 4) 9.1 against 9.8 for (9), 2^10 (5, 5) 9.9
+// against 15.1 for (10); 2^8 in one pass 6.3.  More passes than that lose: 2^19
+// (10, 9) 88 against 98 for (7, 6, 6), 2^20 (10, 10) 157 against 173 for (7, 7, 6).
+// (The autotuner may pick others.)
+constexpr uint32_t kDefaultPassLog = 10, kOneCtaLog = 8;
 
 std::vector<uint32_t> split_passes(uint32_t log_n) {
   uint32_t P = (log_n + kDefaultPassLog - 1) / kDefaultPassLog;
-  if (log_n == 9 || log_n == 10 || log_n == 19) P += 1;
+  if (P == 1 && log_n > kOneCtaLog) P = 2;
   std::vector<uint32_t> s(P, log_n / P);
   for (uint32_t i = 0; i < log_n % P; ++i) s[i] += 1;
   return s;
