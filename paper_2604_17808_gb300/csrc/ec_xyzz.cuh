@@ -559,13 +559,25 @@ __device__ __forceinline__ void quad_dbl(uint32_t v[T::L]) {
   quad_pick<L>(v, lane == 3, h, v);
 }
 
-// v += w (add-2008-s, with the cases it excludes).
+// Whether every point of the warp is O.
+template <class T>
+__device__ __forceinline__ bool quad_all_inf(const uint32_t v[T::L]) {
+  return __all_sync(0xffffffffu, (threadIdx.x & 3) != 2 || fv_is_zero<T::L>(v));
+}
+
+// v += w (add-2008-s, with the cases it excludes).  A warp in which every addition
+// has an operand O skips the products (zero, small and sparse scalars leave most
+// buckets, and the windows above them, empty).
 template <class T>
 __device__ __forceinline__ void quad_add(uint32_t v[T::L], const uint32_t w[T::L]) {
   constexpr int L = T::L;
   const int lane = threadIdx.x & 3;
   const bool v_inf = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(v), 2, 4);
   const bool w_inf = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(w), 2, 4);
+  if (__all_sync(0xffffffffu, v_inf || w_inf)) {
+    quad_pick<L>(v, w_inf, v, w);
+    return;
+  }
   uint32_t g[L], p[L], d[L], a[L], b[L], q[L], r[L], h[L];
   quad_get<L>(g, w, lane ^ 2);
   f_mul<T, true>(p, v, g);                // U1 = X1 ZZ2, S1 = Y1 ZZZ2, U2 = ZZ1 X2, S2 = ZZZ1 Y2

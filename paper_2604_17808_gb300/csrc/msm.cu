@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(kEcThreads)
     }
     quad_add<T>(v, w);
     if (is_b) {
-      quad_dbl<T>(v);                               // B = 2 (B_L + B_R)
+      if (!quad_all_inf<T>(v)) quad_dbl<T>(v);      // B = 2 (B_L + B_R)
     } else {
       if (!leaves) quad_load<T>(w, heap_b, child + 1);
       quad_add<T>(v, w);                            // W = W_L + W_R + B_R (leaves: W_j = B_j)
@@ -727,13 +727,17 @@ __global__ void msm_merge_kernel(uint32_t c, uint32_t kb, uint32_t ke, const uin
     uint32_t w[L];
     if (lb == 0) quad_load_bucket<T>(w, bucket_sum, pieces, offsets, S, (uint64_t)k);
     else quad_load<T>(w, heap_w, ((uint64_t)k << lb) + 1);
+    // (empty windows above the first point: nothing to double)
+    if (quad_all_inf<T>(v)) doublings = 0;
 #pragma unroll 1
     for (uint32_t j = 0; j < doublings; ++j) quad_dbl<T, false>(v);
     quad_add<T>(v, w);
     doublings = c;
   }
+  if (!quad_all_inf<T>(v)) {
 #pragma unroll 1
-  for (uint32_t j = 0; j < c * kb; ++j) quad_dbl<T, false>(v);
+    for (uint32_t j = 0; j < c * kb; ++j) quad_dbl<T, false>(v);
+  }
   // affine: x = X ZZZ / (ZZ ZZZ), y = Y ZZ / (ZZ ZZZ)
   uint32_t z[L], t[L];
   quad_get<L>(z, v, 2);
