@@ -418,8 +418,9 @@ __device__ __forceinline__ void emit_piece(const Xyzz<T> &acc, uint32_t b, uint3
   else store_point_xyzz(pieces, 2 * (uint64_t)t + 1, acc);
 }
 
-__device__ __forceinline__ uint32_t short_span(const MsmTotals *tot, uint64_t nb) {
-  return tot->entries >= nb * tot->seg_len ? kShortSpanLongBuckets : kShortSpan;
+// `used`: the buckets of the windows that the call runs over.
+__device__ __forceinline__ uint32_t short_span(const MsmTotals *tot, uint64_t used) {
+  return tot->entries >= used * tot->seg_len ? kShortSpanLongBuckets : kShortSpan;
 }
 
 // Piece i of a bucket over `span` + 1 segments, in segment t: a node of every
@@ -439,12 +440,12 @@ __device__ __forceinline__ void push_items(MsmTotals *tot, const CombineLists &l
 template <class C>
 __global__ void __launch_bounds__(kEcThreads, C::kMinBlocks)
     msm_accumulate_kernel(const uint4 *__restrict__ pts_m, const uint32_t *__restrict__ sorted,
-                          const uint32_t *__restrict__ offsets, uint64_t nb, EcConst<typename C::T> k,
+                          const uint32_t *__restrict__ offsets, uint64_t nb, uint64_t used, EcConst<typename C::T> k,
                           MsmTotals *tot, CombineLists lists, uint4 *bucket_sum, uint4 *pieces) {
   using T = typename C::T;
   constexpr int L = T::L;
   const uint32_t n_entries = tot->entries, S = tot->seg_len;
-  const uint32_t num_segs = (n_entries + S - 1) / S, limit = short_span(tot, nb);
+  const uint32_t num_segs = (n_entries + S - 1) / S, limit = short_span(tot, used);
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < num_segs; t += gridDim.x * blockDim.x) {
     const uint32_t e0 = t * S, e1 = min(e0 + S, n_entries);
     uint32_t b = bucket_of_entry(offsets, nb, e0);
@@ -1182,13 +1183,16 @@ ntt_status enqueue_msm(msm_plan p, const uint4 *sc, const uint4 *pt, uint64_t n,
                                                                  p->sorted);
     const uint64_t segs = std::min<uint64_t>((n * p->K + 7) / 8, p->max_segments);
     const int g = grid_for(segs, kEcThreads, sms, C::kMinBlocks);
-    msm_accumulate_kernel<C><<<g, kEcThreads, 0, st>>>(pts, p->sorted, p->offsets, nb, k, p->tot, p->lists,
+    const uint64_t used = (uint64_t)(tree_ke - tree_kb) << lb;
+    msm_accumulate_kernel<C><<<g, kEcThreads, 0, st>>>(pts, p->sorted, p->offsets, nb, used, k, p->tot, p->lists,
                                                        p->bucket_sum, p->pieces);
     const int gt = grid_for(segs, kEcThreads, sms, C::kTreeMinBlocks);
     msm_combine_kernel<C><<<gt, kEcThreads, 0, st>>>(p->tot, p->lists.crossing, p->pieces);
     // a bucket holds at most n entries of one window (flat: of all of them), so
     // it crosses at most this many segment ends; empty levels exit at once
-    // (segments of 8 entries at least, at most max_segments of them)
+    // (segments of 8 entries at least, at most max_segments of them; the grid is
+    // for K windows in a range of fewer too: each bucket adds an item to its
+    // segments', and a second round for those costs a level's time again)
     const uint64_t most = flat ? n * p->K : n;
     const uint64_t max_span = std::min<uint64_t>((most + 7) / 8, p->max_segments);
     uint64_t step = 1;
