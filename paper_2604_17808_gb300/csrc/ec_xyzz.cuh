@@ -565,18 +565,21 @@ __device__ __forceinline__ bool quad_all_inf(const uint32_t v[T::L]) {
   return __all_sync(0xffffffffu, (threadIdx.x & 3) != 2 || fv_is_zero<T::L>(v));
 }
 
-// v += w (add-2008-s, with the cases it excludes).  A warp in which every addition
-// has an operand O skips the products (zero, small and sparse scalars leave most
-// buckets, and the windows above them, empty).
-template <class T>
+// v += w (add-2008-s, with the cases it excludes).  With kSkip a warp in which every
+// addition has an operand O skips the products: for buckets and windows, most of
+// which zero, small and sparse scalars leave empty, but not for pieces, which have
+// a point each (2% of a tree's time for the vote).
+template <class T, bool kSkip = false>
 __device__ __forceinline__ void quad_add(uint32_t v[T::L], const uint32_t w[T::L]) {
   constexpr int L = T::L;
   const int lane = threadIdx.x & 3;
   const bool v_inf = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(v), 2, 4);
   const bool w_inf = __shfl_sync(0xffffffffu, (int)fv_is_zero<L>(w), 2, 4);
-  if (__all_sync(0xffffffffu, v_inf || w_inf)) {
-    quad_pick<L>(v, w_inf, v, w);
-    return;
+  if constexpr (kSkip) {
+    if (__all_sync(0xffffffffu, v_inf || w_inf)) {
+      quad_pick<L>(v, w_inf, v, w);
+      return;
+    }
   }
   uint32_t g[L], p[L], d[L], a[L], b[L], q[L], r[L], h[L];
   quad_get<L>(g, w, lane ^ 2);

@@ -698,12 +698,12 @@ __global__ void __launch_bounds__(kEcThreads)
       quad_load<T>(v, is_b ? heap_b : heap_w, child);
       quad_load<T>(w, is_b ? heap_b : heap_w, child + 1);
     }
-    quad_add<T>(v, w);
+    quad_add<T, true>(v, w);
     if (is_b) {
       if (!quad_all_inf<T>(v)) quad_dbl<T>(v);      // B = 2 (B_L + B_R)
     } else {
       if (!leaves) quad_load<T>(w, heap_b, child + 1);
-      quad_add<T>(v, w);                            // W = W_L + W_R + B_R (leaves: W_j = B_j)
+      quad_add<T, true>(v, w);                            // W = W_L + W_R + B_R (leaves: W_j = B_j)
     }
     if (live) quad_store<T>(is_b ? heap_b : heap_w, node, v);
   }
@@ -732,7 +732,7 @@ __global__ void msm_merge_kernel(uint32_t c, uint32_t kb, uint32_t ke, const uin
     if (quad_all_inf<T>(v)) doublings = 0;
 #pragma unroll 1
     for (uint32_t j = 0; j < doublings; ++j) quad_dbl<T, false>(v);
-    quad_add<T>(v, w);
+    quad_add<T, true>(v, w);
     doublings = c;
   }
   if (!quad_all_inf<T>(v)) {
