@@ -685,7 +685,11 @@ __global__ void __launch_bounds__(kMatThreads, 1)
           }
         }
       }
-      if (!mbar_wait(&acc_full[buf], (uint32_t)((it >> 1) & 1), ma, abort)) break;
+      // Every lane goes on whatever its wait says: after a timeout elsewhere lanes
+      // can disagree (buffer complete, abort seen first), and tcgen05.ld needs the
+      // whole warp.  What is stored then is void, the error word says so, and the
+      // waits of the tiles left return after one suspended try each.
+      mbar_wait(&acc_full[buf], (uint32_t)((it >> 1) & 1), ma, abort);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       constexpr int kOuts = S > 4 ? 2 : 1;
       if constexpr (BARRETT) {
