@@ -386,7 +386,8 @@ ntt_status ntt_plan_read_timing(ntt_plan plan, double ms_per_pass[NTT_MAX_PASSES
  * read.  Synchronises the device.  In a debug build of the library (compiled
  * with NTT_DEBUG: every vector and table access of the butterfly pass
  * kernels, single and batched, is checked against the extent the plan
- * recorded for it, and an access out of range is skipped instead of made),
+ * recorded for it, and every shared-memory access against its tile; an
+ * access out of range is skipped instead of made),
  * a failed check reports NTT_ERR_BOUNDS here.  ntt_build_is_debug tells
  * which build is loaded.
  */

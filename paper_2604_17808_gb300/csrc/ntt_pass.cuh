@@ -177,6 +177,7 @@ __device__ __forceinline__ uint32_t swz(uint32_t e) {
 template <class F>
 struct Elem256 {
   static constexpr int W = 8;
+  static constexpr uint32_t kTileRow = 32;        // tile offsets of 2^tl elements are below kTileRow 2^tl
   static constexpr bool kPreByPosition = false;   // pass-0 multipliers are indexed by n_0
 
   // low half of element e; the high half is at the offset ^ 16
@@ -247,6 +248,40 @@ struct Elem256 {
 
 __device__ __forceinline__ void tile_copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// ------------------------------------------------- checked tile accesses
+// Tile offsets and twiddle indices are computed at run time from the tile shape:
+// debug builds check them against the tile and the table of 2^logs points, as they
+// do the vectors (out of range: NTT_ERR_BOUNDS, the access skipped, zero loaded).
+template <int W>
+__device__ __forceinline__ void words_zero(uint32_t *x) {
+#pragma unroll
+  for (int k = 0; k < W; ++k) x[k] = 0;
+}
+
+template <class El>
+__device__ __forceinline__ void tile_get(const PassArgs &a, const TileShape &s, uint32_t *x, uint32_t tile,
+                                         uint32_t off) {
+  if (dbg_in(a, off, El::kTileRow << s.tl)) El::tile_load(x, tile, off, s.tl);
+  else words_zero<El::W>(x);
+}
+
+template <class El>
+__device__ __forceinline__ void tile_put(const PassArgs &a, const TileShape &s, uint32_t tile, uint32_t off,
+                                         const uint32_t *x) {
+  if (dbg_in(a, off, El::kTileRow << s.tl)) El::tile_store(tile, off, s.tl, x);
+}
+
+template <class El>
+__device__ __forceinline__ void twiddle_get(const PassArgs &a, const TileShape &s, uint32_t *A, uint32_t *B,
+                                            uint32_t w) {
+  if (dbg_in(a, w, s.logs > 1 ? 1u << (s.logs - 1) : 1u)) {
+    El::load_twiddle(A, B, a.dft_tw, w);
+  } else {
+    words_zero<El::W>(A);
+    words_zero<El::W>(B);
+  }
+}
+
 // ----------------------------------------------------------- butterflies
 
 // A thread's 2^pl elements of one round: tile offset of the first, and the
@@ -277,7 +312,7 @@ __device__ __forceinline__ Private private_set(const TileShape &s, uint32_t e, u
 // b, twiddle omega_S^((p mod h) S / 2h) with h = 2^(T + b), p the position in
 // the sub-transform; low = its bits below T.
 template <class El>
-__device__ __forceinline__ void private_stages(uint32_t tile, const uint4 *dft_tw, const TileShape &s, const Private &v,
+__device__ __forceinline__ void private_stages(const PassArgs &a, uint32_t tile, const TileShape &s, const Private &v,
                                                uint32_t T, int hi, int lo, uint32_t low) {
 #pragma unroll 1
   for (int b = hi - 1; b >= lo; --b) {
@@ -290,23 +325,23 @@ __device__ __forceinline__ void private_stages(uint32_t tile, const uint4 *dft_t
       const uint32_t w = (low | ((j & mask) << T)) << sh;
       uint32_t x[El::W], y[El::W], d[El::W];
       if (T == 0 && (j & mask) == 0) {   // twiddle 1, for every thread
-        El::tile_load(x, tile, c, s.tl);
-        El::tile_load(y, tile, c ^ db, s.tl);
+        tile_get<El>(a, s, x, tile, c);
+        tile_get<El>(a, s, y, tile, c ^ db);
         El::sub(d, x, y);
         El::add(x, x, y);
-        El::tile_store(tile, c, s.tl, x);
-        El::tile_store(tile, c ^ db, s.tl, d);
+        tile_put<El>(a, s, tile, c, x);
+        tile_put<El>(a, s, tile, c ^ db, d);
         continue;
       }
       uint32_t A[El::W], B[El::W];
-      El::load_twiddle(A, B, dft_tw, w);
-      El::tile_load(x, tile, c, s.tl);
-      El::tile_load(y, tile, c ^ db, s.tl);
+      twiddle_get<El>(a, s, A, B, w);
+      tile_get<El>(a, s, x, tile, c);
+      tile_get<El>(a, s, y, tile, c ^ db);
       El::sub(d, x, y);
       El::add(x, x, y);
-      El::tile_store(tile, c, s.tl, x);
+      tile_put<El>(a, s, tile, c, x);
       El::mul_twiddle(d, d, A, B);
-      El::tile_store(tile, c ^ db, s.tl, d);
+      tile_put<El>(a, s, tile, c ^ db, d);
     }
   }
 }
@@ -371,11 +406,11 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
       if (!linear) pos = elem_pos<MODE>(a, logs, d, low | ((j & rmask) << T));
       if (d >= a.num_sub) continue;
       const uint32_t c = private_offset(v, j);
-      if (dbg_in(a, pos, a.n_vec)) {
+      if (dbg_in(a, pos, a.n_vec) && dbg_in(a, c, El::kTileRow << s.tl)) {
         El::copy_async(smem, c, s.tl, a.src, pos);
       } else {
         uint32_t z[El::W] = {};
-        El::tile_store(smem, c, s.tl, z);
+        tile_put<El>(a, s, smem, c, z);
       }
     }
     if constexpr (MODE != kModeFirst) {
@@ -408,14 +443,14 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
         for (int k = 0; k < El::W; ++k) w[k] = next[k];
         if (j + 1 < count) load_mul(next, j + 1);
         uint32_t x[El::W];
-        El::tile_load(x, smem, c, s.tl);
+        tile_get<El>(a, s, x, smem, c);
         El::mul_in(x, w);
-        El::tile_store(smem, c, s.tl, x);
+        tile_put<El>(a, s, smem, c, x);
       }
     } else {
       tile_copy_wait();
     }
-    if (T > 0) private_stages<El>(smem, a.dft_tw, s, v, T, (int)r, 0, low);
+    if (T > 0) private_stages<El>(a, smem, s, v, T, (int)r, 0, low);
   }
 
   // ---- middle rounds
@@ -426,7 +461,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     group_sync<GROUPED>(group, threads);
     const uint32_t low = t & ((1u << T) - 1u);
     const Private v = private_set<El>(s, low | ((t >> T) << (T + r)), T, r);
-    private_stages<El>(smem, a.dft_tw, s, v, T, (int)r, 0, low);
+    private_stages<El>(a, smem, s, v, T, (int)r, 0, low);
   }
 
   // ---- last round: stages last - 1 .. 0; inner passes vary sub-transforms
@@ -439,7 +474,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
   const uint32_t p0 = tbits ? (__brev(tt) >> (32 - tbits)) << last : 0u;
   const Private v = private_set<El>(s, (dl << logs) | p0, 0, last);
   const uint32_t lmask = (1u << last) - 1u, half = 1u << (logs - 1);
-  private_stages<El>(smem, a.dft_tw, s, v, 0, (int)last, last >= 2 ? 2 : 1, 0);
+  private_stages<El>(a, smem, s, v, 0, (int)last, last >= 2 ? 2 : 1, 0);
   const uint32_t unit = last >= 2 ? 4u : 2u;
 #pragma unroll 1
   for (uint32_t j = 0; j < (1u << pl); j += unit) {
@@ -459,15 +494,15 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
       uint32_t x2[El::W], x3[El::W];
       {
         uint32_t A[El::W], B[El::W];   // omega_4 = omega_S^(S/4)
-        El::load_twiddle(A, B, a.dft_tw, half >> 1);
-        El::tile_load(x1, smem, c ^ v.d0, s.tl);
-        El::tile_load(x3, smem, c ^ v.d0 ^ v.d1, s.tl);
+        twiddle_get<El>(a, s, A, B, half >> 1);
+        tile_get<El>(a, s, x1, smem, c ^ v.d0);
+        tile_get<El>(a, s, x3, smem, c ^ v.d0 ^ v.d1);
         El::sub(y, x1, x3);
         El::add(x1, x1, x3);
         El::mul_twiddle(x3, y, A, B);
       }
-      El::tile_load(x0, smem, c, s.tl);
-      El::tile_load(x2, smem, c ^ v.d1, s.tl);
+      tile_get<El>(a, s, x0, smem, c);
+      tile_get<El>(a, s, x2, smem, c ^ v.d1);
       El::sub(y, x0, x2);
       El::add(x0, x0, x2);
       El::add(x2, y, x3);
@@ -477,8 +512,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
         store_output<El>(a, out + ((uint64_t)(k + (half >> 1) + half) << sh), x3);
       }
     } else {
-      El::tile_load(x0, smem, c, s.tl);
-      El::tile_load(x1, smem, c ^ v.d0, s.tl);
+      tile_get<El>(a, s, x0, smem, c);
+      tile_get<El>(a, s, x1, smem, c ^ v.d0);
     }
     El::sub(y, x0, x1);
     El::add(x0, x0, x1);

@@ -46,6 +46,7 @@ struct WideConst {
 template <class F>
 struct ElemWide {
   static constexpr int W = F::L;
+  static constexpr uint32_t kTileRow = 16;
   static constexpr bool kPreByPosition = true;
 
   __device__ static __forceinline__ uint32_t tile_offset(uint32_t e) {
