@@ -12,7 +12,9 @@
 //     (twiddles, coset powers, N^-1) is stored in MONTGOMERY form c*2^256, so
 //     mont_mul(x, c*2^256) = x*c mod p is again standard.  No conversion
 //     passes are needed at the ABI boundary;
-//   * every value is canonical in [0, p) before and after each operation.
+//   * values at the ABI are canonical, in [0, p), and operations take and leave
+//     canonical values where their comment does not say otherwise; inside a
+//     transform pass values are lazy, in [0, 2p) or [0, 3p) (below).
 //
 // mont_mul is Montgomery multiplication by operand scanning (CIOS; Koc, Acar,
 // Kaliski, "Analyzing and comparing Montgomery multiplication algorithms",
@@ -445,21 +447,6 @@ __device__ __forceinline__ void mont_mul_lazy(uint32_t r[8], const uint32_t a[8]
 // below 2^288, but T - T_0 r can be negative too, so the sign is a word of its
 // own, s (0 or all ones, weight 2^288), which every chain that ends in column
 // 8 carries into.
-__device__ __forceinline__ void pairs_mad4_s(uint32_t d[8], uint32_t &s, uint32_t x0, uint32_t x1, uint32_t x2,
-                                             uint32_t x3, uint32_t y) {
-  asm("mad.lo.cc.u32  %0, %9,  %13, %0;\n\t"
-      "madc.hi.cc.u32 %1, %9,  %13, %1;\n\t"
-      "madc.lo.cc.u32 %2, %10, %13, %2;\n\t"
-      "madc.hi.cc.u32 %3, %10, %13, %3;\n\t"
-      "madc.lo.cc.u32 %4, %11, %13, %4;\n\t"
-      "madc.hi.cc.u32 %5, %11, %13, %5;\n\t"
-      "madc.lo.cc.u32 %6, %12, %13, %6;\n\t"
-      "madc.hi.cc.u32 %7, %12, %13, %7;\n\t"
-      "addc.u32       %8, %8, 0;"
-      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7]), "+r"(s)
-      : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(y));
-}
-
 __device__ __forceinline__ void pairs_mad4_top_s(uint32_t d[8], uint32_t &top, uint32_t &s, uint32_t x0, uint32_t x1,
                                                  uint32_t x2, uint32_t x3, uint32_t y) {
   asm("mad.lo.cc.u32  %0, %10, %14, %0;\n\t"
@@ -556,7 +543,7 @@ __device__ __forceinline__ void mul_split(uint32_t r[8], const uint32_t x[8], co
       }
     }
     if constexpr (F::kSubtract) {
-      pairs_mad4_s(O, s, B[1], B[3], B[5], B[7], x[4 + i]);
+      pairs_mad4_top(O, s, B[1], B[3], B[5], B[7], x[4 + i]);
       pairs_mad4_top_s(E, O[7], s, B[0], B[2], B[4], B[6], x[4 + i]);
       redc_row_s<F>(E, O, s);
     } else {
@@ -654,15 +641,6 @@ __device__ __forceinline__ void fe_load_global(uint32_t r[8], const uint4 *base,
   asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
       : "l"(base + 2 * elem));
-}
-
-// L2-coherent load (ld.global.cg): for data another CTA wrote earlier in the
-// same kernel launch (volatile: never moved above the wait that orders it).
-__device__ __forceinline__ void fe_load_global_cg(uint32_t r[8], const uint4 *base, uint64_t elem) {
-  asm volatile("ld.global.cg.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "l"(base + 2 * elem)
-               : "memory");
 }
 
 __device__ __forceinline__ void fe_store_global(uint4 *base, uint64_t elem, const uint32_t a[8]) {

@@ -45,17 +45,7 @@ __device__ __forceinline__ void pairs_mad_chain(uint32_t *d, uint32_t &top, cons
         : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(top)
         : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(y));
   } else if constexpr (N == 4) {
-    asm("mad.lo.cc.u32  %0, %9, %13, %0;\n\t"
-        "madc.hi.cc.u32 %1, %9, %13, %1;\n\t"
-        "madc.lo.cc.u32 %2, %10, %13, %2;\n\t"
-        "madc.hi.cc.u32 %3, %10, %13, %3;\n\t"
-        "madc.lo.cc.u32 %4, %11, %13, %4;\n\t"
-        "madc.hi.cc.u32 %5, %11, %13, %5;\n\t"
-        "madc.lo.cc.u32 %6, %12, %13, %6;\n\t"
-        "madc.hi.cc.u32 %7, %12, %13, %7;\n\t"
-        "addc.u32       %8, %8, 0;"
-        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7]), "+r"(top)
-        : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(y));
+    pairs_mad4_top(d, top, x[0], x[1], x[2], x[3], y);
   } else if constexpr (N == 5) {
     asm("mad.lo.cc.u32  %0, %11, %16, %0;\n\t"
         "madc.hi.cc.u32 %1, %11, %16, %1;\n\t"
@@ -72,22 +62,7 @@ __device__ __forceinline__ void pairs_mad_chain(uint32_t *d, uint32_t &top, cons
           "+r"(d[9]), "+r"(top)
         : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(y));
   } else if constexpr (N == 6) {
-    asm("mad.lo.cc.u32  %0, %13, %19, %0;\n\t"
-        "madc.hi.cc.u32 %1, %13, %19, %1;\n\t"
-        "madc.lo.cc.u32 %2, %14, %19, %2;\n\t"
-        "madc.hi.cc.u32 %3, %14, %19, %3;\n\t"
-        "madc.lo.cc.u32 %4, %15, %19, %4;\n\t"
-        "madc.hi.cc.u32 %5, %15, %19, %5;\n\t"
-        "madc.lo.cc.u32 %6, %16, %19, %6;\n\t"
-        "madc.hi.cc.u32 %7, %16, %19, %7;\n\t"
-        "madc.lo.cc.u32 %8, %17, %19, %8;\n\t"
-        "madc.hi.cc.u32 %9, %17, %19, %9;\n\t"
-        "madc.lo.cc.u32 %10, %18, %19, %10;\n\t"
-        "madc.hi.cc.u32 %11, %18, %19, %11;\n\t"
-        "addc.u32       %12, %12, 0;"
-        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7]), "+r"(d[8]),
-          "+r"(d[9]), "+r"(d[10]), "+r"(d[11]), "+r"(top)
-        : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(y));
+    fp384::pairs_mad6_top(d, top, x[0], x[1], x[2], x[3], x[4], x[5], y);
   } else {
     static_assert(N >= 1 && N <= 6, "chain length");
   }

@@ -90,11 +90,15 @@ constexpr uint32_t kSignBit = 0x80000000u;
 // crosses several ends nearly all of them do, and one thread for each fills the
 // GPU (BLS12-381 commitment, 2^20 points: 6655 us with 8, 6713 with 3).
 constexpr uint32_t kShortSpan = 3, kShortSpanLongBuckets = 8;
-// Entries that one sweep of the scatter writes, 4 bytes each at random places of
-// its windows' part of the sorted array: 64 MiB stay in the L2 (129 MB) until
-// their sectors are complete, while the scalars are read again for each sweep.
-// 2^22 points of BN254: 1134 us in one sweep of 15 windows, 804 in five (the whole
-// call 12.65 ms, 12.39 with 2^23 entries, 12.29 with 2^24, 12.34 with 2^25).
+// Entries that one sweep of the scatter is meant to write, 4 bytes each at random
+// places of its windows' part of the sorted array: 64 MiB stay in the L2 (129 MB)
+// until their sectors are complete, while the scalars are read again for each
+// sweep.  (The sweeps of a block follow one another, those of different blocks need
+// not.)  2^22 points of BN254: 1134 us in one sweep of 15 windows, 804 in five (the
+// whole call 12.65 ms, 12.39 with 2^23 entries, 12.29 with 2^24, 12.34 with 2^25).
+// Above 2^24 points a sweep is one window, larger than that, and still the best:
+// whole calls of BN254, one window a sweep, two, all: 2^25 84.6, 87.4 and 91.3 ms,
+// 2^26 170, 176 and 183 ms; BLS12-381 2^25 172.5, 175.3 and 179.2 ms.
 constexpr uint64_t kSweepEntries = 1ull << 24;
 constexpr uint32_t kSegMask = (1u << 28) - 1u;   // a segment index (span - 1 above it in a crossing item)
 constexpr int kLongLevels = 14;    // 4^14 pieces
@@ -1049,9 +1053,16 @@ ntt_status check_device(int *dev_out, int *sms) {
 // K c >= S^BL + 1 (signed digits)
 uint32_t num_windows(uint32_t c, uint32_t scalar_bits) { return (scalar_bits + 1 + c - 1) / c; }
 
-// Window size minimising the modelled multiply count K (10 n + 26 2^(c-1)):
-// one 10-product mixed addition per point and window, about 26 products per
-// bucket in the reduction tree.
+// Window size minimising a modelled multiply count K (10 n + 26 2^(c-1)): one
+// 10-product mixed addition per point and window and 26 products per bucket.  The
+// 26 was fitted to an earlier reduction tree (a bucket now takes 28 products by
+// running sums, a tree node 51 or a few four-lane steps), so small and middle sizes
+// get windows up to 3 bits from their best; larger ones are at it.  GB300, uniform
+// scalars, us with the default window and with the best one: BN254 10^4 766 (10)
+// and 681 (11), 5 10^4 980 (13) and 858 (11), 2^20 3914 (16), 2^22 12312 (17), 2^24
+// 44005 (20); BLS12-381 5 10^4 1853 (13) and 1559 (11), 2.5 10^5 3864 (14) and 2942
+// (15), 2^20 7834 (16), 2^22 28724 (18) and 25074 (17).  Windows that leave the top
+// one nearly full bits (11, 15, 17, 20) are the good ones.
 uint32_t default_window(uint64_t n, uint32_t scalar_bits) {
   uint32_t best = 4;
   double best_cost = 1e300;
@@ -1070,7 +1081,8 @@ uint32_t default_window(uint64_t n, uint32_t scalar_bits) {
 // whole number of times (1 to 8 times the threads that are resident, so that the
 // last wave is not nearly empty), with 64 additions or more each where there
 // are enough entries: longer segments cut the buckets that cross a segment end,
-// hence the combine work.
+// hence the combine work.  At most 128 entries: calls with more than 8 waves of
+// those (80 M entries for BN254) take as many waves as it needs, 22 at 2^24 points.
 uint32_t segment_length(uint64_t max_n, uint32_t K, int sms, int blocks_per_sm) {
   const uint64_t entries = max_n * K, resident = (uint64_t)sms * blocks_per_sm * kEcThreads;
   const uint64_t waves = std::max<uint64_t>(1, std::min<uint64_t>(8, entries / (resident * 64)));

@@ -71,7 +71,8 @@ struct TileShape {
 //   896 threads        seven 1024-element tiles with 8 elements per thread,
 //                      one CTA per SM, for passes that are one wave this way:
 //                      the 1024 tiles of a 2^20-point pass took two waves of
-//                      six (99 and 80 us a pass against 90 and 75).  With many
+//                      six (99 and 80 us a pass against 90 and 75; on 152 SMs
+//                      this is the one power of two with such passes).  With many
 //                      waves the CTAs that come and go on their own are faster
 //                      (2^24: 2.9 against 3.1 ms);
 //   256 threads        one 2048-element tile, 3 CTAs per SM.
@@ -395,7 +396,8 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     const Private v = private_set<El>(s, (dl << logs) | low, T, r);
     const uint32_t count = 1u << pl, rmask = (1u << r) - 1u;
     // element j is input low + ((j mod 2^r) << T) of sub-transform d; with r =
-    // pl (all but sub-transforms of 2 and 4 points) its position is linear in j
+    // pl (sub-transforms of 2^pl points, and of 2^(2 pl) or more) its position is
+    // linear in j
     const uint64_t dfirst = d0 + dl, step = 1ull << (a.log_mp + T);
     const bool linear = r == pl;
     auto sub_of = [&](uint32_t j) { return dfirst + ((uint64_t)(j >> r) << gbits); };

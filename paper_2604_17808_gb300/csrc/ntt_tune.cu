@@ -4,7 +4,7 @@
 // Candidates for N = 2^log_n:
 //   * butterfly path: balanced splits for every maximum pass size 2^4..2^11
 //     (distinct ones), each also with its passes in reverse order, each with
-//     the 1024-element tile (7 CTAs/SM) or the 2048-element tile (3 CTAs/SM);
+//     the 1024-element tile (6 CTAs/SM) or the 2048-element tile (3 CTAs/SM);
 //   * matrix path (tensor-core passes of at most 2^3 points).
 // Each candidate builds its own tables, runs one untimed forward transform,
 // then `reps` timed ones (CUDA events); the fastest wins and the plan is
