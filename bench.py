@@ -13,10 +13,12 @@ elements counts N), whole job over all ranks.
 Printed as ONE JSON line on rank 0, with
   * roofline: the dominant kernel (the pass kernel with the largest device
     time) against the 32-bit integer multiply-add (IMAD) pipe:
-    algorithmic IMAD per launch = modmuls of the pass * 272 (one 8-limb CIOS
-    Montgomery product, lo and hi multiplies counted), modmuls of a pass =
-    (N/2) log2 S (radix-2 butterflies) + N (the pass's per-element multiplier
-    when it has one); peak = 152 SMs * 64 IMAD/clk * 2.07 GHz;
+    IMAD of the products that a launch executes: 176 for a product by a DFT
+    twiddle (kept as two residues) and 224 for one by a per-element multiplier
+    (32 x 32 + 64 bit multiply-adds, two IMAD slots each); of S points' log2 S
+    stages the last has none, the two before it N/4 and 3N/8, the others N/2,
+    and N multipliers where the pass has them; peak = 152 SMs * 64 IMAD/clk *
+    2.07 GHz;
   * e2e: the same metric through ntt_transform_host (pinned host buffers,
     host-to-device and device-to-host copies inside the timed region);
   * cpu_baseline: the C oracle on this host's cores on a bounded sample of
@@ -60,7 +62,10 @@ from ntt_synth import MODULI as MODULI_R, config_seed, uniform_elements  # noqa:
 
 METRIC = "255-bit NTT field elements/s (BLS12-381 Fr, n=2^20, forward+inverse, butterfly path)"
 UNIT = "elements/s"
-IMAD_PER_MODMUL = 272
+# IMAD slots of the products executed over BLS12-381 Fr, two for each 32 x 32 + 64
+# bit multiply-add of a carry chain: 64 limb products and 24 or 48 of the reduction
+IMAD_SPLIT_PRODUCT = 2 * (64 + 24)   # by a twiddle kept as two residues
+IMAD_PRODUCT = 2 * (64 + 48)
 SMS = 152
 IMAD_PER_CLK_PER_SM = 64
 SM_MAX_MHZ = 2070.0
@@ -116,15 +121,17 @@ def profiled_traffic(kernel_tag: str) -> int | None:
     return traffic if src == kernel_source_hash() else None
 
 
-def pass_modmuls(log_n: int, pass_log: list[int], j: int, has_multiplier: bool) -> int:
-    n = 1 << log_n
-    return (n // 2) * pass_log[j] + (n if has_multiplier else 0)
+def pass_imad(log_n: int, log_s: int, has_multiplier: bool) -> float:
+    """IMAD of the products of one pass: sub-transforms of 2^log_s points, tiles of
+    8 elements per thread (2^20 points and more)."""
+    per_stage = {0: 0.0, 1: 0.25, 2: 0.375}   # trivial twiddles in the last round
+    split = sum(per_stage.get(b, 0.5) for b in range(log_s))
+    return (1 << log_n) * (split * IMAD_SPLIT_PRODUCT + (IMAD_PRODUCT if has_multiplier else 0))
 
 
-def transform_modmuls(log_n: int) -> int:
-    """Algorithmic modmuls of one transform: (N/2) log2 N butterflies + 2N."""
-    n = 1 << log_n
-    return (n // 2) * log_n + 2 * n
+def transform_imad(log_n: int, pass_log: list[int]) -> float:
+    """The same of a whole forward transform."""
+    return sum(pass_imad(log_n, ls, j >= 1) for j, ls in enumerate(pass_log))
 
 
 # ----------------------------------------------------------------- clocks
@@ -305,13 +312,13 @@ def measure_2_24(torch, N, stream, steps: int) -> dict:
         pass_ms, pass_cnt = N.ntt_plan_read_timing(plan)
         N.ntt_plan_enable_timing(plan, False)
         peak = imad_peak_tops()
-        alg = transform_modmuls(log_n) * IMAD_PER_MODMUL
+        alg = transform_imad(log_n, desc["pass_log"])
         per_pass = []
         for j, ls in enumerate(desc["pass_log"]):
             avg = pass_ms[j] / max(1, pass_cnt[j])
-            mm = pass_modmuls(log_n, desc["pass_log"], j, j >= 1)
+            imad = pass_imad(log_n, ls, j >= 1)
             per_pass.append({"pass": j, "log_s": ls, "avg_ms": round(avg, 4),
-                             "frac": round(mm * IMAD_PER_MODMUL / (avg * 1e-3) / 1e12 / peak, 4)})
+                             "frac": round(imad / (avg * 1e-3) / 1e12 / peak, 4)})
         # the same transform on the matrix (tensor-core) path, outputs compared
         N.ntt_plan_set_path(plan, "matrix")
         ym = torch.empty_like(ys[0])
@@ -370,7 +377,7 @@ def measure_large(torch, N, stream, steps: int, log_n: int = 28) -> dict:
         stop.record(stream)
         stop.synchronize()
         ms = start.elapsed_time(stop) / steps
-        alg = transform_modmuls(log_n) * IMAD_PER_MODMUL
+        alg = transform_imad(log_n, desc["pass_log"][:desc["num_passes"]])
         return {"workload": f"BLS12-381 Fr forward NTT, n=2^{log_n}, passes {desc['pass_log'][:desc['num_passes']]}",
                 "ms": round(ms, 3), "elements_per_s": (1 << log_n) / (ms * 1e-3),
                 "imad_roofline_frac": round(alg / (ms * 1e-3) / 1e12 / imad_peak_tops(), 4),
@@ -507,13 +514,15 @@ def measure_msm(torch, N, stream, reps: int, log_sizes=(22, 24), curve: str = "b
             bases_ms = {"ms": round(float(np.median(tb)), 3), "set_bases_ms": round(set_ms, 1),
                         "same_result": bool(torch.equal(res_b, first))}
         c, K = info["window_bits"], info["num_windows"]
-        # algorithmic products: one 10-product mixed addition per point and
-        # window, about 26 per bucket (2^(c-1) per window) in the reduction tree;
-        # a product of D 32-bit limbs is 2 (2 D^2 + D) IMAD (272 for D = 8)
-        modmuls = K * n * 10 + K * (1 << (c - 1)) * 26
+        # products: a mixed addition per point and window (6 products, 2 squares,
+        # one difference of two products under one reduction) and two additions
+        # per bucket (10, 2 and one difference each); over D 32-bit limbs a
+        # product is 2 D^2 multiply-adds, a square D (D + 1) / 2 + D^2, a
+        # difference 3 D^2, each two IMAD slots
+        modmuls = K * n * 10 + K * (1 << (c - 1)) * 28
         limbs = pts.shape[1]  # 32-bit limbs per coordinate = 64-bit words per point
-        imad_per = 2 * (2 * limbs * limbs + limbs)
-        achieved = modmuls * imad_per / (ms * 1e-3) / 1e12
+        mixed, full = 18 * limbs * limbs + limbs, 26 * limbs * limbs + limbs
+        achieved = 2 * K * (n * mixed + (1 << (c - 1)) * 2 * full) / (ms * 1e-3) / 1e12
         out[f"n_2_{lg}"] = {"ms": round(ms, 3), "points_per_s": n / (ms * 1e-3), "window_bits": c, "windows": K,
                             "segment_length": info["segment_length"], "plan_device_gb":
                             round(info["device_bytes"] / 1e9, 2), "algorithmic_modmuls": modmuls,
@@ -689,8 +698,8 @@ def measure_quotient(torch, N, stream, reps: int, log_n: int = 20, blowup_log: i
         mid.record(stream)
         mid.synchronize()
         q_ms = start.elapsed_time(mid) / reps
-        # two products and one reduction per element (2.5 modmul equivalents)
-        q_frac = 2.5 * m * IMAD_PER_MODMUL / (q_ms * 1e-3) / 1e12 / imad_peak_tops()
+        # two products per element (c enters the first one's accumulators)
+        q_frac = 2 * m * IMAD_PRODUCT / (q_ms * 1e-3) / 1e12 / imad_peak_tops()
         return {"workload": f"prover quotient step, BLS12-381 Fr, n=2^{log_n}, coset of m=2^{log_n + blowup_log} "
                             "points: 3 coset NTTs + fused pointwise (a b - c)/Z_H + coset inverse NTT",
                 "ms": round(ms, 4), "coset_points_per_s": m / (ms * 1e-3),
@@ -732,8 +741,10 @@ def measure_modmul(torch, N, stream, count: int = 1 << 22, reps: int = 64) -> di
         stop.record(stream)
         stop.synchronize()
         ms = start.elapsed_time(stop)
+        # eight lanes: 64 + 64 limb products and eight times the reduction factors
+        imad = IMAD_PRODUCT if variant == 0 else 2 * (64 + 64) + 64
         res[name] = {"ms": round(ms, 4), "modmul_per_s": count * reps / (ms * 1e-3),
-                     "imad_frac_alg": count * reps * IMAD_PER_MODMUL / (ms * 1e-3) / 1e12 / imad_peak_tops()}
+                     "imad_frac": count * reps * imad / (ms * 1e-3) / 1e12 / imad_peak_tops()}
         outs.append(z)
     res["identical"] = bool(torch.equal(outs[0], outs[1]))
     res["workload"] = f"{count} BLS12-381 elements x {reps} dependent Montgomery products"
@@ -1098,8 +1109,7 @@ def run_ours(args) -> None:
     peak = imad_peak_tops()
     dom = max(range(desc["num_passes"]), key=lambda j: pass_ms[j])
     avg_ms = pass_ms[dom] / max(1, pass_cnt[dom])
-    mm = pass_modmuls(log_n, desc["pass_log"], dom, dom >= 1)
-    achieved = mm * IMAD_PER_MODMUL / (avg_ms * 1e-3) / 1e12
+    achieved = pass_imad(log_n, desc["pass_log"][dom], dom >= 1) / (avg_ms * 1e-3) / 1e12
     launches = args.steps * 2 * desc["launches_per_transform"]
 
     secondary = None
