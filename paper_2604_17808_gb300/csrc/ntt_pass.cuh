@@ -274,9 +274,9 @@ __device__ __forceinline__ void tile_put(const PassArgs &a, const TileShape &s, 
 
 template <class El>
 __device__ __forceinline__ void twiddle_get(const PassArgs &a, const TileShape &s, uint32_t *A, uint32_t *B,
-                                            uint32_t w) {
+                                            const uint4 *dft_tw, uint32_t w) {
   if (dbg_in(a, w, s.logs > 1 ? 1u << (s.logs - 1) : 1u)) {
-    El::load_twiddle(A, B, a.dft_tw, w);
+    El::load_twiddle(A, B, dft_tw, w);
   } else {
     words_zero<El::W>(A);
     words_zero<El::W>(B);
@@ -311,10 +311,13 @@ __device__ __forceinline__ Private private_set(const TileShape &s, uint32_t e, u
 
 // Private stages T + hi - 1 down to T + lo: pairs that differ in private bit
 // b, twiddle omega_S^((p mod h) S / 2h) with h = 2^(T + b), p the position in
-// the sub-transform; low = its bits below T.
+// the sub-transform; low = its bits below T.  (dft_tw is a.dft_tw in a register: the
+// batched kernel's `a` is in global memory, and a load of the pointer before every
+// twiddle made lists of 8 small jobs 2% to 8% slower.)
 template <class El>
-__device__ __forceinline__ void private_stages(const PassArgs &a, uint32_t tile, const TileShape &s, const Private &v,
-                                               uint32_t T, int hi, int lo, uint32_t low) {
+__device__ __forceinline__ void private_stages(const PassArgs &a, uint32_t tile, const uint4 *dft_tw,
+                                               const TileShape &s, const Private &v, uint32_t T, int hi, int lo,
+                                               uint32_t low) {
 #pragma unroll 1
   for (int b = hi - 1; b >= lo; --b) {
     const uint32_t mask = (1u << b) - 1u, sh = s.logs - 1u - (T + (uint32_t)b);
@@ -335,7 +338,7 @@ __device__ __forceinline__ void private_stages(const PassArgs &a, uint32_t tile,
         continue;
       }
       uint32_t A[El::W], B[El::W];
-      twiddle_get<El>(a, s, A, B, w);
+      twiddle_get<El>(a, s, A, B, dft_tw, w);
       tile_get<El>(a, s, x, tile, c);
       tile_get<El>(a, s, y, tile, c ^ db);
       El::sub(d, x, y);
@@ -452,7 +455,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     } else {
       tile_copy_wait();
     }
-    if (T > 0) private_stages<El>(a, smem, s, v, T, (int)r, 0, low);
+    if (T > 0) private_stages<El>(a, smem, a.dft_tw, s, v, T, (int)r, 0, low);
   }
 
   // ---- middle rounds
@@ -463,7 +466,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
     group_sync<GROUPED>(group, threads);
     const uint32_t low = t & ((1u << T) - 1u);
     const Private v = private_set<El>(s, low | ((t >> T) << (T + r)), T, r);
-    private_stages<El>(a, smem, s, v, T, (int)r, 0, low);
+    private_stages<El>(a, smem, a.dft_tw, s, v, T, (int)r, 0, low);
   }
 
   // ---- last round: stages last - 1 .. 0; inner passes vary sub-transforms
@@ -476,7 +479,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
   const uint32_t p0 = tbits ? (__brev(tt) >> (32 - tbits)) << last : 0u;
   const Private v = private_set<El>(s, (dl << logs) | p0, 0, last);
   const uint32_t lmask = (1u << last) - 1u, half = 1u << (logs - 1);
-  private_stages<El>(a, smem, s, v, 0, (int)last, last >= 2 ? 2 : 1, 0);
+  private_stages<El>(a, smem, a.dft_tw, s, v, 0, (int)last, last >= 2 ? 2 : 1, 0);
   const uint32_t unit = last >= 2 ? 4u : 2u;
 #pragma unroll 1
   for (uint32_t j = 0; j < (1u << pl); j += unit) {
@@ -496,7 +499,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, const TileShape s, 
       uint32_t x2[El::W], x3[El::W];
       {
         uint32_t A[El::W], B[El::W];   // omega_4 = omega_S^(S/4)
-        twiddle_get<El>(a, s, A, B, half >> 1);
+        twiddle_get<El>(a, s, A, B, a.dft_tw, half >> 1);
         tile_get<El>(a, s, x1, smem, c ^ v.d0);
         tile_get<El>(a, s, x3, smem, c ^ v.d0 ^ v.d1);
         El::sub(y, x1, x3);

@@ -67,7 +67,7 @@ __global__ void probe(const uint4 *table, uint32_t *err, uint32_t index, int wha
   for (uint32_t i = 0; i < 2 * 64; ++i) El::tile_store(tile, 32 * i, 7, ones);
   if (what == 0) tile_get<El>(a, s, A, tile, index);
   if (what == 1) { tile_put<El>(a, s, tile, index, A); El::tile_load(A, tile, index, 7); }
-  if (what == 2) twiddle_get<El>(a, s, A, B, index);
+  if (what == 2) twiddle_get<El>(a, s, A, B, table, index);
   out[0] = A[0];
   out[1] = B[0];
 }
