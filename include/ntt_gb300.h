@@ -42,7 +42,8 @@
  * transform is one pass and does not use the scratch, whatever the number of
  * passes out of place, unless ntt_plan_set_passes or the autotuner chose the
  * plan's passes.  ntt_transform_host and ntt_transform_host_async transform
- * in place.
+ * in place (up to 2^10 points the former, which ends its work before it
+ * returns, uses the scratch when no other call of it does).
  *
  * Errors: every call returns an ntt_status; NTT_ERR_INVALID_ARG for a NULL
  * plan or buffer, a misaligned buffer or an unknown enum value;

@@ -253,19 +253,22 @@ ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *
     NTT_CUDA(L.gen_1d(p->pre_one[kInverse], 1ull << log_n, make_ladder(F, u256(1), log_n), n_inv_m, st));
   }
   if (p->has_coset) NTT_TRY(build_coset_tables(p, F.reduce_small(F.generator), st));
-  if (P > 1 && !p->in_place_one) NTT_TRY(alloc_tab(p, &p->scratch, 1ull << log_n));
+  if (P > 1) NTT_TRY(alloc_tab(p, &p->scratch, 1ull << log_n));
   p->launches = P;
   return NTT_OK;
 }
 
 // Whether a call runs as the plan's single in-place pass.
-static bool runs_one_pass(ntt_plan p, const void *in, const void *out) { return in == out && p->in_place_one; }
+static bool runs_one_pass(ntt_plan p, const void *in, const void *out, bool own_scratch) {
+  return in == out && p->in_place_one && !own_scratch;
+}
 
 // Arguments of pass j of one transform: pass 0 reads `in`; every later pass
 // works in place on `work` (out, or the plan's scratch for in-place calls);
 // the last pass writes `out`.
-void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j, PassArgs *a, int *mode) {
-  const bool one = runs_one_pass(p, in, out);
+void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j, PassArgs *a, int *mode,
+                     bool own_scratch) {
+  const bool one = runs_one_pass(p, in, out, own_scratch);
   const uint32_t P = one ? 1 : p->num_passes, log_n = p->log_n;
   const int tk = table_kind(kind);
   const int dir = tk == kInverse ? 1 : 0;
@@ -345,15 +348,15 @@ TileShape batch_shape(uint64_t elements, uint32_t logs, uint32_t tile_log, int s
 }
 
 // Enqueue one transform: one kernel launch per pass.
-ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st) {
+ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st, bool own_scratch) {
   const FieldLaunchers &L = launchers(p->field);
   const bool shrink = p->debug_shrink;   // debug-build test hook (see ntt_debug_shrink_next_extent)
   p->debug_shrink = false;
-  const bool one = runs_one_pass(p, in, out);
+  const bool one = runs_one_pass(p, in, out, own_scratch);
   for (uint32_t j = 0; j < (one ? 1 : p->num_passes); ++j) {
     PassArgs a;
     int mode;
-    build_pass_args(p, kind, in, out, j, &a, &mode);
+    build_pass_args(p, kind, in, out, j, &a, &mode, own_scratch);
     if (shrink) a.n_vec >>= 1;
     const uint32_t logs = one ? p->log_n : p->pass_log[j];
     cudaError_t e = timing_begin(p, (int)j, st);
@@ -517,11 +520,19 @@ ntt_status ntt_transform_host(ntt_plan plan, ntt_kind kind, const void *h_in, vo
   NTT_TRY(check_buffer(d_work));
   const size_t bytes = (size_t)32 << plan->log_n;
   cudaStream_t st = (cudaStream_t)stream;
+  // This call ends its work before it returns, so that where in-place transforms
+  // leave the scratch alone it may use it under the lock (2^10 points, whole call:
+  // 28 us in two passes, 38 in one); another thread's call meanwhile does without.
+  std::unique_lock<std::mutex> scratch(plan->scratch_mu, std::defer_lock);
+  const bool own = plan->in_place_one && plan->path != NTT_PATH_MATRIX && kind_is_valid((int)kind, plan->has_coset) &&
+                   scratch.try_lock();
   NTT_CUDA(cudaMemcpyAsync(d_work, h_in, bytes, cudaMemcpyHostToDevice, st));
-  NTT_TRY(ntt_execute(plan, kind, d_work, d_work, stream));
-  NTT_CUDA(cudaMemcpyAsync(h_out, d_work, bytes, cudaMemcpyDeviceToHost, st));
-  NTT_CUDA(cudaStreamSynchronize(st));
-  return NTT_OK;
+  ntt_status s = own ? enqueue_transform(plan, (int)kind, d_work, d_work, st, true)
+                     : ntt_execute(plan, kind, d_work, d_work, stream);
+  if (s == NTT_OK) s = cuda_status(cudaMemcpyAsync(h_out, d_work, bytes, cudaMemcpyDeviceToHost, st));
+  if (s != NTT_OK && !own) return s;
+  const cudaError_t e = cudaStreamSynchronize(st);   // with the scratch on errors too
+  return s != NTT_OK ? s : cuda_status(e);
 }
 
 ntt_status ntt_transform_host_async(ntt_plan plan, ntt_kind kind, const void *h_in, void *h_out, void *d_work,

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -46,10 +47,12 @@ struct ntt_plan_s {
   uint4 *fac_coset[gb300ntt::kMaxPasses] = {};  // [pass >= 1]: s^(n N / M_j), n < S_j
   uint4 *post_coset_inv = nullptr;  // s^-n, n < N: output multipliers of the coset inverse
   uint4 *scratch = nullptr;      // N elements (in-place transforms with > 1 pass)
-  // in-place transforms run as one pass, without the scratch, although the plan
-  // has more (see build_plan); its pass-0 multipliers [N] by kind
+  // In-place transforms run as one pass, without the scratch, although the plan
+  // has more (see build_plan); its pass-0 multipliers [N] by kind.  The scratch is
+  // then for calls that end before they return, one at a time (scratch_mu).
   bool in_place_one = false;
   uint4 *pre_one[3] = {};
+  std::mutex scratch_mu;
   uint32_t *d_err = nullptr;     // device error word
   bool debug_shrink = false;     // debug builds: next transform with its vector extent halved
   std::vector<void *> allocations;
@@ -91,10 +94,13 @@ std::vector<uint32_t> split_passes_max(uint32_t log_n, uint32_t max_log);
 // has_coset, sm_count set) for the given pass split (nullptr = default).
 ntt_status build_plan(ntt_plan p, cudaStream_t st, const std::vector<uint32_t> *forced_split);
 uint64_t pass_tiles(uint32_t log_n, uint32_t logs, uint32_t tl);
-ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st);
+ntt_status enqueue_transform(ntt_plan p, int kind, const void *in, void *out, cudaStream_t st,
+                             bool own_scratch = false);
 ntt_status cuda_status(cudaError_t e);
 struct PassArgs;
-void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j, PassArgs *a, int *mode);
+// own_scratch: the caller holds the plan's scratch_mu until the transform has ended
+void build_pass_args(ntt_plan p, int kind, const void *in, void *out, uint32_t j, PassArgs *a, int *mode,
+                     bool own_scratch = false);
 ntt_status check_buffer(const void *ptr);
 // Timing hooks around one launch of pass `pass` (no-ops unless timing is on).
 cudaError_t timing_begin(ntt_plan p, int pass, cudaStream_t st);

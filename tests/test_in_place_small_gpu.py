@@ -89,3 +89,47 @@ def test_one_pass_split(field, log_n):
             assert np.array_equal(d_y.cpu().numpy().view(np.uint64), oracle.c_transform(field, kind, x)), kind
     finally:
         N.ntt_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("field", ["bls12_381_fr", "bn254_fr"])
+@pytest.mark.parametrize("log_n", [9, 10])
+def test_host_transforms_from_several_threads(field, log_n):
+    """Host transforms of one plan from threads with streams of their own, next to
+    in-place transforms of device buffers: only one of them at a time may use the
+    plan's scratch."""
+    import threading
+
+    from paper_2604_17808_gb300 import _native as N
+
+    n, threads, reps = 1 << log_n, 4, 60
+    plan = N.ntt_plan_create(field, log_n, coset=True)
+    try:
+        xs = [uniform_elements(field, n, 40 * t + log_n) for t in range(threads)]
+        want = [[oracle.c_transform(field, kind, x) for kind in KINDS] for x in xs]
+        wrong = []
+
+        def work(t):
+            stream, w = torch.cuda.Stream(), torch.empty((n, 4), dtype=torch.int64, device="cuda")
+            h_in = torch.from_numpy(xs[t].view(np.int64)).pin_memory()
+            h_out = torch.empty_like(h_in).pin_memory()
+            for i in range(reps):
+                kind = KINDS[(i + t) % 4]
+                if t == 0:
+                    with torch.cuda.stream(stream):
+                        w.copy_(h_in)
+                        N.ntt_execute(plan, kind, w, w, stream)
+                        got = w.cpu()
+                else:
+                    N.ntt_transform_host(plan, kind, h_in, h_out, w, stream)
+                    got = h_out
+                if not np.array_equal(got.numpy().view(np.uint64), want[t][(i + t) % 4]):
+                    wrong.append((t, i))
+
+        pool = [threading.Thread(target=work, args=(t,)) for t in range(threads)]
+        for p in pool:
+            p.start()
+        for p in pool:
+            p.join()
+        assert not wrong
+    finally:
+        N.ntt_plan_destroy(plan)
