@@ -488,11 +488,11 @@ ntt_status ntt_pointwise_quotient(ntt_field field, const void *d_a, const void *
  * (resp. 24) little-endian uint32 words at byte offset 48 i (resp. 96 i),
  * standard form, canonical, natural order; device buffers 16-byte aligned;
  * d_in == d_out allowed.  Same pass decomposition as the 256-bit
- * transforms, with a generic-limb Montgomery product; the coset factors
+ * transforms, on 32-bit words; the coset factors
  * s^i ride on the first pass's loads and the coset inverse's s^-i on the
  * last pass's stores.  The first call for a (device, field, log_n) builds
  * the tables on the device, and the first coset call of either coset kind
- * the two coset tables (2 * 4 * LP * 2^log_n bytes, LP = 16 resp. 28);
+ * the two coset tables (2 * 48 resp. 96 bytes * 2^log_n);
  * both synchronous, kept until the process exits.  Stream-ordered.  The
  * tables and an in-place call's scratch vector belong to the (device,
  * field, log_n), not to the caller: two in-place calls of the same field

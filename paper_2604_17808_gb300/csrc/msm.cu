@@ -1204,7 +1204,7 @@ ntt_status enqueue_msm(msm_plan p, const uint4 *sc, const uint4 *pt, uint64_t n,
     // it crosses at most this many segment ends; empty levels exit at once
     // (segments of 8 entries at least, at most max_segments of them; the grid is
     // for K windows in a range of fewer too: each bucket adds an item to its
-    // segments', and a second round for those costs a level's time again)
+    // segments', and going round the loop again for those doubles a level's time)
     const uint64_t most = flat ? n * p->K : n;
     const uint64_t max_span = std::min<uint64_t>((most + 7) / 8, p->max_segments);
     uint64_t step = 1;
